@@ -135,6 +135,7 @@ enum Slot {
     S_GAP,                           // eigen-gaps of the basis slices (strict mode)
     S_WIDX0, S_WIDX1, S_WB64, S_WB32, S_WZ, S_WF, S_WU, S_WGX, S_WG2, S_WRED,   // weight tuning by SURE
     S_CSCR, S_CNUM, S_CDEN,          // hyperspectral cubes: per-CTA Haar slots, numerator, denominator
+    S_BMTC,                          // planes and box sums of the tensor-core grouping
     S_PROJ,                          // split BF16 basis matrix of htsvd_project_patches
     S_VMOM, S_VB64, S_VNUM, S_VDEN,  // MRI volumes: moments, bases, numerator, denominator
     S_NSLOT
@@ -150,6 +151,7 @@ struct Workspace {
     cudaStream_t side = nullptr;          // moments + basis run here (highest priority), concurrently with
                                           // block matching
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    int* timeout = nullptr;               // pinned word a kernel sets when one of its waits runs out
 };
 
 std::mutex g_mu;
@@ -293,7 +295,7 @@ struct VideoCtx {
     int f0, nfr, fref;
 };
 
-htsvd_status run_block_match(const uint8_t* q, const Geo& g, const Resolved& r, int rstep, int32_t* idx,
+htsvd_status run_block_match(Workspace* w, const uint8_t* q, const Geo& g, const Resolved& r, int rstep, int32_t* idx,
                              cudaStream_t s, const VideoCtx* vc = nullptr) {
     BMArgs a{};
     a.img = q;
@@ -314,6 +316,19 @@ htsvd_status run_block_match(const uint8_t* q, const Geo& g, const Resolved& r, 
     bm_fit_tiles(a);
     if (bm_smem_bytes(a) > 227 * 1024) return HTSVD_ERR_UNSUPPORTED;   // e.g. too many frames in reach
     a.idx = idx;
+    if (const size_t tcb = bm_tc_scratch(a)) {
+        void* scratch;
+        if (ws_get(w, S_BMTC, tcb, &scratch) == HTSVD_OK) {
+            if (!w->timeout) {
+                CK(cudaMallocHost(&w->timeout, sizeof(int)));
+                *w->timeout = 0;
+            }
+            if (*w->timeout) return HTSVD_ERR_TIMEOUT;
+            ProfScope ps_("block_match", s);
+            CK(launch_block_match_tc(a, scratch, w->timeout, s));
+            return HTSVD_OK;
+        }
+    }
     { ProfScope ps_("block_match", s); CK(launch_block_match(a, s)); }
     return HTSVD_OK;
 }
@@ -405,7 +420,7 @@ htsvd_status enqueue_sigma_inputs(Workspace* w, const uint8_t* q, const Geo& g, 
         void *idx2, *ranks;
         ST(ws_get(w, S_IDX2, sizeof(int32_t) * ny8 * nx8 * g.K, &idx2));
         ST(ws_get(w, S_RANKS, sizeof(int32_t) * ny8 * nx8, &ranks));
-        ST(run_block_match(q, g, r, 8, (int32_t*)idx2, s));
+        ST(run_block_match(w, q, g, r, 8, (int32_t*)idx2, s));
         { ProfScope ps_("group_rank", s); CK(launch_group_rank(q, g, (const int32_t*)idx2, ny8 * nx8, (int32_t*)ranks, s)); }
         CK(cudaMemcpyAsync(h + (size_t)d * d + d, ranks, sizeof(int32_t) * ny8 * nx8, cudaMemcpyDeviceToHost, s));
     }
@@ -560,7 +575,7 @@ htsvd_status denoise_impl(const void* d_in, int is_float, int H, int W, int C, d
     if (r.strict_basis) ST(ws_get(w, S_GAP, sizeof(double) * basis_problems(C), &gap));
     ST(run_basis(w, q, g, &b64, &b32, w->side, (const unsigned long long*)fullM, (double*)gap));
     CK(cudaEventRecord(w->ev_join, w->side));
-    ST(run_block_match(q, g, r, 1, idx, s));
+    ST(run_block_match(w, q, g, r, 1, idx, s));
     CK(cudaStreamWaitEvent(s, w->ev_join, 0));
     if (p && p->d_basis_out)
         CK(cudaMemcpyAsync(p->d_basis_out, b64, sizeof(double) * 2 * 2 * C * PS2, cudaMemcpyDeviceToDevice, s));
@@ -616,7 +631,7 @@ htsvd_status video_impl(const uint8_t* d_vid, int F, int H, int W, int C, int T,
         CK(cudaEventRecord(w->ev_join, w->side));
         const int f0 = std::max(0, t - T), f1 = std::min(F - 1, t + T);
         const VideoCtx vc{d_vid, fr, f0, f1 - f0 + 1, t};
-        ST(run_block_match(q, g, r, 1, idx, s, &vc));
+        ST(run_block_match(w, q, g, r, 1, idx, s, &vc));
         CK(cudaStreamWaitEvent(s, w->ev_join, 0));
         if (sg < 0) {
             if (cudaEventSynchronize(hev.ev) != cudaSuccess) return HTSVD_ERR_CUDA;
@@ -668,7 +683,7 @@ htsvd_status sweep_impl(const uint8_t* d_in, int H, int W, int C, double sigma, 
     if (sigma < 0) ST(ws_get(w, S_FULLM, sizeof(unsigned long long) * PS2 * C * PS2 * C, &fullM));
     ST(run_basis(w, d_in, g, &b64, &b32, w->side, (const unsigned long long*)fullM));
     CK(cudaEventRecord(w->ev_join, w->side));
-    ST(run_block_match(d_in, g, r, 1, idx, s));
+    ST(run_block_match(w, d_in, g, r, 1, idx, s));
     CK(cudaStreamWaitEvent(s, w->ev_join, 0));
     // the noisy coefficients (tau plays no part in the analysis)
     CoefCache cache{(float*)cc, (float*)cp, (int*)cn, FM_ANALYZE};
@@ -799,7 +814,7 @@ htsvd_status sure_w_prepare(Workspace* w, const float* d_y, int H, int W, int C,
         ST(run_basis(w, (const uint8_t*)qb, c.g, &p64, &p32, s));
         CK(cudaMemcpyAsync(c.b64[k], p64, sizeof(double) * 2 * 2 * C * PS2, cudaMemcpyDeviceToDevice, s));
         CK(cudaMemcpyAsync(c.b32[k], p32, sizeof(float) * 512, cudaMemcpyDeviceToDevice, s));
-        ST(run_block_match((const uint8_t*)qb, c.g, c.r, 1, c.idx[k], s));
+        ST(run_block_match(w, (const uint8_t*)qb, c.g, c.r, 1, c.idx[k], s));
     }
     return HTSVD_OK;
 }
@@ -856,7 +871,7 @@ int32_t htsvd_internal_sampled_ranks(const uint8_t* d_img, int32_t H, int32_t W,
     if (ws_get(w, S_IDX2, sizeof(int32_t) * n * g.K, &idx2) != HTSVD_OK ||
         ws_get(w, S_RANKS, sizeof(int32_t) * n, &ranks) != HTSVD_OK)
         return -1;
-    if (run_block_match(d_img, g, r, 8, (int32_t*)idx2, nullptr) != HTSVD_OK) return -1;
+    if (run_block_match(w, d_img, g, r, 8, (int32_t*)idx2, nullptr) != HTSVD_OK) return -1;
     if (launch_group_rank(d_img, g, (const int32_t*)idx2, n, (int32_t*)ranks, nullptr) != cudaSuccess) return -1;
     if (cudaMemcpy(h_ranks, ranks, sizeof(int32_t) * n, cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
     return n;
@@ -1079,7 +1094,7 @@ htsvd_status htsvd_sure(const float* d_y, int32_t H, int32_t W, int32_t C, doubl
         double* b64;
         float* b32;
         ST(run_basis(w, (const uint8_t*)qb, g, &b64, &b32, s));
-        ST(run_block_match((const uint8_t*)qb, g, r, 1, (int32_t*)idx, s));
+        ST(run_block_match(w, (const uint8_t*)qb, g, r, 1, (int32_t*)idx, s));
         for (int i = 0; i < n_tau; ++i) {
             const Resolved& ri = rs[i];
             const double tau = ri.tau_mult * sigma;
@@ -1514,6 +1529,7 @@ htsvd_status htsvd_release_workspace(void) {
             for (int i = 0; i < S_NSLOT; ++i)
                 if (w->buf[i]) cudaFree(w->buf[i]);
             if (w->hpin) cudaFreeHost(w->hpin);
+            if (w->timeout) cudaFreeHost(w->timeout);
             if (w->side) cudaStreamDestroy(w->side);
             if (w->ev_fork) cudaEventDestroy(w->ev_fork);
             if (w->ev_join) cudaEventDestroy(w->ev_join);

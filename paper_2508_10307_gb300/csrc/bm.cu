@@ -17,7 +17,11 @@
 // merged so far) are appended to a per-warp buffer; 32 buffered keys at a time are sorted and
 // merged into the warp-wide sorted list (lane l holds the l-th smallest). Ties therefore break
 // by the lowest linear index. Slot 0 of every group is the reference itself.
+#include <algorithm>
+#include <cuda_fp16.h>
+
 #include "kernels.h"
+#include "tc.cuh"
 
 namespace htsvd {
 
@@ -622,6 +626,8 @@ __global__ void __launch_bounds__(BM_THREADS, 2) block_match_batch_kernel(const 
     }
 }
 
+#include "bm_tc.cuh"
+
 constexpr size_t BM_SMEM_TARGET = 100 * 1024;    // leaves room for two CTAs per SM
 constexpr size_t BM_SMEM_MAX = 227 * 1024;
 
@@ -672,6 +678,104 @@ cudaError_t launch_block_match(const BMArgs& a, cudaStream_t s) {
     dim3 grid((a.nrx_s + a.TRx - 1) / a.TRx, (a.nry_s + a.TRy - 1) / a.TRy);
     fn<<<grid, BM_THREADS, smem, s>>>(a);
     return cudaGetLastError();
+}
+
+namespace {
+
+struct BtPlan {
+    int npl, nsv, nfr, TX, XP, SR, ib, pitch;
+    size_t planes, svv;      // bytes over all frames
+};
+
+// The tensor-core form takes images of one or three channels with every reference, candidate rows of at
+// most 128 columns per tile and at most 4,096 candidates per reference (keys then hold SSD < 2^20).
+bool bt_plan(const BMArgs& a, BtPlan& p) {
+    const Geo& g = a.g;
+    if (a.rstep != 1 || (g.C != 1 && g.C != 3)) return false;
+    p.npl = bt_planes(a.mode, g.C);
+    p.nsv = p.npl == 2 ? 2 : 1;
+    p.nfr = a.nfr > 0 ? a.nfr : 1;
+    // 4 x 32 references share their rows of candidates best; 8 x 16 where those are longer than an accumulator
+    for (p.TX = 32;; p.TX = 16) {
+        p.XP = (std::min((p.TX - 1) * g.s + g.wnx, g.npx) + 15) & ~15;
+        if (p.XP <= BT_ACC) break;
+        if (p.TX == 16) return false;
+    }
+    const int64_t nc = (int64_t)p.nfr * g.wny * g.wnx;
+    if (nc > 4096) return false;
+    p.ib = 8;                // at least 8: the exponent of SSD + 2^23 then falls out of the key
+    while (((int64_t)1 << p.ib) < nc) ++p.ib;
+    p.pitch = (g.W + 39) & ~7;
+    p.planes = sizeof(__half) * p.nfr * ((size_t)p.npl * g.H * p.pitch + 64);
+    p.svv = sizeof(float) * p.nfr * ((size_t)p.nsv * (g.H - PS + 1) * p.pitch + 64);
+    // strip rows: as many as let two CTAs share an SM, at least three rows of candidates
+    for (p.SR = BT_SR; p.SR > PS + 2 && bt_layout(p.npl, p.nsv, p.XP, p.SR).total > 113 * 1024; --p.SR) {}
+    return bt_layout(p.npl, p.nsv, p.XP, p.SR).total <= (int)BM_SMEM_MAX;
+}
+
+template <int NPL, bool GCP>
+cudaError_t launch_bt(const BMArgs& a, const BtPlan& p, void* scratch, int* timeout, cudaStream_t s) {
+    const Geo& g = a.g;
+    BtArgs A{};
+    A.b = a;
+    A.fstride_p = (long long)NPL * g.H * p.pitch;
+    A.fstride_s = (long long)p.nsv * (g.H - PS + 1) * p.pitch;
+    A.planes = static_cast<const __half*>(scratch);
+    A.svv = reinterpret_cast<const float*>(static_cast<unsigned char*>(scratch) + ((p.planes + 255) & ~(size_t)255));
+    A.pitch = p.pitch;
+    A.XP = p.XP;
+    A.SR = p.SR;
+    A.TX = p.TX;
+    A.ib = p.ib;
+    A.timeout = timeout;
+    for (int f = 0; f < p.nfr; ++f) {
+        BtPrep b{};
+        b.img = a.nfr > 0 ? a.vid + (a.f0 + f) * a.fstride : a.img;
+        b.H = g.H;
+        b.W = g.W;
+        b.C = g.C;
+        b.mode = a.mode;
+        b.planes = const_cast<__half*>(A.planes) + f * A.fstride_p;
+        b.svv = const_cast<float*>(A.svv) + f * A.fstride_s;
+        b.pitch = p.pitch;
+        bt_prep_kernel<NPL, GCP><<<dim3((g.W + BP_X - 1) / BP_X, (g.H + BP_Y - 1) / BP_Y), 256, 0, s>>>(b);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    // at most two CTAs per SM: each takes half of the tensor memory
+    const int smem = std::max(bt_layout(NPL, p.nsv, p.XP, p.SR).total, 77 * 1024);
+    auto fn = block_match_tc_kernel<NPL, GCP>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e != cudaSuccess) return e;
+    const int TY = BT_REFS / p.TX;
+    fn<<<dim3((g.nrx + p.TX - 1) / p.TX, (g.nry + TY - 1) / TY), BT_THREADS, smem, s>>>(A);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t bm_tc_scratch(const BMArgs& a) {
+    BtPlan p;
+    if (!bt_plan(a, p)) return 0;
+    const Geo& g = a.g;
+    const int TY = BT_REFS / p.TX;
+    const int64_t tiles = (int64_t)((g.nrx + p.TX - 1) / p.TX) * ((g.nry + TY - 1) / TY);
+    // A tile takes 70 us (window 21, gray) to 140 us (window 31, RGB) from end to end however few there are; the
+    // CUDA-core kernel cuts the image finer (32 references per CTA) and wins below about 9,500 references:
+    // us at 84^2 / 106^2 / 170^2 references, tensor cores against CUDA cores: gray, window 21: 74 / 75 / 98
+    // against 56 / 96 / 172; RGB, window 18: 91 / 91 / 154 against 73 / 126 / 200; RGB, window 31:
+    // 144 / 142 / 214 against 99 / 167 / 297. 8 x 16 tiles (gray, window 31, stride 4): 171 against 146 at
+    // 127^2 references (128 tiles): they wait for a full wave of tiles.
+    if (tiles < (p.TX == 32 ? 76 : 152)) return 0;
+    return ((p.planes + 255) & ~(size_t)255) + p.svv;
+}
+
+cudaError_t launch_block_match_tc(const BMArgs& a, void* scratch, int* timeout, cudaStream_t s) {
+    BtPlan p;
+    if (!bt_plan(a, p)) return cudaErrorInvalidValue;
+    if (p.npl == 2) return launch_bt<2, true>(a, p, scratch, timeout, s);
+    return p.npl == 3 ? launch_bt<3, false>(a, p, scratch, timeout, s) : launch_bt<1, false>(a, p, scratch, timeout, s);
 }
 
 }  // namespace htsvd

@@ -33,6 +33,10 @@ size_t bm_smem_bytes(const BMArgs& a);
 // Halves the tile (TRx, TRy) until its shared-memory footprint leaves room for two CTAs per SM.
 void bm_fit_tiles(BMArgs& a);
 cudaError_t launch_block_match(const BMArgs& a, cudaStream_t s);
+// Tensor-core form: bytes of device scratch it needs (0: not for this geometry, or not faster there), and
+// its launch. timeout: host-readable word set if a wait inside the kernel runs out.
+size_t bm_tc_scratch(const BMArgs& a);
+cudaError_t launch_block_match_tc(const BMArgs& a, void* scratch, int* timeout, cudaStream_t s);
 
 // ---- second moments and bases (moments.cu)
 // Row/column second moments of the reference patches, exact:
