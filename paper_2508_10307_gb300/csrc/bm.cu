@@ -21,6 +21,7 @@
 #include <cuda_fp16.h>
 
 #include "kernels.h"
+#include "lane_sort.cuh"
 #include "tc.cuh"
 
 namespace htsvd {

@@ -24,6 +24,7 @@
 #include <cstring>
 
 #include "kernels.h"
+#include "lane_sort.cuh"
 
 namespace htsvd {
 
@@ -33,6 +34,7 @@ constexpr int VPS = 4;                 // cube edge
 constexpr int VTR = 4;                 // references per tile edge of the filter
 constexpr int kVolWarps = 6;
 constexpr int kMaxCand = 512;          // W^3 <= 512 (W <= 8)
+constexpr long long kLaneRefs = 6000;  // references from which grouping takes a thread for each
 constexpr int kHcBytes = kVolWarps * 32 * 65 * 4;
 
 __host__ __device__ inline int vref_count(int n, int s) {
@@ -132,6 +134,115 @@ block_match_volume_kernel(const uint8_t* __restrict__ vol, VolGeo g, int32_t* __
             if (rank < g.K - 1) out[1 + rank] = (int32_t)(k & 0xffffffffull);
         }
         __syncwarp();
+    }
+}
+
+// Windows of W^3 candidates with every extent W (4 to 6): one thread per reference. The candidates of a
+// plane of the window are taken CYB rows at a time (at most 32): each image row is loaded once for the
+// candidate rows and cube rows it meets, its W shifts formed by funnel shifts, and the SSDs stay in
+// registers. Keys (SSD << 9 | window index) are sorted by a network in registers and merged into the
+// thread's 32 smallest: no shared memory, no votes, and every lane of the warp has a reference. The warp
+// per reference form above spends its time on loads and ballots (a bit of a key at a time): 2.95 -> 0.48 ms on
+// the 780 K references of a 176 x 208 x 176 volume (W = 5, K 32). Issue bound: the sorting network alone is 191
+// compare-exchanges a batch.
+template <int W, bool VEC>
+__global__ void __launch_bounds__(128) block_match_volume_lane_kernel(const uint8_t* __restrict__ vol, VolGeo g,
+                                                                      int32_t* __restrict__ idx) {
+    constexpr int CYB = W <= 5 ? W : 3;                // candidate rows per sort (CYB W <= 32)
+    constexpr int IB = 9;                              // W^3 <= 512; SSD < 2^22
+    const long long nref = (long long)g.nrz * g.nry * g.nrx;
+    const long long r = (long long)blockIdx.x * 128 + threadIdx.x;
+    if (r >= nref) return;
+    const long long total = (long long)g.D * g.H * g.W;
+    const int plane = g.H * g.W;
+    const int iz = (int)(r / ((long long)g.nry * g.nrx));
+    const int rem = (int)(r - (long long)iz * g.nry * g.nrx);
+    const int iy = rem / g.nrx, ix = rem - iy * g.nrx;
+    const int z = vref_pos(iz, g.s, g.D), y = vref_pos(iy, g.s, g.H), x = vref_pos(ix, g.s, g.W);
+    const int me = z * plane + y * g.W + x;
+    uint32_t ref[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) ref[q] = bytes4(vol, (long long)me + (q >> 2) * plane + (q & 3) * g.W, total);
+    const int z0 = win_start(z, g.npz, g.win), y0 = win_start(y, g.npy, g.win), x0 = win_start(x, g.npx, g.win);
+    const int first = z0 * plane + y0 * g.W + x0;
+    const uint32_t self = (uint32_t)(((z - z0) * W + (y - y0)) * W + (x - x0));
+    uint32_t list[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) list[i] = ~0u;
+#pragma unroll 1
+    for (int cz = 0; cz < W; ++cz)
+#pragma unroll 1
+        for (int cy0 = 0; cy0 < W; cy0 += CYB) {
+            uint32_t acc[CYB][W];
+#pragma unroll
+            for (int i = 0; i < CYB; ++i)
+#pragma unroll
+                for (int dx = 0; dx < W; ++dx) acc[i][dx] = 0u;
+#pragma unroll
+            for (int c = 0; c < VPS; ++c)
+#pragma unroll
+                for (int t = 0; t < CYB + VPS - 1; ++t) {
+                    // (rows past the window, in a last chunk that is not full, are read inside the volume)
+                    const int yy = min(y0 + cy0 + t, g.H - 1) - y0;
+                    const long long off = (long long)first + (long long)(cz + c) * plane + yy * g.W;
+                    const long long al = off & ~3ll;
+                    uint32_t w[3];
+                    if (al + 12 <= total) {
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) w[k] = __ldg(reinterpret_cast<const uint32_t*>(vol + al) + k);
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            w[k] = 0u;
+                            for (int b = 0; b < 4; ++b)
+                                if (al + 4 * k + b < total) w[k] |= (uint32_t)vol[al + 4 * k + b] << (8 * b);
+                        }
+                    }
+                    // the row from its first byte: 9 bytes at most (W + 3)
+                    const int sh = (int)(off & 3) * 8;
+                    const uint32_t a0 = __funnelshift_r(w[0], w[1], sh), a1 = __funnelshift_r(w[1], w[2], sh);
+                    const uint32_t a2 = w[2] >> sh;
+#pragma unroll
+                    for (int dx = 0; dx < W; ++dx) {
+                        const uint32_t v = dx < 4 ? __funnelshift_r(a0, a1, 8 * dx) : __funnelshift_r(a1, a2, 8 * (dx - 4));
+#pragma unroll
+                        for (int a = 0; a < VPS; ++a) {
+                            const int i = t - a;
+                            if (i < 0 || i >= CYB) continue;
+                            const uint32_t d = __vabsdiffu4(ref[c * 4 + a], v);
+                            acc[i][dx] = __dp4a(d, d, acc[i][dx]);
+                        }
+                    }
+                }
+            uint32_t b[32];
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                b[i] = ~0u;
+                if (i < CYB * W) {
+                    const int cy = cy0 + i / W;
+                    const uint32_t code = (uint32_t)((cz * W + cy) * W + i % W);
+                    if (cy < W && code != self) b[i] = (acc[i / W][i % W] << IB) | code;
+                }
+            }
+            bt_sort(b);
+            bt_merge(list, b);
+        }
+    int32_t out[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        const uint32_t code = i == 0 ? self : list[i > 0 ? i - 1 : 0] & ((1u << IB) - 1u);
+        const int dz = code / (W * W), q = code % (W * W);
+        out[i] = first + dz * plane + (q / W) * g.W + q % W;
+    }
+    int32_t* dst = idx + r * g.K;
+    if (VEC) {                                         // K a multiple of 4 and idx aligned
+#pragma unroll
+        for (int i = 0; i < 32; i += 4)
+            if (i < g.K) *reinterpret_cast<int4*>(dst + i) = make_int4(out[i], out[i + 1], out[i + 2], out[i + 3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (i < g.K) dst[i] = out[i];
     }
 }
 
@@ -767,6 +878,18 @@ int volume_max_window() { return 8; }
 
 cudaError_t launch_block_match_volume(const uint8_t* vol, const VolGeo& g, int32_t* idx, cudaStream_t s) {
     const long long nref = (long long)g.nrz * g.nry * g.nrx;
+    // one thread per reference where the window is a full cube of 4 to 6 and there are references enough (a
+    // warp's 32 references take about 36 us however few there are; window 5, K 32, us, this form / the other:
+    // 36 / 31 at 3,375 references, 36 / 44 at 6,859, 41 / 131 at 29,791, 89 / 413 at 103,823)
+    if (g.wnz == g.win && g.wny == g.win && g.wnx == g.win && g.win >= 4 && g.win <= 6 && nref >= kLaneRefs) {
+        const int nb = (int)((nref + 127) / 128);
+        const bool vec = g.K % 4 == 0 && (reinterpret_cast<uintptr_t>(idx) & 15) == 0;
+        auto fn = g.win == 4   ? (vec ? block_match_volume_lane_kernel<4, true> : block_match_volume_lane_kernel<4, false>)
+                  : g.win == 5 ? (vec ? block_match_volume_lane_kernel<5, true> : block_match_volume_lane_kernel<5, false>)
+                               : (vec ? block_match_volume_lane_kernel<6, true> : block_match_volume_lane_kernel<6, false>);
+        fn<<<nb, 128, 0, s>>>(vol, g, idx);
+        return cudaGetLastError();
+    }
     const long long blocks = (nref + kVolWarps - 1) / kVolWarps;
     const long long cap = (long long)device_sm_count() * 16;
     block_match_volume_kernel<<<(int)(blocks < cap ? blocks : cap), kVolWarps * 32, 0, s>>>(vol, g, idx);
