@@ -18,12 +18,12 @@ namespace {
 
 // ----------------------------------------------------------------------------- moments
 
-constexpr int MOM_CHUNK = 256;     // references per CTA (uint32 partials: 256 * 8 * 255^2 < 2^32)
+constexpr int MOM_CHUNK = 256;     // references per CTA at most (uint32 partials: 256 * 8 * 255^2 < 2^32)
 constexpr int MOM_BATCH = 32;      // references staged at once
 
-// Moments of the references [chunk * MOM_CHUNK, (chunk + 1) * MOM_CHUNK) added into out.
+// Moments of the references [chunk * per, (chunk + 1) * per) added into out.
 template <int C>
-__device__ __forceinline__ void moments_chunk(const uint8_t* __restrict__ img, const Geo& g, int chunk,
+__device__ __forceinline__ void moments_chunk(const uint8_t* __restrict__ img, const Geo& g, int chunk, int per,
                                               unsigned long long* __restrict__ out) {
     // rows[j][c][a] = 8 bytes of row a of channel c; cols[j][c][b] = 8 bytes of column b.
     __shared__ uint32_t rows[MOM_BATCH][C][PS][2];
@@ -35,8 +35,8 @@ __device__ __forceinline__ void moments_chunk(const uint8_t* __restrict__ img, c
     for (int e = 0; e < EPT; ++e) acc[e] = 0;
 
     const int N = g.ngroups();
-    const int r0 = chunk * MOM_CHUNK;
-    const int r1 = min(r0 + MOM_CHUNK, N);
+    const int r0 = chunk * per;
+    const int r1 = min(r0 + per, N);
     for (int rb = r0; rb < r1; rb += MOM_BATCH) {
         const int nb = min(MOM_BATCH, r1 - rb);
         __syncthreads();
@@ -129,9 +129,9 @@ __device__ __forceinline__ void moments_chunk(const uint8_t* __restrict__ img, c
 }
 
 template <int C>
-__global__ void __launch_bounds__(256) moments_kernel(const uint8_t* __restrict__ img, Geo g,
+__global__ void __launch_bounds__(256) moments_kernel(const uint8_t* __restrict__ img, Geo g, int per,
                                                       unsigned long long* __restrict__ out) {
-    moments_chunk<C>(img, g, blockIdx.x, out);
+    moments_chunk<C>(img, g, blockIdx.x, per, out);
 }
 
 // Batch form: chunk items of all images, item w -> image by prefix[].
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(256) moments_batch_kernel(const BMArgs* __rest
             if (prefix[mid] <= w) lo = mid;
             else hi = mid - 1;
         }
-        moments_chunk<C>(args[lo].img, args[lo].g, w - prefix[lo], moms[lo]);
+        moments_chunk<C>(args[lo].img, args[lo].g, w - prefix[lo], MOM_CHUNK, moms[lo]);
     }
 }
 
@@ -493,21 +493,20 @@ __host__ __device__ void canonicalise(double (*Ar)[PS], double (*Vr)[PS], double
     }
 }
 
-// Device form of canonicalise for one warp: lane 0 orders the eigenvalues (the same selection
-// sort), then lane c < 8 treats output column c. The largest-modulus entry is found on squared
+// Device form of canonicalise for one warp: lane i < 8 ranks eigenvalue i, then lane c < 8 treats output column c. The largest-modulus entry is found on squared
 // moduli and the phase takes one reciprocal square root (FP64 square root and division are long
 // sequences on this GPU).
 __device__ void canonicalise_warp(double (*Ar)[PS], double (*Vr)[PS], double (*Vi)[PS], double (*Out)[PS][2],
                                   int* order, int lane) {
-    if (lane == 0) {
-        for (int i = 0; i < PS; ++i) order[i] = i;
-        for (int i = 0; i < PS; ++i)          // selection sort, descending, as in canonicalise
-            for (int j = i + 1; j < PS; ++j)
-                if (Ar[order[j]][order[j]] > Ar[order[i]][order[i]]) {
-                    const int t = order[i];
-                    order[i] = order[j];
-                    order[j] = t;
-                }
+    if (lane < PS) {                          // descending, ties by index
+        int rank = 0;
+        const double mine = Ar[lane][lane];
+#pragma unroll
+        for (int j = 0; j < PS; ++j) {
+            const double v = Ar[j][j];
+            rank += v > mine || (v == mine && j < lane) ? 1 : 0;
+        }
+        order[rank] = lane;
     }
     __syncwarp();
     if (lane < PS) {
@@ -570,20 +569,33 @@ __host__ __device__ void slice_basis(const unsigned long long* mom, int C, int w
 
 // Device form of the solver: parallel (round-robin) Jacobi. Each sweep runs 7 rounds of 4
 // rotations on disjoint index pairs (circle schedule: pairs (p[i], p[7-i]) with p a rotation of
-// 1..7 around 0), so the FP64 latency chain per sweep is 7 rotations deep instead of 28.
+// 1..7 around 0), so the latency chain per sweep is 7 rotations deep instead of 28.
 // Lane i < 4 computes rotation i of a round; lane 8i + k applies it to row/column k.
-// The 2x2 block of a pair is touched only by its own rotation, so each rotation zeroes its pivot
-// exactly as the cyclic solver's would.
-// rot: [5][10] shared scratch: rows 0..3 the rotations of a round
-// (er, ei, c, s, t*r, skip, p, q, a_pp, a_qq), row 4 the convergence flag.
-__device__ void jacobi_herm8_warp(double (*Ar)[PS], double (*Ai)[PS], double (*Vr)[PS], double (*Vi)[PS],
-                                  double (*rot)[10], int lane) {
-    if (lane < PS)
-        for (int j = 0; j < PS; ++j) {
-            Vr[lane][j] = lane == j ? 1.0 : 0.0;
-            Vi[lane][j] = 0.0;
-        }
-    __syncwarp();
+//
+// FP64 runs at 1.7 FMA per clock and SM on this part, and a division or square root takes it thousands of
+// cycles: the solver was 150 us for four problems, almost all of it in the rotations' angles. Any angle
+// gives a similarity transform as long as the rotation itself is unitary to working precision, so the
+// angle comes from FP32 and only cos, sin and the phase are normalised in FP64 (a Newton step on an FP32
+// reciprocal square root). The first sweeps run in FP32 altogether; their eigenvectors, made orthonormal
+// in FP64, transform the FP64 matrix to a nearly diagonal one that two or three FP64 sweeps finish: 80 us (a
+// serial chain of one warp per problem).
+__device__ __forceinline__ float jac_rsqrt(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double jac_rsqrt(double x) {        // 1e-36 < x < 1e36
+    double y = (double)rsqrtf((float)x);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const double e = fma(-(x * y), y, 1.0);
+        y = fma(0.5 * y, e, y);
+    }
+    return y;
+}
+
+// A: Hermitian, largest diagonal entry in [1/2, 1); V is updated (V <- V J). tol: ends when the
+// off-diagonal sum of squares is at most tol times the diagonal's. rot: [4][8] shared scratch (er, ei, c,
+// s, skip, p, q).
+template <typename T>
+__device__ void jacobi_herm8_warp(T (*Ar)[PS], T (*Ai)[PS], T (*Vr)[PS], T (*Vi)[PS], T (*rot)[8], T tol, int sweeps,
+                                  int lane) {
     const int pr_i = lane >> 3, k = lane & 7;          // rotation of this lane, row/column it updates
     // lane l < 28 holds the off-diagonal pair (oi, oj), oi < oj, of the convergence test
     int oi = 0, oj = 0;
@@ -595,15 +607,15 @@ __device__ void jacobi_herm8_warp(double (*Ar)[PS], double (*Ai)[PS], double (*V
         }
         oj = oi + 1 + rem;
     }
-    for (int sweep = 0; sweep < 60; ++sweep) {
-        double off = lane < PS * (PS - 1) / 2 ? Ar[oi][oj] * Ar[oi][oj] + Ai[oi][oj] * Ai[oi][oj] : 0.0;
-        double dia = lane < PS ? Ar[lane][lane] * Ar[lane][lane] : 0.0;
+    for (int sweep = 0; sweep < sweeps; ++sweep) {
+        T off = lane < PS * (PS - 1) / 2 ? Ar[oi][oj] * Ar[oi][oj] + Ai[oi][oj] * Ai[oi][oj] : (T)0;
+        T dia = lane < PS ? Ar[lane][lane] * Ar[lane][lane] : (T)0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             off += __shfl_xor_sync(0xffffffffu, off, o);
             dia += __shfl_xor_sync(0xffffffffu, dia, o);
         }
-        if (off <= 1e-32 * dia || off == 0.0) break;      // same value in every lane
+        if (off <= tol * dia || off == (T)0) break;       // same value in every lane
         __syncwarp();
         for (int r = 0; r < PS - 1; ++r) {
             // pair of rotation i in round r
@@ -611,41 +623,36 @@ __device__ void jacobi_herm8_warp(double (*Ar)[PS], double (*Ai)[PS], double (*V
             if (lane < 4) {
                 int p = at(lane), q = at(PS - 1 - lane);
                 if (p > q) { const int t = p; p = q; q = t; }
-                const double xr = Ar[p][q], xi = Ai[p][q];
-                const double r2 = xr * xr + xi * xi;
-                const double app = Ar[p][p], aqq = Ar[q][q];
-                double* R = rot[lane];
-                R[6] = p;
-                R[7] = q;
-                R[8] = app;
-                R[9] = aqq;
-                // FP64 division and square root are long sequences on this GPU: |a_pq|, its phase and
-                // theta share one reciprocal square root, c takes another
-                if (r2 == 0.0 || r2 < 1e-34 * fabs(app * aqq)) {
-                    R[5] = 1.0;
+                const T xr = Ar[p][q], xi = Ai[p][q];
+                const T r2 = xr * xr + xi * xi;
+                const T app = Ar[p][p], aqq = Ar[q][q];
+                T* R = rot[lane];
+                R[5] = (T)p;
+                R[6] = (T)q;
+                if (r2 < (T)1e-36) {                      // below rounding of the largest entry, squared
+                    R[4] = (T)1;
                 } else {
-                    const double ir = rsqrt(r2), rr = r2 * ir;
-                    const double th = 0.5 * (aqq - app) * ir;
-                    double t;
-                    if (fabs(th) > 1e150) t = 0.5 / th;
-                    else t = (th >= 0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
-                    const double c = rsqrt(t * t + 1.0);
+                    const T ir = jac_rsqrt(r2);
+                    const float th = 0.5f * (float)((aqq - app) * ir);
+                    const float tf = fabsf(th) > 1e18f ? 0.5f / th
+                                                       : copysignf(1.f, th) / (fabsf(th) + sqrtf(fmaf(th, th, 1.f)));
+                    const T t = (T)tf;
+                    const T c = jac_rsqrt(t * t + (T)1);
                     R[0] = xr * ir;
                     R[1] = xi * ir;
                     R[2] = c;
                     R[3] = t * c;
-                    R[4] = t * rr;
-                    R[5] = 0.0;
+                    R[4] = (T)0;
                 }
             }
             __syncwarp();
-            const double* R = rot[pr_i];
-            const bool skip = R[5] != 0.0;
-            const int p = (int)R[6], q = (int)R[7];
-            const double er = R[0], ei = R[1], c = R[2], sn = R[3];
+            const T* R = rot[pr_i];
+            const bool skip = R[4] != (T)0;
+            const int p = (int)R[5], q = (int)R[6];
+            const T er = R[0], ei = R[1], c = R[2], sn = R[3];
             if (!skip) {     // columns p, q: a_kp <- c a_kp - s conj(e) a_kq ; a_kq <- s a_kp + c conj(e) a_kq
-                const double pr = Ar[k][p], pi = Ai[k][p], qr = Ar[k][q], qi = Ai[k][q];
-                const double mr = er * qr + ei * qi, mi = er * qi - ei * qr;
+                const T pr = Ar[k][p], pi = Ai[k][p], qr = Ar[k][q], qi = Ai[k][q];
+                const T mr = er * qr + ei * qi, mi = er * qi - ei * qr;
                 Ar[k][p] = c * pr - sn * mr;
                 Ai[k][p] = c * pi - sn * mi;
                 Ar[k][q] = sn * pr + c * mr;
@@ -653,34 +660,102 @@ __device__ void jacobi_herm8_warp(double (*Ar)[PS], double (*Ai)[PS], double (*V
             }
             __syncwarp();
             if (!skip) {     // rows p, q: a_pk <- c a_pk - s e a_qk ; a_qk <- s a_pk + c e a_qk ; and V
-                const double pr = Ar[p][k], pi = Ai[p][k], qr = Ar[q][k], qi = Ai[q][k];
-                const double mr = er * qr - ei * qi, mi = er * qi + ei * qr;
+                const T pr = Ar[p][k], pi = Ai[p][k], qr = Ar[q][k], qi = Ai[q][k];
+                const T mr = er * qr - ei * qi, mi = er * qi + ei * qr;
                 Ar[p][k] = c * pr - sn * mr;
-                Ai[p][k] = c * pi - sn * mi;
+                Ai[p][k] = k == p ? (T)0 : c * pi - sn * mi;
                 Ar[q][k] = sn * pr + c * mr;
-                Ai[q][k] = sn * pi + c * mi;
-                const double vpr = Vr[k][p], vpi = Vi[k][p], vqr = Vr[k][q], vqi = Vi[k][q];
-                const double nr = er * vqr + ei * vqi, ni = er * vqi - ei * vqr;
+                Ai[q][k] = k == q ? (T)0 : sn * pi + c * mi;
+                const T vpr = Vr[k][p], vpi = Vi[k][p], vqr = Vr[k][q], vqi = Vi[k][q];
+                const T nr = er * vqr + ei * vqi, ni = er * vqi - ei * vqr;
                 Vr[k][p] = c * vpr - sn * nr;
                 Vi[k][p] = c * vpi - sn * ni;
                 Vr[k][q] = sn * vpr + c * nr;
                 Vi[k][q] = sn * vpi + c * ni;
             }
             __syncwarp();
-            if (lane < 4) {
-                // the rotated 2x2 block: diagonal a_pp - t r, a_qq + t r (a_pp, a_qq before the round), zero pivot
-                const double* Rl = rot[lane];
-                const int pl = (int)Rl[6], ql = (int)Rl[7];
-                if (Rl[5] == 0.0) {
-                    Ar[pl][pl] = Rl[8] - Rl[4];
-                    Ar[ql][ql] = Rl[9] + Rl[4];
-                    Ai[pl][pl] = Ai[ql][ql] = 0.0;
-                }
-                Ar[pl][ql] = Ai[pl][ql] = Ar[ql][pl] = Ai[ql][pl] = 0.0;
-            }
-            __syncwarp();
         }
     }
+}
+
+// O = X Y (or X^H Y) of 8 x 8 complex matrices, by one warp.
+template <bool HERM>
+__device__ __forceinline__ void mat8_mul(double (*Or)[PS], double (*Oi)[PS], double (*Xr)[PS], double (*Xi)[PS],
+                                         double (*Yr)[PS], double (*Yi)[PS], int lane) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int i = (lane >> 3) + 4 * h, j = lane & 7;
+        double sr = 0.0, si = 0.0;
+#pragma unroll
+        for (int k = 0; k < PS; ++k) {
+            const double xr = HERM ? Xr[k][i] : Xr[i][k], xi = HERM ? -Xi[k][i] : Xi[i][k];
+            const double yr = Yr[k][j], yi = Yi[k][j];
+            sr = fma(xr, yr, fma(-xi, yi, sr));
+            si = fma(xr, yi, fma(xi, yr, si));
+        }
+        Or[i][j] = sr;
+        Oi[i][j] = si;
+    }
+    __syncwarp();
+}
+
+struct EigWork {
+    double A[2][PS][PS], V[2][PS][PS], B[2][PS][PS], W[2][PS][PS];
+    float a[2][PS][PS], v[2][PS][PS];
+    double rot[4][8];
+    float rotf[4][8];
+};
+
+// Eigenvalues (diagonal of w.A) and eigenvectors (columns of w.V) of the Hermitian matrix in w.A, by one
+// warp. w.A is scaled by a power of two (exact; the eigenvectors and eigenvalue ratios do not change).
+__device__ void eig_herm8_warp(EigWork& w, int lane) {
+    double mx = lane < PS ? fabs(w.A[0][lane][lane]) : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    int ex = 0;
+    if (mx > 0.0) ex = ilogb(mx) + 1;
+    for (int e = lane; e < PS2; e += 32) {
+        const int i = e >> 3, j = e & 7;
+        const double ar = ldexp(w.A[0][i][j], -ex), ai = ldexp(w.A[1][i][j], -ex);
+        w.A[0][i][j] = ar;
+        w.A[1][i][j] = ai;
+        w.a[0][i][j] = (float)ar;
+        w.a[1][i][j] = (float)ai;
+        w.v[0][i][j] = i == j ? 1.f : 0.f;
+        w.v[1][i][j] = 0.f;
+    }
+    __syncwarp();
+    jacobi_herm8_warp<float>(w.a[0], w.a[1], w.v[0], w.v[1], w.rotf, 1e-13f, 8, lane);
+    __syncwarp();
+    for (int e = lane; e < PS2; e += 32) {
+        const int i = e >> 3, j = e & 7;
+        w.V[0][i][j] = (double)w.v[0][i][j];
+        w.V[1][i][j] = (double)w.v[1][i][j];
+    }
+    __syncwarp();
+    // V <- V (3 - V^H V) / 2, twice: orthonormal to 1e-6, 1e-12, rounding
+    for (int it = 0; it < 2; ++it) {
+        mat8_mul<true>(w.B[0], w.B[1], w.V[0], w.V[1], w.V[0], w.V[1], lane);
+        for (int e = lane; e < PS2; e += 32) {
+            const int i = e >> 3, j = e & 7;
+            w.B[0][i][j] = (i == j ? 1.5 : 0.0) - 0.5 * w.B[0][i][j];
+            w.B[1][i][j] = -0.5 * w.B[1][i][j];
+        }
+        __syncwarp();
+        mat8_mul<false>(w.W[0], w.W[1], w.V[0], w.V[1], w.B[0], w.B[1], lane);
+        for (int e = lane; e < PS2; e += 32) {
+            const int i = e >> 3, j = e & 7;
+            w.V[0][i][j] = w.W[0][i][j];
+            w.V[1][i][j] = w.W[1][i][j];
+        }
+        __syncwarp();
+    }
+    // A <- V^H A V
+    mat8_mul<false>(w.B[0], w.B[1], w.A[0], w.A[1], w.V[0], w.V[1], lane);
+    mat8_mul<true>(w.A[0], w.A[1], w.V[0], w.V[1], w.B[0], w.B[1], lane);
+    if (lane < PS) w.A[1][lane][lane] = 0.0;
+    __syncwarp();
+    jacobi_herm8_warp<double>(w.A[0], w.A[1], w.V[0], w.V[1], w.rot, 1e-32, 60, lane);
 }
 
 // One warp per (U or V, slice f) problem w, f = 0 .. C/2; writes its slice of the outputs.
@@ -688,15 +763,14 @@ __device__ __forceinline__ void basis_problem(const unsigned long long* __restri
                                               double* __restrict__ b64, float* __restrict__ b32,
                                               double* __restrict__ gap_out) {
     __shared__ double Res[PS][PS][2];
-    __shared__ double work[4 * PS2];
-    __shared__ double rot[5][10];
+    __shared__ EigWork work;
     const int nf = C / 2 + 1;
     const int lane = threadIdx.x & 31;
     const int which = w / nf, f = w % nf;
-    double (*Ar)[PS] = reinterpret_cast<double (*)[PS]>(work);
-    double (*Ai)[PS] = reinterpret_cast<double (*)[PS]>(work + PS2);
-    double (*Vr)[PS] = reinterpret_cast<double (*)[PS]>(work + 2 * PS2);
-    double (*Vi)[PS] = reinterpret_cast<double (*)[PS]>(work + 3 * PS2);
+    double (*Ar)[PS] = work.A[0];
+    double (*Ai)[PS] = work.A[1];
+    double (*Vr)[PS] = work.V[0];
+    double (*Vi)[PS] = work.V[1];
     const unsigned long long* M = mom + (size_t)which * PS * PS * C * C;
     // w^k, w = exp(-2 pi i / C), k < C: exact constants for C = 3, the library's cospi / sinpi otherwise
     __shared__ double phr[64], phi[64];
@@ -738,7 +812,7 @@ __device__ __forceinline__ void basis_problem(const unsigned long long* __restri
         Ai[u][v] = u == v ? 0.0 : acci;
     }
     __syncwarp();
-    jacobi_herm8_warp(Ar, Ai, Vr, Vi, rot, lane);
+    eig_herm8_warp(work, lane);
     __shared__ int order[PS];
     canonicalise_warp(Ar, Vr, Vi, Res, order, lane);
     if (gap_out && lane == 0) {
@@ -931,11 +1005,16 @@ extern "C" int htsvd_internal_basis(const unsigned long long* d_mom, int C, doub
 
 cudaError_t launch_moments(const uint8_t* img, const Geo& g, unsigned long long* d_mom, cudaStream_t s) {
     const int n = g.ngroups();
-    const int blocks = (n + MOM_CHUNK - 1) / MOM_CHUNK;
+    // about two CTAs per SM where there are references enough, in whole staging batches (a 481 x 321 image has
+    // 66 chunks of 256 references: 148 us alone on the chip)
+    const int want = 2 * device_sm_count();
+    int per = ((n + want - 1) / want + MOM_BATCH - 1) / MOM_BATCH * MOM_BATCH;
+    if (per > MOM_CHUNK) per = MOM_CHUNK;
+    const int blocks = (n + per - 1) / per;
     cudaError_t e = cudaMemsetAsync(d_mom, 0, sizeof(unsigned long long) * 2 * PS2 * g.C * g.C, s);
     if (e != cudaSuccess) return e;
-    if (g.C == 3) moments_kernel<3><<<blocks, 256, 0, s>>>(img, g, d_mom);
-    else moments_kernel<1><<<blocks, 256, 0, s>>>(img, g, d_mom);
+    if (g.C == 3) moments_kernel<3><<<blocks, 256, 0, s>>>(img, g, per, d_mom);
+    else moments_kernel<1><<<blocks, 256, 0, s>>>(img, g, per, d_mom);
     return cudaGetLastError();
 }
 
