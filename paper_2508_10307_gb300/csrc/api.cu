@@ -131,6 +131,8 @@ enum Slot {
     S_IDX, S_MOM, S_B64, S_B32, S_PART, S_FULLM, S_FULLS, S_RANKS, S_IDX2, S_Q, S_DEN, S_R, S_TMP,
     S_AIN, S_AOUT,                   // S_AIN, S_AOUT: parts of the adaptive image and volume calls
     S_COEF, S_CPN, S_CNRM,           // coefficient cache of htsvd_denoise_tau_sweep
+    S_PLANE, S_PNRM, S_SPILL, S_CTR, S_DOT, // group filter: projection planes, patch norms, spilled rows,
+                                                // tile counter, patch products of the VJP
     S_SOUT, S_SGX, S_SIDX, S_SRED,   // htsvd_sure: estimate, adjoint or perturbed image, grouping, sums
     S_GAP,                           // eigen-gaps of the basis slices (strict mode)
     S_WIDX0, S_WIDX1, S_WB64, S_WB32, S_WZ, S_WF, S_WU, S_WGX, S_WG2, S_WRED,   // weight tuning by SURE
@@ -140,6 +142,12 @@ enum Slot {
     S_VMOM, S_VB64, S_VNUM, S_VDEN,  // MRI volumes: moments, bases, numerator, denominator
     S_NSLOT
 };
+
+// Largest workspace taken for projection planes. A 3840 x 2160 RGB frame's plane (6.3 GB) fits, so that
+// every image of the usual sizes is filtered in one band; larger ones are cut into bands of tile rows,
+// whose planes overlap by a footprint (43 position rows at window 31), and the 32-bit element offsets
+// of a plane stay below 2^31.
+constexpr size_t kPlaneBytes = (size_t)8 << 30;
 
 struct Workspace {
     int device = -1;
@@ -152,6 +160,7 @@ struct Workspace {
                                           // block matching
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int* timeout = nullptr;               // pinned word a kernel sets when one of its waits runs out
+    size_t plane_cap = kPlaneBytes;       // most it may hold as projection planes
 };
 
 std::mutex g_mu;
@@ -453,12 +462,6 @@ htsvd_status finish_sigma(const void* hbuf, const Geo& g, const Resolved& r, dou
     return HTSVD_OK;
 }
 
-struct FilterOut {
-    float* out;
-    float* den_out;
-};
-
-// Filter + reduce for the forward pass.
 // Coefficient cache of the noisy groups (FM_ANALYZE writes it, FM_SYNTH reads it).
 struct CoefCache {
     float* coef;
@@ -467,6 +470,87 @@ struct CoefCache {
     int mode;                // FM_ANALYZE or FM_SYNTH
 };
 
+// Position rows of the planes that the tile rows [t0, t1) gather from.
+void band_rows(const Geo& g, int TR, int t0, int t1, int& y0, int& y1) {
+    int lo, hi;
+    tile_span(t0, TR, g.nry, g.s, g.H, g.npy, g.wny, g.win, lo, hi);
+    y0 = lo;
+    tile_span(t1 - 1, TR, g.nry, g.s, g.H, g.npy, g.wny, g.win, lo, hi);
+    y1 = hi - PS + 1;
+}
+
+// Projection planes of the band's rows: coefficients and patch norms of every frame in reach.
+struct Planes {
+    float* coef = nullptr;
+    float* pn = nullptr;
+    int* counter = nullptr;
+    int* sample = nullptr;       // launch_sample_rows' words
+    const int* dense = nullptr;  // its verdict, where it is asked
+    long long stride = 0;        // positions per frame
+    int y0 = 0, y1 = 0;          // position rows held
+};
+
+// Tile rows per band: as many as fit the workspace's share; where the device cannot give that much, halved until
+// the planes can be allocated (at least one tile row).
+htsvd_status plane_bands(Workspace* w, const Geo& g, int TR, int nty, int ntiles, int nfr, int& per, Planes& P) {
+    const size_t row = (size_t)g.npx * nfr;                       // positions per plane row, all frames
+    for (per = nty;; per = (per + 1) / 2) {
+        int most = 0;
+        for (int t = 0; t < nty; t += per) {
+            int y0, y1;
+            band_rows(g, TR, t, std::min(nty, t + per), y0, y1);
+            most = std::max(most, y1 - y0);
+        }
+        const size_t bytes = (size_t)most * row * PS2 * g.C * sizeof(float);
+        if ((bytes > w->plane_cap || most > 65535) && per > 1) continue;
+        void *c, *n, *k;
+        const htsvd_status st = ws_get(w, S_PLANE, bytes, &c);
+        if (st != HTSVD_OK) {
+            if (per > 1) continue;
+            return st;
+        }
+        ST(ws_get(w, S_PNRM, (size_t)most * row * sizeof(float), &n));
+        ST(ws_get(w, S_CTR, sizeof(int) * (2 + (size_t)ntiles + 3), &k));
+        P.coef = (float*)c;
+        P.pn = (float*)n;
+        P.counter = (int*)k;
+        P.sample = P.counter + 2 + ntiles;
+        return HTSVD_OK;
+    }
+}
+
+htsvd_status fill_planes(const void* img, int is_float, const Geo& g, const float* b32, int y0, int y1,
+                         const VideoCtx* vc, Planes& P, cudaStream_t s) {
+    const int nfr = vc ? vc->nfr : 1;
+    P.y0 = y0;
+    P.y1 = y1;
+    P.stride = (long long)(y1 - y0) * g.npx;
+    for (int f = 0; f < nfr; ++f) {
+        PlaneArgs pa{};
+        pa.img = vc ? (const void*)(vc->vid + (vc->f0 + f) * vc->fstride) : img;
+        pa.is_float = is_float;
+        pa.H = g.H;
+        pa.W = g.W;
+        pa.C = g.C;
+        pa.py0 = y0;
+        pa.rows = y1 - y0;
+        pa.basis32 = b32;
+        pa.coef = P.coef + f * P.stride * PS2 * g.C;
+        pa.pn = P.pn + f * P.stride;
+        pa.counter = P.counter;
+        pa.dense = P.dense;
+        ProfScope ps_("planes", s);
+        CK(launch_plane(pa, s));
+    }
+    return HTSVD_OK;
+}
+
+// References from which the projection planes pay: planes and filter against the tile kernel alone, us per
+// call: RGB, K 32: 131 / 123 at 2,704 references, 172 / 182 at 4,225, 261 / 300 at 7,056; gray, K 32: 53 / 41
+// at 1,681, 79 / 81 at 2,704, 103 / 123 at 4,225.
+constexpr int kPlaneGroups = 3000;
+
+// Filter + reduce for the forward pass.
 htsvd_status run_forward_filter(Workspace* w, const void* img, int is_float, const Geo& g, const Resolved& r,
                                 const int32_t* idx, const double* b64, const float* b32, double tau,
                                 const float* w_in, const htsvd_params* p, float* d_out, cudaStream_t s,
@@ -474,7 +558,8 @@ htsvd_status run_forward_filter(Workspace* w, const void* img, int is_float, con
     const int mode = vc ? FM_VIDEO : cc ? cc->mode : FM_FORWARD;
     FilterTiling t = choose_filter_tiling(g, is_float ? 4 : 1, mode, r.tile, vc ? vc->nfr : 1);
     if (t.TR == 0) return HTSVD_ERR_UNSUPPORTED;
-    FilterArgs a{};
+    GroupArgs ga{};
+    FilterArgs& a = ga.f;
     a.img = img;
     a.img_is_float = is_float;
     a.g = g;
@@ -508,7 +593,7 @@ htsvd_status run_forward_filter(Workspace* w, const void* img, int is_float, con
     a.mask_out = p ? p->d_mask_out : nullptr;
     a.weights_out = p ? p->d_weights_out : nullptr;
     a.coef_out = p ? p->d_coef_out : nullptr;
-    void* part;
+    void *part, *spill = nullptr;
     const int acc = g.C == 3 ? 4 : 2;
     ST(ws_get(w, S_PART, sizeof(float) * (size_t)t.ntx * t.nty * t.FHmax * t.FWmax * acc, &part));
     a.partials = (float*)part;
@@ -517,7 +602,56 @@ htsvd_status run_forward_filter(Workspace* w, const void* img, int is_float, con
         CK(launch_filter(a, s));
         return HTSVD_OK;
     }
-    { ProfScope ps_(mode == FM_SYNTH ? "filter_synth" : "filter", s); CK(launch_filter(a, s)); }
+    // the projection planes where they pay and the device has room for them, else the tile kernel alone
+    Planes P;
+    int per = t.nty, grid = 0;
+    bool planes = !cc && g.ngroups() >= kPlaneGroups;
+    if (planes) {
+        htsvd_status st = plane_bands(w, g, t.TR, t.nty, t.nty * t.ntx, vc ? vc->nfr : 1, per, P);
+        if (st == HTSVD_OK) {
+            ga.nty_band = per;
+            grid = group_grid(ga);
+            st = ws_get(w, S_SPILL, sizeof(float) * group_spill_floats(ga, grid), &spill);
+        }
+        if (st != HTSVD_OK && st != HTSVD_ERR_OOM) return st;
+        planes = st == HTSVD_OK;
+    }
+    if (!planes) {
+        { ProfScope ps_(cc ? "filter_synth" : "filter", s); CK(launch_filter(a, s)); }
+        { ProfScope ps_("reduce", s); CK(launch_reduce((float*)part, g, t.TR, t.ntx, t.nty, t.FHmax, t.FWmax, d_out, nullptr, 0, nullptr, s)); }
+        return HTSVD_OK;
+    }
+    ga.spill = (float*)spill;
+    if (r.K > 8) {                             // (with fewer slots the group filter is the faster one at any threshold)
+        ProfScope ps_("sample_rows", s);
+        CK(cudaMemsetAsync(P.sample, 0, 3 * sizeof(int), s));
+        CK(launch_sample_rows(a, P.sample, s));
+        P.dense = a.dense = P.sample + 2;
+    }
+    if (a.mask_out)
+        CK(cudaMemsetAsync(a.mask_out, 0, sizeof(uint32_t) * (size_t)g.ngroups() * (g.K * PS2 * g.C / 32), s));
+    for (int t0 = 0; t0 < t.nty; t0 += per) {
+        const int t1 = std::min(t.nty, t0 + per);
+        int y0, y1;
+        band_rows(g, t.TR, t0, t1, y0, y1);
+        ST(fill_planes(img, is_float, g, b32, y0, y1, vc, P, s));
+        ga.coef = P.coef;
+        ga.pn = P.pn;
+        ga.planestride = P.stride;
+        ga.py0 = P.y0;
+        ga.counter = P.counter;
+        ga.ty0 = t0;
+        ga.nty_band = t1 - t0;
+        ProfScope ps_("filter", s);
+        CK(launch_group(ga, std::min(grid, (t1 - t0) * t.ntx), s));
+        if (r.K > 8) {                         // (below that no group has rows enough to be left over)
+            a.left = P.counter;
+            a.left_first = t0 * t.ntx;
+            a.left_tiles = (t1 - t0) * t.ntx;
+            CK(launch_filter(a, s));
+            a.left = nullptr;
+        }
+    }
     { ProfScope ps_("reduce", s); CK(launch_reduce((float*)part, g, t.TR, t.ntx, t.nty, t.FHmax, t.FWmax, d_out, nullptr, 0, nullptr, s)); }
     return HTSVD_OK;
 }
@@ -531,13 +665,9 @@ struct HostEvent {
     }
 };
 
-htsvd_status denoise_impl(const void* d_in, int is_float, int H, int W, int C, double sigma, const htsvd_params* p,
-                          const float* d_w, float* d_out, int32_t* d_idx_out, cudaStream_t s) {
-    if (!d_in || !d_out) return HTSVD_ERR_INVALID_ARG;
-    Resolved r;
-    ST(resolve(p, C, r));
-    ST(check_image(H, W, C, r));
-    if (std::isnan(sigma)) return HTSVD_ERR_INVALID_ARG;
+// Alg. 1 with the arguments checked.
+htsvd_status denoise_checked(const void* d_in, int is_float, int H, int W, int C, double sigma, const htsvd_params* p,
+                             const Resolved& r, const float* d_w, float* d_out, int32_t* d_idx_out, cudaStream_t s) {
     Workspace* w = workspace_for(s);
     if (!w) return HTSVD_ERR_OOM;
     const Geo g = make_geo(H, W, C, r.s, r.win, r.K);
@@ -588,6 +718,16 @@ htsvd_status denoise_impl(const void* d_in, int is_float, int H, int W, int C, d
     const double tau = r.tau_mult * sigma;
     return run_forward_filter(w, is_float ? d_in : (const void*)q, is_float, g, r, idx, b64, b32, tau, d_w, p, d_out,
                               s);
+}
+
+htsvd_status denoise_impl(const void* d_in, int is_float, int H, int W, int C, double sigma, const htsvd_params* p,
+                          const float* d_w, float* d_out, int32_t* d_idx_out, cudaStream_t s) {
+    if (!d_in || !d_out) return HTSVD_ERR_INVALID_ARG;
+    Resolved r;
+    ST(resolve(p, C, r));
+    ST(check_image(H, W, C, r));
+    if (std::isnan(sigma)) return HTSVD_ERR_INVALID_ARG;
+    return denoise_checked(d_in, is_float, H, W, C, sigma, p, r, d_w, d_out, d_idx_out, s);
 }
 
 // A clip, frame by frame (real-world color video denoising, Sec. IV): output frame t is Alg. 1 on
@@ -714,9 +854,10 @@ htsvd_status vjp_core(Workspace* w, const float* d_x, const Geo& g, const Resolv
     ST(ws_get(w, S_TMP, sizeof(float) * npix * C, &tmp));
 
     // D = sum_g w_g Scatter_g 1
-    FilterTiling td = choose_filter_tiling(g, 4, FM_DENOM, r.tile);
-    if (td.TR == 0) return HTSVD_ERR_UNSUPPORTED;
-    FilterArgs a{};
+    const FilterTiling t = choose_filter_tiling(g, 4, FM_ADJOINT, r.tile);
+    if (t.TR == 0) return HTSVD_ERR_UNSUPPORTED;
+    GroupArgs ga{};
+    FilterArgs& a = ga.f;
     a.img = d_x;
     a.img_is_float = 1;
     a.g = g;
@@ -729,37 +870,74 @@ htsvd_status vjp_core(Workspace* w, const float* d_x, const Geo& g, const Resolv
     a.band_abs = (float)(tau * kBandTau) + 1e-6f;
     a.w_in = d_w;
     a.agg_mode = 0;
-    a.mode = FM_DENOM;
-    a.TR = td.TR;
-    a.ntx = td.ntx;
-    a.nty = td.nty;
-    a.FHmax = td.FHmax;
-    a.FWmax = td.FWmax;
+    a.TR = t.TR;
+    a.ntx = t.ntx;
+    a.nty = t.nty;
+    a.FHmax = t.FHmax;
+    a.FWmax = t.FWmax;
     const int acc = C == 3 ? 4 : 2;
-    void* part;
-    ST(ws_get(w, S_PART, sizeof(float) * (size_t)td.ntx * td.nty * td.FHmax * td.FWmax * acc, &part));
+    void *part, *spill = nullptr, *rc, *dot;
+    ST(ws_get(w, S_PART, sizeof(float) * (size_t)t.ntx * t.nty * t.FHmax * t.FWmax * acc, &part));
     a.partials = (float*)part;
-    { ProfScope ps_("filter", s); CK(launch_filter(a, s)); }
-    { ProfScope ps_("reduce", s); CK(launch_reduce((float*)part, g, td.TR, td.ntx, td.nty, td.FHmax, td.FWmax, (float*)tmp, (float*)den, 0,
+    Geo g1 = g;
+    g1.C = 1;
+    { ProfScope ps_("denom", s); CK(launch_denom(a, s)); }
+    { ProfScope ps_("reduce", s); CK(launch_reduce((float*)part, g1, t.TR, t.ntx, t.nty, t.FHmax, t.FWmax, (float*)tmp, (float*)den, 0,
                      nullptr, s)); }
     { ProfScope ps_("div", s); CK(launch_div(d_grad_out, (const float*)den, npix, C, (float*)rimg, s)); }
 
-    // adjoint filter on r = gout / D with the masks of x
-    FilterTiling ta = choose_filter_tiling(g, 4, FM_ADJOINT, r.tile);
-    if (ta.TR == 0) return HTSVD_ERR_UNSUPPORTED;
+    // adjoint filter on r = gout / D with the masks of x: the planes of both images in the same bands
     a.mode = FM_ADJOINT;
-    a.TR = ta.TR;
-    a.ntx = ta.ntx;
-    a.nty = ta.nty;
-    a.FHmax = ta.FHmax;
-    a.FWmax = ta.FWmax;
     a.r_img = (const float*)rimg;
     a.out_img = d_out;
     a.grad_w = d_grad_w;
-    ST(ws_get(w, S_PART, sizeof(float) * (size_t)ta.ntx * ta.nty * ta.FHmax * ta.FWmax * acc, &part));
-    a.partials = (float*)part;
-    { ProfScope ps_("filter", s); CK(launch_filter(a, s)); }
-    { ProfScope ps_("reduce", s); CK(launch_reduce((float*)part, g, ta.TR, ta.ntx, ta.nty, ta.FHmax, ta.FWmax, d_grad_x, nullptr, 1, nullptr, s)); }
+    Planes P, R;
+    int per = t.nty, grid = 0;
+    htsvd_status st = plane_bands(w, g, t.TR, t.nty, t.nty * t.ntx, 2, per, P);       // (two images: as two frames)
+    if (st == HTSVD_OK) {
+        ga.nty_band = per;
+        grid = group_grid(ga);
+        st = ws_get(w, S_SPILL, sizeof(float) * group_spill_floats(ga, grid), &spill);
+    }
+    if (st != HTSVD_OK && st != HTSVD_ERR_OOM) return st;
+    if (st != HTSVD_OK) {                          // no room for the planes: the tile kernel alone
+        ProfScope ps_("adjoint", s);
+        CK(launch_filter(a, s));
+        per = t.nty + 1;
+    }
+    ga.spill = (float*)spill;
+    for (int t0 = 0; per <= t.nty && t0 < t.nty; t0 += per) {
+        const int t1 = std::min(t.nty, t0 + per);
+        int y0, y1;
+        band_rows(g, t.TR, t0, t1, y0, y1);
+        const size_t pos = (size_t)(y1 - y0) * g.npx;
+        R.coef = P.coef + pos * PS2 * C;
+        R.pn = P.pn + pos;                                 // (not used)
+        R.counter = P.counter;
+        ST(fill_planes(d_x, 1, g, b32, y0, y1, nullptr, P, s));
+        ST(fill_planes(rimg, 1, g, b32, y0, y1, nullptr, R, s));
+        rc = R.coef;
+        ST(ws_get(w, S_DOT, sizeof(float) * pos, &dot));
+        { ProfScope ps_("patch_dot", s); CK(launch_patch_dot((const float*)rimg, d_out, g.H, g.W, C, y0, y1 - y0, (float*)dot, s)); }
+        ga.coef = P.coef;
+        ga.pn = P.pn;
+        ga.rcoef = (const float*)rc;
+        ga.dot = (const float*)dot;
+        ga.planestride = P.stride;
+        ga.py0 = P.y0;
+        ga.counter = P.counter;
+        ga.ty0 = t0;
+        ga.nty_band = t1 - t0;
+        ProfScope ps_("adjoint", s);
+        CK(launch_group(ga, std::min(grid, (t1 - t0) * t.ntx), s));
+        if (r.K > 8) {
+            a.left = P.counter;
+            a.left_tiles = (t1 - t0) * t.ntx;
+            CK(launch_filter(a, s));
+            a.left = nullptr;
+        }
+    }
+    { ProfScope ps_("reduce", s); CK(launch_reduce((float*)part, g, t.TR, t.ntx, t.nty, t.FHmax, t.FWmax, d_grad_x, nullptr, 1, nullptr, s)); }
     return HTSVD_OK;
 }
 

@@ -1088,7 +1088,7 @@ __device__ __forceinline__ void filter_tile_fwd(const FilterArgs& a, const int t
                 }
                 if (a.coef_out) {
                     float* cdst = a.coef_out + (size_t)grp * K * NF;
-                    haar_for_each<K>([&](int m, int sl, int L) { cdst[m * NF + fib] = v[sl] * rsqrtf((float)L); });
+                    haar_for_each<K>([&](int m, int sl, int L) { cdst[m * NF + fib] = v[sl] * (1.f / sqrtf((float)L)); });
                 }
                 // decided coefficients are scaled (kept, by 1 / L) or zeroed in place; a coefficient
                 // inside the band keeps its raw value until it is decided
@@ -1540,7 +1540,17 @@ __device__ __forceinline__ void filter_tile(const FilterArgs& a, const int tile,
 template <int K, int C, typename Tin, int MODE>
 __global__ void __launch_bounds__(FT_THREADS, 2) filter_kernel(FilterArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
-    filter_tile<K, C, Tin, MODE>(a, blockIdx.x, smem);
+    int tile = blockIdx.x;
+    if (a.left) {                             // the tiles the group filter left over, or every one (blocks beyond: none)
+        if (a.dense && *a.dense) {
+            tile += a.left_first;
+            if ((int)blockIdx.x >= a.left_tiles) return;
+        } else {
+            if (tile >= a.left[1]) return;
+            tile = a.left[2 + tile];
+        }
+    }
+    filter_tile<K, C, Tin, MODE>(a, tile, smem);
 }
 
 // Persistent form over the tiles of many images (same K and C): work item w -> image by prefix[].
@@ -1577,7 +1587,7 @@ cudaError_t launch_filter_t(const FilterArgs& a, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
-    fn<<<a.ntx * a.nty, FT_THREADS, L.total, s>>>(a);
+    fn<<<a.left ? a.left_tiles : a.ntx * a.nty, FT_THREADS, L.total, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,328 @@
+// Dispatch of the group filter on projection planes.
+#include <algorithm>
+#include <type_traits>
+
+#include "group_impl.cuh"
+
+namespace htsvd {
+
+namespace {
+
+template <int K, int C, typename Tin, bool MF, bool ADJ = false>
+cudaError_t launch_group_t(const GroupArgs& a, int grid, cudaStream_t s) {
+    const int smem = group_layout<C>(a.f.FHmax, a.f.FWmax, a.cap, ADJ).total;
+    auto fn = group_kernel<K, C, Tin, MF, ADJ>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e != cudaSuccess) return e;
+    fn<<<grid, GR_THREADS, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <int K, int C>
+cudaError_t dispatch(const GroupArgs& a, int grid, cudaStream_t s) {
+    if (a.f.mode == FM_ADJOINT)
+        return a.f.img_is_float ? launch_group_t<K, C, float, false, true>(a, grid, s) : cudaErrorInvalidValue;
+    if (a.f.mode == FM_VIDEO) return a.f.img_is_float ? cudaErrorInvalidValue : launch_group_t<K, C, uint8_t, true>(a, grid, s);
+    return a.f.img_is_float ? launch_group_t<K, C, float, false>(a, grid, s)
+                            : launch_group_t<K, C, uint8_t, false>(a, grid, s);
+}
+
+template <int C>
+cudaError_t dispatch_k(const GroupArgs& a, int grid, cudaStream_t s) {
+    switch (a.f.g.K) {
+        case 2: return dispatch<2, C>(a, grid, s);
+        case 4: return dispatch<4, C>(a, grid, s);
+        case 8: return dispatch<8, C>(a, grid, s);
+        case 16: return dispatch<16, C>(a, grid, s);
+        case 32: return dispatch<32, C>(a, grid, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+GLayout layout_of(const GroupArgs& a, int cap) {
+    const bool adj = a.f.mode == FM_ADJOINT;
+    return a.f.g.C == 3 ? group_layout<3>(a.f.FHmax, a.f.FWmax, cap, adj)
+                        : group_layout<1>(a.f.FHmax, a.f.FWmax, cap, adj);
+}
+
+// Rows of coefficients that the groups keep, from SR_GROUPS groups spread over the image: one CTA per group
+// projects its patches, takes the Haar transform of every coefficient across them and counts the (slot, basis
+// row) pairs with a coefficient above the threshold. The last CTA compares the mean with the rows up to which
+// the group filter is the faster one (see dense_mean). 9 us, most of it the latency of one group.
+constexpr int SR_GROUPS = 128;
+
+// Mean rows per group at which planes and group filter take as long as filter_tile_fwd alone (us per image, both,
+// by the mean rows): RGB 512 x 512, K 32, stride 3: 611 / 721 at 22, 763 / 750 at 34, 915 / 758 at 39,
+// 1,110 / 820 at 65; RGB 512 x 512, K 16: 473 / 571 at 34, 554 / 619 at 46, 781 / 659 at 61; gray 1280 x 720,
+// K 32: 1,025 / 1,234 at 23, 1,138 / 1,251 at 33, 1,367 / 1,268 at 40.
+__host__ __device__ constexpr int dense_mean(int K) { return K == 32 ? 32 : 48; }
+
+template <int K, int C, typename Tin, bool MF>
+__global__ void __launch_bounds__(K * PS) sample_rows_kernel(FilterArgs a, int* __restrict__ st) {
+    constexpr int NC = C == 3 ? 3 : 1, NF = PS2 * NC;              // floats of a patch
+    __shared__ float sm[K * NF];                                    // [k][i][b or j][NC]
+    __shared__ unsigned mask[PS];
+    const Geo& g = a.g;
+    const int tid = threadIdx.x, ng = g.nry * g.nrx;
+    const int grp = (int)((2ll * blockIdx.x + 1) * ng / (2 * SR_GROUPS));
+    if (tid < PS) mask[tid] = 0u;
+    {
+        // column b of patch k: Y[i][b] = sum_a conj(U[a][i]) X(a, b)
+        const int k = tid >> 3, b = tid & 7;
+        int v = max(a.idx[(size_t)grp * K + k], 0);
+        const Tin* img = reinterpret_cast<const Tin*>(a.img);
+        if constexpr (MF) {
+            const int hw = g.H * g.W, f = v / hw;
+            img = reinterpret_cast<const Tin*>(a.vid) + (size_t)min(f, a.f0 + a.nfr - 1) * a.fstride;
+            v -= f * hw;
+        }
+        const int y = min(v / g.W, g.H - PS), x = min(v % g.W, g.W - PS);
+        float s0[PS] = {}, sr[PS] = {}, si[PS] = {};
+#pragma unroll 2
+        for (int r = 0; r < PS; ++r) {
+            const Tin* p = img + ((size_t)(y + r) * g.W + x + b) * C;
+            if constexpr (C == 3) {
+                const float v0 = (float)p[0], v1 = (float)p[1], v2 = (float)p[2];
+                const float X0 = v0 + v1 + v2, Xr = v0 - 0.5f * (v1 + v2), Xi = G_S3H * (v2 - v1);
+#pragma unroll
+                for (int i = 0; i < PS; ++i) {
+                    const float ur = a.basis32[64 + r * PS + i], ui = a.basis32[128 + r * PS + i];
+                    s0[i] = fmaf(a.basis32[r * PS + i], X0, s0[i]);
+                    sr[i] = fmaf(ur, Xr, fmaf(ui, Xi, sr[i]));
+                    si[i] = fmaf(ur, Xi, fmaf(-ui, Xr, si[i]));
+                }
+            } else {
+                const float X0 = (float)p[0];
+#pragma unroll
+                for (int i = 0; i < PS; ++i) s0[i] = fmaf(a.basis32[r * PS + i], X0, s0[i]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < PS; ++i) {
+            float* d = sm + k * NF + (i * PS + b) * NC;
+            d[0] = s0[i];
+            if constexpr (C == 3) {
+                d[1] = sr[i];
+                d[2] = si[i];
+            }
+        }
+    }
+    __syncthreads();
+    {
+        // row i of patch k: S[i][j] = sum_b Y[i][b] V[b][j] and the inverse channel DFT, over its own floats
+        float* row = sm + (tid >> 3) * NF + (tid & 7) * PS * NC;
+        float s0[PS] = {}, sr[PS] = {}, si[PS] = {};
+        const float* V = a.basis32 + (C == 3 ? 192 : 64);
+#pragma unroll 2
+        for (int b = 0; b < PS; ++b) {
+            const float y0 = row[b * NC], yr = C == 3 ? row[b * NC + (C == 3 ? 1 : 0)] : 0.f;
+            const float yi = C == 3 ? row[b * NC + (C == 3 ? 2 : 0)] : 0.f;
+#pragma unroll
+            for (int j = 0; j < PS; ++j) {
+                s0[j] = fmaf(y0, V[b * PS + j], s0[j]);
+                if constexpr (C == 3) {
+                    const float vr = V[64 + b * PS + j], vi = V[128 + b * PS + j];
+                    sr[j] = fmaf(yr, vr, fmaf(-yi, vi, sr[j]));
+                    si[j] = fmaf(yr, vi, fmaf(yi, vr, si[j]));
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < PS; ++j) {
+            if constexpr (C == 3) {
+                row[j * 3] = (s0[j] + 2.f * sr[j]) * G_THIRD;
+                row[j * 3 + 1] = (s0[j] - sr[j] - G_SQ3 * si[j]) * G_THIRD;
+                row[j * 3 + 2] = (s0[j] - sr[j] + G_SQ3 * si[j]) * G_THIRD;
+            } else {
+                row[j] = s0[j];
+            }
+        }
+    }
+    __syncthreads();
+    for (int t = tid; t < NF; t += K * PS) {
+        // coefficient t across the patches (unnormalised: the threshold grows with the support)
+        float p[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) p[k] = sm[k * NF + t];
+#pragma unroll
+        for (int d = 1; d < K; d <<= 1)
+#pragma unroll
+            for (int m = 0; m < K; m += 2 * d) {
+                const float x = p[m], y = p[m + d];
+                p[m + d] = x - y;
+                p[m] = x + y;
+            }
+        unsigned keep = 0u;
+#pragma unroll
+        for (int l = 0; l < K; ++l)
+            if (fabsf(p[l]) >= a.tau32 * g_root(l == 0 ? g_ctz(K) : g_ctz(l) + 1)) keep |= 1u << l;
+        atomicOr(&mask[t / (PS * NC)], keep);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        int rows = 0;
+        for (int i = 0; i < PS; ++i) rows += __popc(mask[i]);
+        atomicAdd(st, rows);
+        __threadfence();
+        if (atomicAdd(st + 1, 1) == SR_GROUPS - 1) st[2] = atomicAdd(st, 0) > dense_mean(K) * SR_GROUPS;
+    }
+}
+
+template <int K>
+cudaError_t sample_rows(const FilterArgs& a, int* st, cudaStream_t s) {
+    const bool mf = a.mode == FM_VIDEO;
+    if (a.g.C == 3) {
+        if (mf) sample_rows_kernel<K, 3, uint8_t, true><<<SR_GROUPS, K * PS, 0, s>>>(a, st);
+        else if (a.img_is_float) sample_rows_kernel<K, 3, float, false><<<SR_GROUPS, K * PS, 0, s>>>(a, st);
+        else sample_rows_kernel<K, 3, uint8_t, false><<<SR_GROUPS, K * PS, 0, s>>>(a, st);
+    } else {
+        if (mf) sample_rows_kernel<K, 1, uint8_t, true><<<SR_GROUPS, K * PS, 0, s>>>(a, st);
+        else if (a.img_is_float) sample_rows_kernel<K, 1, float, false><<<SR_GROUPS, K * PS, 0, s>>>(a, st);
+        else sample_rows_kernel<K, 1, uint8_t, false><<<SR_GROUPS, K * PS, 0, s>>>(a, st);
+    }
+    return cudaGetLastError();
+}
+
+// Denominator sum_g w_g (patches covering a pixel) of a tile of references: the weights are added at the
+// patches' origins (the K positions of a group are distinct, one lane each, groups in order: a fixed order of
+// sums), and every pixel takes the 8 x 8 box sum of the origins that reach it. Partials as the group
+// filter's for one channel, (0, denominator). 32 adds per group in place of 2,048 weights.
+constexpr int DN_THREADS = 128;
+
+__global__ void __launch_bounds__(DN_THREADS) denom_kernel(FilterArgs a) {
+    extern __shared__ float dsm[];
+    const Geo& g = a.g;
+    const int tid = threadIdx.x, ty = blockIdx.x / a.ntx, tx = blockIdx.x - ty * a.ntx;
+    int FY0, FY1, FX0, FX1;
+    tile_span(ty, a.TR, g.nry, g.s, g.H, g.npy, g.wny, g.win, FY0, FY1);
+    tile_span(tx, a.TR, g.nrx, g.s, g.W, g.npx, g.wnx, g.win, FX0, FX1);
+    const int FH = FY1 - FY0, FW = FX1 - FX0, OH = FH - PS + 1, OW = FW - PS + 1;
+    float* org = dsm;                                  // [OH][OW]
+    float* row = dsm + a.FHmax * a.FWmax;              // [OH][FW]: sums of 8 origins along x
+    for (int t = tid; t < OH * OW; t += DN_THREADS) org[t] = 0.f;
+    __syncthreads();
+    if (tid < 32) {
+        const int iy0 = ty * a.TR, ix0 = tx * a.TR;
+        const int th = min(a.TR, g.nry - iy0), tw = min(a.TR, g.nrx - ix0);
+        for (int q = 0; q < th * tw; ++q) {
+            const int grp = (iy0 + q / tw) * g.nrx + ix0 + q % tw;
+            const float w = a.w_in ? a.w_in[grp] : 1.f;
+            if (tid < g.K) {
+                // (a caller-given index outside the footprint is clamped into it; two lanes may then meet)
+                const int v = a.idx[(size_t)grp * g.K + tid];
+                const int y = v / g.W, x = v - y * g.W;
+                const int oy = min(max(y - FY0, 0), OH - 1), ox = min(max(x - FX0, 0), OW - 1);
+                atomicAdd(org + oy * OW + ox, w);
+            }
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    for (int t = tid; t < OH * FW; t += DN_THREADS) {
+        const int y = t / FW, x = t - y * FW;
+        float s = 0.f;
+        for (int j = max(0, x - OW + 1); j < PS && j <= x; ++j) s += org[y * OW + x - j];
+        row[t] = s;
+    }
+    __syncthreads();
+    float2* dst = reinterpret_cast<float2*>(a.partials) + (size_t)blockIdx.x * a.FHmax * a.FWmax;
+    for (int t = tid; t < FH * FW; t += DN_THREADS) {
+        const int y = t / FW, x = t - y * FW;
+        float s = 0.f;
+        for (int i = max(0, y - OH + 1); i < PS && i <= y; ++i) s += row[(y - i) * FW + x];
+        dst[y * a.FWmax + x] = make_float2(0.f, s);
+    }
+}
+
+// dot[position] = <patch of u, patch of v> over the image (8 x 8 box sums of the channels' products), rows
+// py0 .. py0 + rows - 1 of positions.
+constexpr int DP_X = 64, DP_Y = 16;
+
+__global__ void __launch_bounds__(256) patch_dot_kernel(const float* __restrict__ u, const float* __restrict__ v, int H,
+                                                        int W, int C, int py0, int rows, float* __restrict__ dot) {
+    __shared__ float e[DP_Y + PS - 1][DP_X + PS], hs[DP_Y + PS - 1][DP_X];
+    const int x0 = blockIdx.x * DP_X, r0 = blockIdx.y * DP_Y, y0 = py0 + r0, tid = threadIdx.x;
+    for (int t = tid; t < (DP_Y + PS - 1) * (DP_X + PS - 1); t += 256) {
+        const int r = t / (DP_X + PS - 1), c = t - r * (DP_X + PS - 1);
+        float s = 0.f;
+        if (y0 + r < H && x0 + c < W) {
+            const size_t p = ((size_t)(y0 + r) * W + x0 + c) * C;
+            for (int k = 0; k < C; ++k) s = fmaf(u[p + k], v[p + k], s);
+        }
+        e[r][c] = s;
+    }
+    __syncthreads();
+    for (int t = tid; t < (DP_Y + PS - 1) * DP_X; t += 256) {
+        const int r = t / DP_X, c = t - r * DP_X;
+        float s = 0.f;
+#pragma unroll
+        for (int j = 0; j < PS; ++j) s += e[r][c + j];
+        hs[r][c] = s;
+    }
+    __syncthreads();
+    for (int t = tid; t < DP_Y * DP_X; t += 256) {
+        const int r = t / DP_X, c = t - r * DP_X;
+        if (r0 + r >= rows || x0 + c > W - PS) continue;
+        float s = 0.f;
+#pragma unroll
+        for (int i = 0; i < PS; ++i) s += hs[r + i][c];
+        dot[(size_t)(r0 + r) * (W - PS + 1) + x0 + c] = s;
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_sample_rows(const FilterArgs& a, int* st, cudaStream_t s) {
+    return a.g.K == 32 ? sample_rows<32>(a, st, s) : a.g.K == 16 ? sample_rows<16>(a, st, s) : cudaErrorInvalidValue;
+}
+
+cudaError_t launch_denom(const FilterArgs& a, cudaStream_t s) {
+    const size_t smem = 2 * sizeof(float) * a.FHmax * a.FWmax;
+    cudaError_t e = cudaFuncSetAttribute(denom_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    denom_kernel<<<a.ntx * a.nty, DN_THREADS, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_patch_dot(const float* u, const float* v, int H, int W, int C, int py0, int rows, float* dot,
+                             cudaStream_t s) {
+    patch_dot_kernel<<<dim3((W - PS + DP_X) / DP_X, (rows + DP_Y - 1) / DP_Y), 256, 0, s>>>(u, v, H, W, C, py0, rows, dot);
+    return cudaGetLastError();
+}
+
+int group_grid(GroupArgs& a) {
+    // as many CTAs per SM as the registers allow and whose accumulators leave room for the row lists
+    const int rows = a.f.g.K * PS;                        // every row of every slot
+    const int row_bytes = GR_WARPS * PS * a.f.g.C * 4;     // all warps
+    const int fixed = layout_of(a, 0).total + 1024 + 64;
+    int per_sm = 1;
+    a.cap = std::min(rows, 8);
+    for (int n = GR_CTAS; n >= 1; --n) {
+        const int room = 228 * 1024 / n - fixed;
+        const int cap = std::min(rows, room / row_bytes);
+        if (cap >= std::min(rows, 16) || n == 1) {
+            per_sm = n;
+            a.cap = std::max(cap, 0);
+            break;
+        }
+    }
+    // Candidate rows of a first step from which a tile is left to filter_tile_fwd. us per 512 x 512 RGB image, K 32,
+    // stride 3, for limits 12 / 18 / 24 / 30 / 38: 973 / 897 / 908 / 842 / 838 at sigma 25 and multiplier 3.2,
+    // 860 / 816 / 762 / 764 / 763 at sigma 15 and 4.2, 1,483 / 1,489 / 1,479 / 1,781 / 1,860 at sigma 8 and 2.0. With
+    // 8 patches or fewer a group has 64 rows at most and nothing is left.
+    a.dense_rows = a.f.g.K <= 8 ? 1 << 20 : 30;
+    return std::min(a.nty_band * a.f.ntx, per_sm * device_sm_count());
+}
+
+size_t group_spill_floats(const GroupArgs& a, int grid) {
+    return (size_t)grid * GR_WARPS * group_spill_warp(a.f.g.K, a.f.g.C);
+}
+
+cudaError_t launch_group(const GroupArgs& args, int grid, cudaStream_t s) {
+    GroupArgs a = args;
+    a.wrec = (unsigned)(((unsigned long long)1 << 32) / (unsigned)a.f.g.W);
+    return a.f.g.C == 3 ? dispatch_k<3>(a, grid, s) : dispatch_k<1>(a, grid, s);
+}
+
+}  // namespace htsvd

@@ -66,6 +66,22 @@ inline int basis32_floats(int C) { return (C == 1 || C == 3) ? 512 : 2 * (C / 2 
 // Quantise a float image: q = clip(rint(x), 0, 255).
 cudaError_t launch_quantize(const float* x, int64_t n, uint8_t* q, cudaStream_t s);
 
+// ---- projection planes (plane.cu): the projected patch at every position of the image rows
+// py0 .. py0 + rows - 1 (positions), 64 C floats each in the group filter's lane order, and its
+// squared norm. basis32: the packed FP32 bases of launch_basis.
+struct PlaneArgs {
+    const void* img;         // uint8 or float H x W x C
+    int is_float;
+    int H, W, C;
+    int py0, rows;
+    const float* basis32;
+    float* coef;             // [rows][W - 7][64 C]
+    float* pn;               // [rows][W - 7]
+    int* counter;            // optional: two words zeroed (the group filter's counters)
+    const int* dense;        // optional: nothing else is done where it is set
+};
+cudaError_t launch_plane(const PlaneArgs& a, cudaStream_t s);
+
 // ---- group filter and aggregation (filter.cu)
 enum FilterMode { FM_FORWARD = 0, FM_DENOM = 1, FM_ADJOINT = 2, FM_VIDEO = 3, FM_ANALYZE = 4, FM_SYNTH = 5 };
 
@@ -114,7 +130,46 @@ struct FilterArgs {
     float* cache_coef;
     float* cache_pn;
     int* cache_nrm;
+    // Tiles to filter (optional, device): counter[1] of them from counter[2] on, as the group filter leaves them.
+    const int* left;
+    // Where dense points to a word that is set: all left_tiles tiles from left_first on (the group filter has done none).
+    const int* dense;
+    int left_first, left_tiles;
 };
+// Group filter on projection planes (group.cu): the tiles of tile rows ty0 .. ty0 + nty_band - 1, their
+// groups' coefficients gathered from the planes (one per frame in reach, planestride positions apart)
+// instead of projected in the CTA; same partials as launch_filter. FM_FORWARD and FM_VIDEO.
+struct GroupArgs {
+    FilterArgs f;
+    const float* coef;
+    const float* pn;
+    long long planestride;   // positions per frame plane
+    int py0;                 // image row of the planes' first position row
+    int ty0, nty_band;
+    int cap;                 // rows of kept coefficients a warp holds in shared memory
+    float* spill;            // rows beyond cap, group_spill_floats(...) in all
+    const float* rcoef;      // adjoint: planes of r
+    const float* dot;        // adjoint: per position, <patch of r, patch of the output>
+    // [0] tile counter, [1] number of tiles left over, [2 ...] those tiles: [0] and [1] zero at launch. A tile is
+    // left over (no partial written) where its first groups keep more than dense_rows rows.
+    int* counter;
+    int dense_rows;
+    unsigned wrec;           // 2^32 / W, rounded down (filled by the launch)
+};
+// Sets st[2] where the sampled groups of the image keep more rows of coefficients than the group filter is the
+// faster one for (st: three zeroed words); FilterArgs as for the filter. K 16 or 32.
+cudaError_t launch_sample_rows(const FilterArgs& a, int* st, cudaStream_t s);
+// Fills a.cap and returns the grid (persistent CTAs) of a launch.
+int group_grid(GroupArgs& a);
+size_t group_spill_floats(const GroupArgs& a, int grid);
+cudaError_t launch_group(const GroupArgs& a, int grid, cudaStream_t s);
+
+// Denominator partials of a tiling (two floats per footprint pixel, (0, sum of the covering patches' weights)).
+cudaError_t launch_denom(const FilterArgs& a, cudaStream_t s);
+// dot[position] = <patch of u, patch of v> of two float images, position rows py0 .. py0 + rows - 1.
+cudaError_t launch_patch_dot(const float* u, const float* v, int H, int W, int C, int py0, int rows, float* dot,
+                             cudaStream_t s);
+
 size_t filter_smem_bytes(const FilterArgs& a);
 cudaError_t launch_filter(const FilterArgs& a, cudaStream_t s);
 // out[p] = sum_tiles num / sum_tiles den (deterministic tile order). If den_out is set, the
