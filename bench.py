@@ -444,7 +444,7 @@ def make_workload(name):
         outs = [None]
         cfg = {"workload": "batch64_rgb_uneven", "images": "64 RGB uint8, W~U{256..2048}, H~U{256..1536}",
                "noise": "gaussian, sigma_j~U(10,50)", "sigma": "given per image", "ps": 8, "stride": 3,
-               "window": 31, "K": 32, "form": "one persistent launch per phase, CUDA graph replay, autotuned tiles"}
+               "window": 31, "K": 32, "form": "images side by side on eight streams"}
 
         def step(d):
             if outs[0] is None:

@@ -226,13 +226,9 @@ htsvd_status htsvd_denoise_adaptive(const uint8_t* d_noisy, int32_t H, int32_t W
                                     cudaStream_t stream);
 
 /* Alg. 1 on n uint8 images of any sizes (one C for the whole batch) with per-image sigma
- * (>= 0). Each phase (moments, bases, grouping, filter, reduction) is one persistent launch
- * whose CTAs take (image, tile) work items from a queue over all images; the sequence is
- * captured into a CUDA graph that later calls with the same images, sizes, sigmas and
- * parameters replay. The first call for a new batch shape also times candidate tile shapes
- * (autotuning) and synchronises `stream`; replays do not synchronise. If `stream` cannot be
- * captured (for instance because the caller is capturing it), the sequence runs eagerly.
- * Optional outputs of p are ignored. */
+ * (>= 0). The images are spread, largest first, over up to eight streams of the library, each with
+ * a workspace of its own; they start after the work already in `stream` and `stream` continues
+ * after the last of them. No synchronisation with the host. Optional outputs of p are ignored. */
 htsvd_status htsvd_denoise_batch(const htsvd_image* h_imgs, int32_t n, const htsvd_params* p,
                                  cudaStream_t stream);
 

@@ -68,11 +68,12 @@ int resolve_mode(const Resolved& r, int C) {
 
 // ----------------------------------------------------------------------------- tiling choices
 
-FilterTiling choose_filter_tiling(const Geo& g, int in_bytes, int mode, int forced, int nfr) {
+FilterTiling choose_filter_tiling(const Geo& g, int in_bytes, int mode, int forced, int nfr, int share) {
     // Among the tiles whose shared memory lets two CTAs share an SM (228 KB, 1 KB reserved per
     // CTA): the largest that still gives 8 waves of two CTAs per SM (the last, partial wave then
     // costs little), else the largest with one such wave, else the largest that fits at all. A
     // forced edge is taken as given if its shared memory fits a CTA (TR = 0 returned otherwise).
+    // Images that run side by side (share of them) make the waves together.
     const int cands[] = {8, 7, 6, 5, 4, 3, 2, 1};
     const int64_t nsm = device_sm_count();
     FilterTiling fit2{}, fit1{}, wave1{};
@@ -110,7 +111,7 @@ FilterTiling choose_filter_tiling(const Geo& g, int in_bytes, int mode, int forc
         fa.nfr = nfr;
         const size_t smem = filter_smem_bytes(fa);
         if (smem <= 112 * 1024) {
-            const int64_t tiles = (int64_t)t.ntx * t.nty;
+            const int64_t tiles = (int64_t)t.ntx * t.nty * share;
             if (!have2) fit2 = t, have2 = true;
             if (tiles >= 8 * 2 * nsm) return t;
             if (tiles >= 2 * nsm && !havew) wave1 = t, havew = true;
@@ -149,6 +150,10 @@ enum Slot {
 // of a plane stay below 2^31.
 constexpr size_t kPlaneBytes = (size_t)8 << 30;
 
+// Images of a batch in flight at a time. Their kernels overlap at their ends (a small image's moments, bases
+// and last tiles leave most of the chip idle); planes are limited to kPlaneBytes over all lanes.
+constexpr int kBatchLanes = 8;
+
 struct Workspace {
     int device = -1;
     cudaStream_t stream = nullptr;
@@ -161,6 +166,11 @@ struct Workspace {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int* timeout = nullptr;               // pinned word a kernel sets when one of its waits runs out
     size_t plane_cap = kPlaneBytes;       // most it may hold as projection planes
+    int share = 1;                        // images that run side by side (the lanes of a batch)
+    // htsvd_denoise_batch: the streams its images run on (each with a workspace of its own), and their events
+    cudaStream_t lane[kBatchLanes] = {};
+    cudaEvent_t ev_lane[kBatchLanes] = {};
+    cudaEvent_t ev_batch = nullptr;
 };
 
 std::mutex g_mu;
@@ -325,7 +335,7 @@ htsvd_status run_block_match(Workspace* w, const uint8_t* q, const Geo& g, const
     bm_fit_tiles(a);
     if (bm_smem_bytes(a) > 227 * 1024) return HTSVD_ERR_UNSUPPORTED;   // e.g. too many frames in reach
     a.idx = idx;
-    if (const size_t tcb = bm_tc_scratch(a)) {
+    if (const size_t tcb = bm_tc_scratch(a, w->share)) {
         void* scratch;
         if (ws_get(w, S_BMTC, tcb, &scratch) == HTSVD_OK) {
             if (!w->timeout) {
@@ -556,7 +566,7 @@ htsvd_status run_forward_filter(Workspace* w, const void* img, int is_float, con
                                 const float* w_in, const htsvd_params* p, float* d_out, cudaStream_t s,
                                 const VideoCtx* vc = nullptr, const CoefCache* cc = nullptr) {
     const int mode = vc ? FM_VIDEO : cc ? cc->mode : FM_FORWARD;
-    FilterTiling t = choose_filter_tiling(g, is_float ? 4 : 1, mode, r.tile, vc ? vc->nfr : 1);
+    FilterTiling t = choose_filter_tiling(g, is_float ? 4 : 1, mode, r.tile, vc ? vc->nfr : 1, w->share);
     if (t.TR == 0) return HTSVD_ERR_UNSUPPORTED;
     GroupArgs ga{};
     FilterArgs& a = ga.f;
@@ -1103,6 +1113,66 @@ htsvd_status htsvd_estimate_sigma(const uint8_t* d_noisy, int32_t H, int32_t W, 
     ST(launch_sigma_inputs(w, d_noisy, g, r, stream, &hbuf));
     CK(cudaStreamSynchronize(stream));
     return finish_sigma(hbuf, g, r, h_sigma);
+}
+
+htsvd_status htsvd_denoise_batch(const htsvd_image* imgs, int32_t n, const htsvd_params* p, cudaStream_t s) {
+    if (n < 0 || (n > 0 && !imgs)) return HTSVD_ERR_INVALID_ARG;
+    if (n == 0) return HTSVD_OK;
+    // every image is checked before any device work
+    htsvd_params q;
+    std::memset(&q, 0, sizeof(q));
+    if (p) q = *p;
+    q.h_sigma_out = nullptr;                 // the single-image outputs have no place in a batch
+    q.d_mask_out = nullptr;
+    q.d_weights_out = nullptr;
+    q.d_basis_out = nullptr;
+    q.d_coef_out = nullptr;
+    q.strict_basis = 0;
+    q.h_basis_gap_out = nullptr;
+    Resolved r;
+    ST(resolve(&q, imgs[0].C, r));
+    for (int i = 0; i < n; ++i) {
+        const htsvd_image& im = imgs[i];
+        if (!im.d_in || !im.d_out || !(im.sigma >= 0) || im.C != imgs[0].C || (im.C != 1 && im.C != 3) || im.H < PS ||
+            im.W < PS)
+            return HTSVD_ERR_INVALID_ARG;
+        const Geo g = make_geo(im.H, im.W, im.C, r.s, r.win, r.K);
+        if ((int64_t)g.wny * g.wnx < r.K) return HTSVD_ERR_INVALID_ARG;
+        if (choose_filter_tiling(g, 1, FM_FORWARD, r.tile).TR == 0) return HTSVD_ERR_UNSUPPORTED;
+    }
+    Workspace* w = workspace_for(s);
+    if (!w) return HTSVD_ERR_OOM;
+    const int lanes = std::min(n, kBatchLanes);
+    if (!w->ev_batch) CK(cudaEventCreateWithFlags(&w->ev_batch, cudaEventDisableTiming));
+    for (int l = 0; l < lanes; ++l) {
+        if (!w->lane[l]) CK(cudaStreamCreateWithFlags(&w->lane[l], cudaStreamNonBlocking));
+        if (!w->ev_lane[l]) CK(cudaEventCreateWithFlags(&w->ev_lane[l], cudaEventDisableTiming));
+        Workspace* lw = workspace_for(w->lane[l]);
+        if (!lw) return HTSVD_ERR_OOM;
+        lw->plane_cap = kPlaneBytes / kBatchLanes;
+        lw->share = lanes;
+    }
+    // largest images first, each to the lane with the least work so far (a lane's workspace then grows once)
+    std::vector<int> order(n);
+    for (int i = 0; i < n; ++i) order[i] = i;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        return (int64_t)imgs[a].H * imgs[a].W > (int64_t)imgs[b].H * imgs[b].W;
+    });
+    int64_t load[kBatchLanes] = {};
+    CK(cudaEventRecord(w->ev_batch, s));
+    for (int l = 0; l < lanes; ++l) CK(cudaStreamWaitEvent(w->lane[l], w->ev_batch, 0));
+    htsvd_status st = HTSVD_OK;
+    for (int k = 0; k < n && st == HTSVD_OK; ++k) {
+        const htsvd_image& im = imgs[order[k]];
+        const int l = (int)(std::min_element(load, load + lanes) - load);
+        load[l] += (int64_t)im.H * im.W;
+        st = denoise_checked(im.d_in, 0, im.H, im.W, im.C, im.sigma, &q, r, nullptr, im.d_out, im.d_idx_out, w->lane[l]);
+    }
+    for (int l = 0; l < lanes; ++l) {          // joined on every path: the caller's stream covers the lanes' work
+        CK(cudaEventRecord(w->ev_lane[l], w->lane[l]));
+        CK(cudaStreamWaitEvent(s, w->ev_lane[l], 0));
+    }
+    return st;
 }
 
 htsvd_status htsvd_denoise_adaptive(const uint8_t* d_noisy, int32_t H, int32_t W, int32_t C, int32_t sub_h,
@@ -1709,6 +1779,11 @@ htsvd_status htsvd_release_workspace(void) {
             if (w->hpin) cudaFreeHost(w->hpin);
             if (w->timeout) cudaFreeHost(w->timeout);
             if (w->side) cudaStreamDestroy(w->side);
+            for (int l = 0; l < kBatchLanes; ++l) {
+                if (w->lane[l]) cudaStreamDestroy(w->lane[l]);
+                if (w->ev_lane[l]) cudaEventDestroy(w->ev_lane[l]);
+            }
+            if (w->ev_batch) cudaEventDestroy(w->ev_batch);
             if (w->ev_fork) cudaEventDestroy(w->ev_fork);
             if (w->ev_join) cudaEventDestroy(w->ev_join);
             delete w;

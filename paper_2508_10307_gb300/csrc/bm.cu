@@ -601,32 +601,6 @@ __global__ void __launch_bounds__(BM_THREADS, 2) block_match_video_kernel(BMArgs
     bm_tile<true>(a, blockIdx.y, blockIdx.x, bsm);
 }
 
-// Persistent form over the tiles of many images: work item w -> image by prefix[], then tile.
-__global__ void __launch_bounds__(BM_THREADS, 2) block_match_batch_kernel(const BMArgs* __restrict__ args,
-                                                                          const int* __restrict__ prefix, int nimg,
-                                                                          int* __restrict__ counter) {
-    extern __shared__ __align__(16) unsigned char bsm[];
-    __shared__ int item;
-    const int total = prefix[nimg];
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) item = atomicAdd(counter, 1);
-        __syncthreads();
-        const int w = item;
-        if (w >= total) break;
-        int lo = 0, hi = nimg - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (prefix[mid] <= w) lo = mid;
-            else hi = mid - 1;
-        }
-        const BMArgs& a = args[lo];
-        const int t = w - prefix[lo];
-        const int ntx = (a.nrx_s + a.TRx - 1) / a.TRx;
-        bm_tile<false>(a, t / ntx, t % ntx, bsm);
-    }
-}
-
 #include "bm_tc.cuh"
 
 constexpr size_t BM_SMEM_TARGET = 100 * 1024;    // leaves room for two CTAs per SM
@@ -649,20 +623,6 @@ void bm_fit_tiles(BMArgs& a) {
         if (a.TRx >= a.TRy) a.TRx = (a.TRx + 1) / 2;
         else a.TRy = (a.TRy + 1) / 2;
     }
-}
-
-int bm_tiles(const BMArgs& a) {
-    return ((a.nrx_s + a.TRx - 1) / a.TRx) * ((a.nry_s + a.TRy - 1) / a.TRy);
-}
-
-cudaError_t launch_block_match_batch(const BMArgs* d_args, const int* d_prefix, int nimg, size_t smem, int grid,
-                                     int* d_counter, cudaStream_t s) {
-    if (smem > BM_SMEM_MAX) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(block_match_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    block_match_batch_kernel<<<grid, BM_THREADS, smem, s>>>(d_args, d_prefix, nimg, d_counter);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_block_match(const BMArgs& a, cudaStream_t s) {
@@ -756,7 +716,7 @@ cudaError_t launch_bt(const BMArgs& a, const BtPlan& p, void* scratch, int* time
 
 }  // namespace
 
-size_t bm_tc_scratch(const BMArgs& a) {
+size_t bm_tc_scratch(const BMArgs& a, int share) {
     BtPlan p;
     if (!bt_plan(a, p)) return 0;
     const Geo& g = a.g;
@@ -767,8 +727,9 @@ size_t bm_tc_scratch(const BMArgs& a) {
     // us at 84^2 / 106^2 / 170^2 references, tensor cores against CUDA cores: gray, window 21: 74 / 75 / 98
     // against 56 / 96 / 172; RGB, window 18: 91 / 91 / 154 against 73 / 126 / 200; RGB, window 31:
     // 144 / 142 / 214 against 99 / 167 / 297. 8 x 16 tiles (gray, window 31, stride 4): 171 against 146 at
-    // 127^2 references (128 tiles): they wait for a full wave of tiles.
-    if (tiles < (p.TX == 32 ? 76 : 152)) return 0;
+    // 127^2 references (128 tiles): they wait for a full wave of tiles. Images that share the chip (a batch's
+    // lanes) fill it together.
+    if (tiles * share < (p.TX == 32 ? 76 : 152)) return 0;
     return ((p.planes + 255) & ~(size_t)255) + p.svv;
 }
 

@@ -1553,30 +1553,6 @@ __global__ void __launch_bounds__(FT_THREADS, 2) filter_kernel(FilterArgs a) {
     filter_tile<K, C, Tin, MODE>(a, tile, smem);
 }
 
-// Persistent form over the tiles of many images (same K and C): work item w -> image by prefix[].
-template <int K, int C>
-__global__ void __launch_bounds__(FT_THREADS, 2) filter_batch_kernel(const FilterArgs* __restrict__ args,
-                                                                     const int* __restrict__ prefix, int nimg,
-                                                                     int* __restrict__ counter) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int item;
-    const int total = prefix[nimg];
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) item = atomicAdd(counter, 1);
-        __syncthreads();
-        const int w = item;
-        if (w >= total) break;
-        int lo = 0, hi = nimg - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (prefix[mid] <= w) lo = mid;
-            else hi = mid - 1;
-        }
-        filter_tile<K, C, uint8_t, FM_FORWARD>(args[lo], w - prefix[lo], smem);
-    }
-}
-
 template <int K, int C, typename Tin, int MODE>
 cudaError_t launch_filter_t(const FilterArgs& a, cudaStream_t s) {
     const FLayout L = (MODE == FM_FORWARD || MODE == FM_ANALYZE || MODE == FM_SYNTH)

@@ -33,6 +33,7 @@ struct FilterTiling {
 };
 // Tile edge of the group filter: a forced edge (1..16) if its shared memory fits a CTA (TR = 0 if
 // not), else the largest edge that keeps two CTAs per SM and still yields 8 waves.
-FilterTiling choose_filter_tiling(const Geo& g, int in_bytes, int mode, int forced, int nfr = 1);
+FilterTiling choose_filter_tiling(const Geo& g, int in_bytes, int mode, int forced, int nfr = 1,
+                                  int share = 1);
 
 }  // namespace htsvd

@@ -35,7 +35,7 @@ void bm_fit_tiles(BMArgs& a);
 cudaError_t launch_block_match(const BMArgs& a, cudaStream_t s);
 // Tensor-core form: bytes of device scratch it needs (0: not for this geometry, or not faster there), and
 // its launch. timeout: host-readable word set if a wait inside the kernel runs out.
-size_t bm_tc_scratch(const BMArgs& a);
+size_t bm_tc_scratch(const BMArgs& a, int share);
 cudaError_t launch_block_match_tc(const BMArgs& a, void* scratch, int* timeout, cudaStream_t s);
 
 // ---- second moments and bases (moments.cu)
@@ -268,20 +268,6 @@ size_t cube_smem_bytes(int C, int K);
 // CTAs of the persistent cube filter (a few per SM, at most one per group).
 int cube_grid(int C, int K, int64_t ngroups);
 cudaError_t launch_cube_filter(const CubeArgs& a, int grid, cudaStream_t s);
-
-// ---- persistent batch forms over many images (work items -> image by prefix sums)
-int bm_tiles(const BMArgs& a);
-cudaError_t launch_block_match_batch(const BMArgs* d_args, const int* d_prefix, int nimg, size_t smem, int grid,
-                                     int* d_counter, cudaStream_t s);
-int moments_chunks(const Geo& g);
-cudaError_t launch_moments_batch(int C, const BMArgs* d_args, unsigned long long* const* d_moms, const int* d_prefix,
-                                 int nimg, int grid, cudaStream_t s);
-cudaError_t launch_basis_batch(int C, const FilterArgs* d_fargs, unsigned long long* const* d_moms, int nimg,
-                               cudaStream_t s);
-cudaError_t launch_filter_batch(int K, int C, const FilterArgs* d_args, const int* d_prefix, int nimg, size_t smem,
-                                int grid, int* d_counter, cudaStream_t s);
-cudaError_t launch_reduce_batch(int C, const FilterArgs* d_args, float* const* d_outs, const int* d_prefix, int nimg,
-                                int grid, cudaStream_t s);
 
 // ---- sigma adjustment (moments.cu)
 // Rank position a = 1 + #{f : lambda_f < lambda_{K/2}} of each sampled group (Sec. III-D).

@@ -134,23 +134,6 @@ __global__ void __launch_bounds__(256) moments_kernel(const uint8_t* __restrict_
     moments_chunk<C>(img, g, blockIdx.x, per, out);
 }
 
-// Batch form: chunk items of all images, item w -> image by prefix[].
-template <int C>
-__global__ void __launch_bounds__(256) moments_batch_kernel(const BMArgs* __restrict__ args,
-                                                            unsigned long long* const* __restrict__ moms,
-                                                            const int* __restrict__ prefix, int nimg) {
-    const int total = prefix[nimg];
-    for (int w = blockIdx.x; w < total; w += gridDim.x) {
-        int lo = 0, hi = nimg - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (prefix[mid] <= w) lo = mid;
-            else hi = mid - 1;
-        }
-        moments_chunk<C>(args[lo].img, args[lo].g, w - prefix[lo], MOM_CHUNK, moms[lo]);
-    }
-}
-
 // Row and column moments of the reference patches of a cube with any number of bands C, in the
 // layout of moments_chunk ([2][8][8][C][C]): with the 8-byte vectors r_(a,c) = P[a][0..7][c] and
 // q_(b,c) = P[0..7][b][c] of a reference, R[a][a'][c][c'] = sum over references of <r_(a,c), r_(a',c')>
@@ -853,15 +836,6 @@ __global__ void basis_kernel(const unsigned long long* __restrict__ mom, int C, 
     basis_problem(mom, C, blockIdx.x, b64, b32, gap);
 }
 
-// Batch form: block b -> image b / (2 (C/2 + 1)), problem b % (2 (C/2 + 1)).
-__global__ void basis_batch_kernel(const FilterArgs* __restrict__ fargs, unsigned long long* const* __restrict__ moms,
-                                   int C) {
-    const int np = 2 * (C / 2 + 1);
-    const int i = blockIdx.x / np;
-    const FilterArgs& a = fargs[i];
-    basis_problem(moms[i], C, blockIdx.x % np, const_cast<double*>(a.basis64), const_cast<float*>(a.basis32), nullptr);
-}
-
 __global__ void quantize_kernel(const float* __restrict__ x, int64_t n, uint8_t* __restrict__ q) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         float v = rintf(x[i]);
@@ -1015,21 +989,6 @@ cudaError_t launch_moments(const uint8_t* img, const Geo& g, unsigned long long*
     if (e != cudaSuccess) return e;
     if (g.C == 3) moments_kernel<3><<<blocks, 256, 0, s>>>(img, g, per, d_mom);
     else moments_kernel<1><<<blocks, 256, 0, s>>>(img, g, per, d_mom);
-    return cudaGetLastError();
-}
-
-int moments_chunks(const Geo& g) { return (g.ngroups() + MOM_CHUNK - 1) / MOM_CHUNK; }
-
-cudaError_t launch_moments_batch(int C, const BMArgs* d_args, unsigned long long* const* d_moms, const int* d_prefix,
-                                 int nimg, int grid, cudaStream_t s) {
-    if (C == 3) moments_batch_kernel<3><<<grid, 256, 0, s>>>(d_args, d_moms, d_prefix, nimg);
-    else moments_batch_kernel<1><<<grid, 256, 0, s>>>(d_args, d_moms, d_prefix, nimg);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_basis_batch(int C, const FilterArgs* d_fargs, unsigned long long* const* d_moms, int nimg,
-                               cudaStream_t s) {
-    basis_batch_kernel<<<nimg * 2 * (C / 2 + 1), 32, 0, s>>>(d_fargs, d_moms, C);
     return cudaGetLastError();
 }
 
