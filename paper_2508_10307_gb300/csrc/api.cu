@@ -1476,6 +1476,75 @@ htsvd_status htsvd_denoise_cube(const uint8_t* d_cube, int32_t H, int32_t W, int
     return HTSVD_OK;
 }
 
+namespace {
+
+// References from which the planes pay (us per call, window 5, K 32, planes and filter against the filter alone):
+// 173 / 165 at 1,331 references, 181 / 172 at 3,375, 174 / 184 at 6,859, 276 / 401 at 29,791.
+constexpr int64_t kVolPlaneGroups = 5000;
+
+// Filter of a volume: bands of tile planes over the projection planes that fit the workspace's share, or
+// volume_filter_kernel where they do not pay or the device has no room for them.
+htsvd_status run_volume_filter(Workspace* w, const VolFilterArgs& a, int64_t ng, cudaStream_t s) {
+    const VolGeo& g = a.g;
+    const int ntz = volume_tiles_z(g);
+    void *coef, *pn, *rec;
+    bool planes = ng >= kVolPlaneGroups && volume_group_fits(g);
+    int per = ntz;
+    while (planes) {
+        int most = 0;
+        for (int t = 0; t < ntz; t += per) {
+            int z0, z1;
+            volume_band(g, t, std::min(ntz, t + per), z0, z1);
+            most = std::max(most, z1 - z0);
+        }
+        const size_t pos = (size_t)most * g.npy * g.npx;
+        htsvd_status st = HTSVD_ERR_OOM;
+        if (most <= 65535 && pos * 64 * sizeof(float) <= w->plane_cap &&
+            (int64_t)per * volume_tiles_plane(g) < ((int64_t)1 << 31)) {
+            st = ws_get(w, S_PLANE, pos * 64 * sizeof(float), &coef);
+            if (st == HTSVD_OK) st = ws_get(w, S_PNRM, pos * sizeof(float), &pn);
+            if (st == HTSVD_OK) st = ws_get(w, S_SPILL, volume_group_rec_bytes(g, per), &rec);
+        }
+        if (st == HTSVD_OK) break;
+        if (st != HTSVD_ERR_OOM) return st;
+        if (per == 1) planes = false;
+        per = (per + 1) / 2;
+    }
+    if (!planes) {
+        ProfScope ps_("volume_filter", s);
+        CK(launch_volume_filter(a, s));
+        return HTSVD_OK;
+    }
+    if (a.mask_out) CK(cudaMemsetAsync(a.mask_out, 0, sizeof(uint32_t) * 2 * g.K * (size_t)ng, s));
+    for (int t = 0; t < ntz; t += per) {
+        const int tz = std::min(per, ntz - t);
+        int z0, z1;
+        volume_band(g, t, t + tz, z0, z1);
+        VolPlaneArgs pa{};
+        pa.vol = a.vol;
+        pa.D = g.D;
+        pa.H = g.H;
+        pa.W = g.W;
+        pa.pz0 = z0;
+        pa.basis64 = a.basis64;
+        pa.coef = (float*)coef;
+        pa.pn = (float*)pn;
+        { ProfScope ps_("volume_planes", s); CK(launch_volume_plane(pa, z1 - z0, s)); }
+        VolGroupArgs ga{};
+        ga.f = a;
+        ga.coef = (const float*)coef;
+        ga.pn = (const float*)pn;
+        ga.pz0 = z0;
+        ga.tz0 = t;
+        ga.rec = rec;
+        ProfScope ps_("volume_filter", s);
+        CK(launch_volume_group(ga, tz, s));
+    }
+    return HTSVD_OK;
+}
+
+}  // namespace
+
 htsvd_status htsvd_denoise_volume(const uint8_t* d_vol, int32_t D, int32_t H, int32_t W, double sigma,
                                   const htsvd_params* p, float* d_out, int32_t* d_idx_out, cudaStream_t s) {
     if (!d_vol || !d_out || std::isnan(sigma) || std::isinf(sigma)) return HTSVD_ERR_INVALID_ARG;
@@ -1561,7 +1630,7 @@ htsvd_status htsvd_denoise_volume(const uint8_t* d_vol, int32_t D, int32_t H, in
     a.weights_out = p ? p->d_weights_out : nullptr;
     CK(cudaMemsetAsync(num, 0, sizeof(float) * nvox, s));
     CK(cudaMemsetAsync(den, 0, sizeof(float) * nvox, s));
-    { ProfScope ps_("volume_filter", s); CK(launch_volume_filter(a, s)); }
+    ST(run_volume_filter(w, a, ng, s));
     { ProfScope ps_("volume_finalize", s); CK(launch_volume_finalize((const float*)num, (const float*)den, nvox, d_out, s)); }
     return HTSVD_OK;
 }

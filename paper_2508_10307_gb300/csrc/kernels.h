@@ -244,6 +244,33 @@ size_t volume_filter_smem_bytes(const VolGeo& g);
 cudaError_t launch_volume_filter(const VolFilterArgs& a, cudaStream_t s);
 cudaError_t launch_volume_finalize(const float* num, const float* den, long long n, float* out, cudaStream_t s);
 
+// Volume filter on projection planes (volume_group.cu): the projected cube at every position of the z planes
+// pz0 .. pz0 + nz - 1 of positions (64 floats, coefficient order) and its squared norm, gathered by one
+// warp per group; num and den as launch_volume_filter. mask_out words are cleared by the caller.
+struct VolPlaneArgs {
+    const uint8_t* vol;
+    int D, H, W, pz0;
+    const double* basis64;
+    float* coef;             // [nz][H - 3][W - 3][64]
+    float* pn;               // [nz][H - 3][W - 3]
+};
+cudaError_t launch_volume_plane(const VolPlaneArgs& a, int nz, cudaStream_t s);
+struct VolGroupArgs {
+    VolFilterArgs f;
+    const float* coef;
+    const float* pn;
+    int pz0;                 // first z plane of the planes
+    int tz0;                 // first tile plane
+    void* rec;               // volume_group_rec_bytes(g, tile planes)
+};
+bool volume_group_fits(const VolGeo& g);
+int volume_tiles_z(const VolGeo& g);
+int volume_tiles_plane(const VolGeo& g);
+// Position planes [z0, z1) that the tile planes [t0, t1) gather from.
+void volume_band(const VolGeo& g, int t0, int t1, int& z0, int& z1);
+size_t volume_group_rec_bytes(const VolGeo& g, int tz);
+cudaError_t launch_volume_group(const VolGroupArgs& a, int tz, cudaStream_t s);
+
 // ---- hyperspectral cubes (cube.cu): Alg. 1 with C = N bands, one Haar slot of a group at a time
 struct CubeArgs {
     const uint8_t* img;      // H x W x N uint8
