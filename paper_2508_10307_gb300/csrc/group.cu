@@ -49,17 +49,18 @@ GLayout layout_of(const GroupArgs& a, int cap) {
 // Rows of coefficients that the groups keep, from SR_GROUPS groups spread over the image: one CTA per group
 // projects its patches, takes the Haar transform of every coefficient across them and counts the (slot, basis
 // row) pairs with a coefficient above the threshold. The last CTA compares the mean with the rows up to which
-// the group filter is the faster one (see dense_mean). 9 us, most of it the latency of one group.
+// the group filter is the faster one (see dense_mean). 15 us, most of it the latency of one group.
 constexpr int SR_GROUPS = 128;
 
 // Mean rows per group at which planes and group filter take as long as filter_tile_fwd alone (us per image, both,
-// by the mean rows): RGB 512 x 512, K 32, stride 3: 611 / 721 at 22, 763 / 750 at 34, 915 / 758 at 39,
-// 1,110 / 820 at 65; RGB 512 x 512, K 16: 473 / 571 at 34, 554 / 619 at 46, 781 / 659 at 61; gray 1280 x 720,
-// K 32: 1,025 / 1,234 at 23, 1,138 / 1,251 at 33, 1,367 / 1,268 at 40.
-__host__ __device__ constexpr int dense_mean(int K) { return K == 32 ? 32 : 48; }
+// by the mean rows). RGB, K 32: tiles of 5 x 5 groups and more (512 x 512, stride 2): 883 / 1,459 at 17, 1,383 /
+// 1,567 at 41, 2,169 / 1,651 at 61; smaller tiles, whose few groups wait for one another longer (512 x 512, stride
+// 3): 611 / 721 at 22, 763 / 750 at 34, 915 / 758 at 39. K 16: 1,102 / 1,284 at 45, 1,582 / 1,370 at 60. Gray,
+// K 32: 763 / 809 at 34, 859 / 818 at 40.
+int dense_mean(const FilterArgs& a) { return a.g.K == 16 ? 48 : a.g.C == 1 ? 36 : a.TR >= 5 ? 42 : 32; }
 
 template <int K, int C, typename Tin, bool MF>
-__global__ void __launch_bounds__(K * PS) sample_rows_kernel(FilterArgs a, int* __restrict__ st) {
+__global__ void __launch_bounds__(K * PS) sample_rows_kernel(FilterArgs a, int* __restrict__ st, int most) {
     constexpr int NC = C == 3 ? 3 : 1, NF = PS2 * NC;              // floats of a patch
     __shared__ float sm[K * NF];                                    // [k][i][b or j][NC]
     __shared__ unsigned mask[PS];
@@ -165,21 +166,22 @@ __global__ void __launch_bounds__(K * PS) sample_rows_kernel(FilterArgs a, int* 
         for (int i = 0; i < PS; ++i) rows += __popc(mask[i]);
         atomicAdd(st, rows);
         __threadfence();
-        if (atomicAdd(st + 1, 1) == SR_GROUPS - 1) st[2] = atomicAdd(st, 0) > dense_mean(K) * SR_GROUPS;
+        if (atomicAdd(st + 1, 1) == SR_GROUPS - 1) st[2] = atomicAdd(st, 0) > most;
     }
 }
 
 template <int K>
 cudaError_t sample_rows(const FilterArgs& a, int* st, cudaStream_t s) {
     const bool mf = a.mode == FM_VIDEO;
+    const int most = dense_mean(a) * SR_GROUPS;
     if (a.g.C == 3) {
-        if (mf) sample_rows_kernel<K, 3, uint8_t, true><<<SR_GROUPS, K * PS, 0, s>>>(a, st);
-        else if (a.img_is_float) sample_rows_kernel<K, 3, float, false><<<SR_GROUPS, K * PS, 0, s>>>(a, st);
-        else sample_rows_kernel<K, 3, uint8_t, false><<<SR_GROUPS, K * PS, 0, s>>>(a, st);
+        if (mf) sample_rows_kernel<K, 3, uint8_t, true><<<SR_GROUPS, K * PS, 0, s>>>(a, st, most);
+        else if (a.img_is_float) sample_rows_kernel<K, 3, float, false><<<SR_GROUPS, K * PS, 0, s>>>(a, st, most);
+        else sample_rows_kernel<K, 3, uint8_t, false><<<SR_GROUPS, K * PS, 0, s>>>(a, st, most);
     } else {
-        if (mf) sample_rows_kernel<K, 1, uint8_t, true><<<SR_GROUPS, K * PS, 0, s>>>(a, st);
-        else if (a.img_is_float) sample_rows_kernel<K, 1, float, false><<<SR_GROUPS, K * PS, 0, s>>>(a, st);
-        else sample_rows_kernel<K, 1, uint8_t, false><<<SR_GROUPS, K * PS, 0, s>>>(a, st);
+        if (mf) sample_rows_kernel<K, 1, uint8_t, true><<<SR_GROUPS, K * PS, 0, s>>>(a, st, most);
+        else if (a.img_is_float) sample_rows_kernel<K, 1, float, false><<<SR_GROUPS, K * PS, 0, s>>>(a, st, most);
+        else sample_rows_kernel<K, 1, uint8_t, false><<<SR_GROUPS, K * PS, 0, s>>>(a, st, most);
     }
     return cudaGetLastError();
 }
