@@ -12,8 +12,6 @@ cudaError_t dispatch_mode(const FilterArgs& a, cudaStream_t s) {
         case FM_FORWARD:
             return a.img_is_float ? launch_filter_t<K, C, float, FM_FORWARD>(a, s)
                                   : launch_filter_t<K, C, uint8_t, FM_FORWARD>(a, s);
-        case FM_DENOM:
-            return launch_filter_t<K, C, float, FM_DENOM>(a, s);
         case FM_ADJOINT:
             return a.img_is_float ? launch_filter_t<K, C, float, FM_ADJOINT>(a, s) : cudaErrorInvalidValue;
         case FM_VIDEO:

@@ -69,7 +69,7 @@ __host__ __device__ inline FLayout f_layout(int FH, int FW, int in_bytes, int mo
     L.off_rkeep = o; o += 192 * 4;
     L.off_misc = o; o += 16 * 4;
     L.off_acc = o; o += FH * FW * G::ACC * 4;
-    L.off_img = o; o += ((mode == FM_DENOM ? 0 : FH * FW * C * in_bytes) + 15) / 16 * 16;
+    L.off_img = o; o += (FH * FW * C * in_bytes + 15) / 16 * 16;
     L.off_r = o; o += (mode == FM_ADJOINT) ? FH * FW * C * 4 : 0;
     L.total = o;
     return L;
@@ -1326,7 +1326,7 @@ __device__ __forceinline__ void filter_tile(const FilterArgs& a, const int tile,
     float* r_s = reinterpret_cast<float*>(smem + L.off_r);
 
     // Stage the basis, the image footprint and clear the accumulator.
-    if constexpr (MODE != FM_DENOM) {
+    {
         stage_basis<C>(a.basis32, bas, tid);
         const Tin* img = reinterpret_cast<const Tin*>(a.img);
         const int rowb = FW * C;
@@ -1366,7 +1366,7 @@ __device__ __forceinline__ void filter_tile(const FilterArgs& a, const int tile,
         float wg = 1.f;
         float cx[K];          // FM_ADJOINT: coefficients at x of this thread's fibre
         uint32_t keepb = 0;
-        if constexpr (MODE != FM_DENOM) {
+        {
             // ---- A, B on the filtered image
             // A and B of patch k run on threads 8k..8k+7 of one warp (one column or row per thread;
             // the two-wide forms spill here, where the x coefficients stay live): a warp barrier
@@ -1501,16 +1501,14 @@ __device__ __forceinline__ void filter_tile(const FilterArgs& a, const int tile,
             float* ap = acc + (row * FW + px) * G::ACC;
             if constexpr (C == 3) {
                 if (lane < 24) {
-                    if constexpr (MODE != FM_DENOM) {
-                        const int j = lane / 3, c = lane - 3 * (lane / 3);
-                        ap[j * 4 + c] += wg * gb[k * G::GS + i * G::ROW + lane];
-                    }
+                    const int j = lane / 3, c = lane - 3 * (lane / 3);
+                    ap[j * 4 + c] += wg * gb[k * G::GS + i * G::ROW + lane];
                 } else if (MODE != FM_ADJOINT) {
                     ap[(lane - 24) * 4 + 3] += wg;
                 }
             } else {
                 if (lane < 8) {
-                    if constexpr (MODE != FM_DENOM) ap[lane * 2] += wg * gb[k * G::GS + i * G::ROW + lane];
+                    ap[lane * 2] += wg * gb[k * G::GS + i * G::ROW + lane];
                 } else if (lane < 16 && MODE != FM_ADJOINT) {
                     ap[(lane - 8) * 2 + 1] += wg;
                 }

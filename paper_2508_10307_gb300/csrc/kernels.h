@@ -83,7 +83,7 @@ struct PlaneArgs {
 cudaError_t launch_plane(const PlaneArgs& a, cudaStream_t s);
 
 // ---- group filter and aggregation (filter.cu)
-enum FilterMode { FM_FORWARD = 0, FM_DENOM = 1, FM_ADJOINT = 2, FM_VIDEO = 3, FM_ANALYZE = 4, FM_SYNTH = 5 };
+enum FilterMode { FM_FORWARD = 0, FM_ADJOINT = 2, FM_VIDEO = 3, FM_ANALYZE = 4, FM_SYNTH = 5 };
 
 // Guard band of the threshold decision: a coefficient whose FP32 value lies within
 // kBandRel * ||G||_F + kBandTau * tau of tau is decided again in FP64 (||G||_F: Frobenius
