@@ -49,14 +49,6 @@ FP32_LANES_PER_SM = 128          # FP32 FMA lanes per SM (Blackwell)
 MAX_SM_MHZ = 2070.0              # GB300 maximum SM clock
 
 
-# DRAM bytes (read + write) of one launch of the forward filter kernel, from one ncu capture of
-# the current kernel (dram__bytes_read.sum + dram__bytes_write.sum) on the 1920x1080x3 workload,
-# which has the 3840x2160 frames' geometry and tile edge; a 3840x2160 launch scales it by its
-# groups (919,601 / 229,401: the traffic is the tile partials and indices, both proportional).
-FILTER_DRAM_BYTES = {"rgb1080": 37.154816e6 + 304.592384e6,
-                     "rgb4k": (37.154816e6 + 304.592384e6) * 919601 / 229401}
-
-
 def volume_flops_per_group(K: int) -> int:
     """Algorithmic FP32 flops of one group of 4 x 4 x 4 cubes: per cube and direction the per-slice
     projections (slices 0 and 2 real, 2 x 64 MACs each; slice 1 complex, 2 x 64 complex MACs: 1,536
@@ -823,12 +815,13 @@ def run_gpu(args):
     probe = {name: float(_lib.load().htsvd_internal_alu_probe(op, 2048)) for op, name in
              ((0, "ffma"), (1, "imad"), (2, "dp4a"))}
     if dom == "filter":
-        n_launch, ms = prof["filter"]
+        # (the projections are formed by the planes kernel, where the filter takes planes)
+        n_launch, ms = prof["filter"][0], sum(prof[k][1] for k in ("filter", "planes", "sample_rows") if k in prof)
         flops = wl.groups_per_step * filter_flops_per_group(wl.C, wl.K) * args.steps / n_launch
         achieved = flops / (ms / n_launch / 1000.0) / 1e12
         peak = nsm * FP32_LANES_PER_SM * 2 * MAX_SM_MHZ * 1e6 / 1e12
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": FILTER_DRAM_BYTES.get(args.workload), "kernel": "group_filter",
+                "traffic": None, "kernel": "group_filter",
                 "peak_basis": f"FP32 FMA: {nsm} SMs (device query) x {FP32_LANES_PER_SM} lanes x 2 flop x "
                               f"{MAX_SM_MHZ:.0f} MHz (unit counts and max clock); issue-rate probe in this run: "
                               f"{probe['ffma']:.1f} FFMA, {probe['imad']:.1f} IMAD, {probe['dp4a']:.1f} DP4A per SM clock"}
