@@ -42,8 +42,12 @@ typedef enum htsvd_status {
     HTSVD_ERR_UNSUPPORTED = 2,   /* valid for the method, not built here (ps != 8, K > 32, window > 64) */
     HTSVD_ERR_CUDA = 3,          /* a CUDA runtime call failed */
     HTSVD_ERR_OOM = 4,           /* workspace allocation failed */
-    HTSVD_ERR_TIMEOUT = 5,       /* an earlier call on the stream gave up a wait for the tensor cores (bounded, about
-                                    two seconds; no kernel waits on another CTA) */
+    HTSVD_ERR_TIMEOUT = 5,       /* a kernel gave up a wait for the tensor cores (bounded, about two seconds; no kernel
+                                    waits on another CTA) in an earlier call on the stream, or in this call before the
+                                    point where it waits for the device. That call's results are not to be used: its
+                                    groups hold valid positions, but not the nearest ones. Reported once by the next
+                                    call that groups on the tensor cores or returns a host result (for a batch or an
+                                    adaptive call: by the next of these on the same stream); the call after it runs */
     HTSVD_ERR_DEGENERATE_BASIS = 6, /* strict mode only: a global-basis slice has a relative eigen-gap below 1e-9,
                                        so its eigenvectors (and the coefficients) are not unique (Sec. III-B.1) */
 } htsvd_status;

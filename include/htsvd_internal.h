@@ -47,6 +47,10 @@ double htsvd_internal_sigma_from_moments(const unsigned long long* M, const unsi
 int32_t htsvd_internal_sampled_ranks(const uint8_t* d_img, int32_t H, int32_t W, int32_t C, const htsvd_params* p,
                                      int32_t* h_ranks, int32_t max_ranks);
 
+/* Limit of a kernel's wait for the tensor cores in the later calls on stream, in nanoseconds (negative: the
+ * library's own, about two seconds; 0: every wait counts as run out at once). Host only. */
+htsvd_status htsvd_internal_wait_limit(int64_t ns, cudaStream_t stream);
+
 /* Tile edge (references per tile side) that the forward filter of htsvd_denoise takes for an H x W x C
  * uint8 image with parameters p on the current device (it follows the SM count), or -1 on bad
  * arguments. Host only; launches nothing. */

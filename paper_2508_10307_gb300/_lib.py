@@ -102,6 +102,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.htsvd_internal_volume_bases.restype = ctypes.c_double
     lib.htsvd_internal_alu_probe.argtypes = [i32, i32]
     lib.htsvd_internal_alu_probe.restype = ctypes.c_double
+    lib.htsvd_internal_wait_limit.argtypes = [ctypes.c_int64, vp]
     lib.htsvd_internal_filter_tile.argtypes = [i32, i32, i32, P]
     lib.htsvd_internal_filter_tile.restype = i32
     lib.htsvd_internal_noalloc_bytes.argtypes = [i32, i32, i32, P]

@@ -154,6 +154,8 @@ constexpr size_t kPlaneBytes = (size_t)8 << 30;
 // and last tiles leave most of the chip idle); planes are limited to kPlaneBytes over all lanes.
 constexpr int kBatchLanes = 8;
 
+constexpr unsigned long long kWaitLimitNs = 2000000000ull;
+
 struct Workspace {
     int device = -1;
     cudaStream_t stream = nullptr;
@@ -165,6 +167,7 @@ struct Workspace {
                                           // block matching
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int* timeout = nullptr;               // pinned word a kernel sets when one of its waits runs out
+    unsigned long long wait_ns = kWaitLimitNs;   // limit of such a wait
     size_t plane_cap = kPlaneBytes;       // most it may hold as projection planes
     int share = 1;                        // images that run side by side (the lanes of a batch)
     // htsvd_denoise_batch: the streams its images run on (each with a workspace of its own), and their events
@@ -207,6 +210,14 @@ htsvd_status ws_get(Workspace* w, int slot, size_t bytes, void** out) {
     }
     *out = w->buf[slot];
     return HTSVD_OK;
+}
+
+// TIMEOUT, once, where a kernel of the workspace's stream that has run by now gave up a wait.
+htsvd_status take_timeout(Workspace* w) {
+    volatile int* word = w->timeout;
+    if (!word || !*word) return HTSVD_OK;
+    *word = 0;
+    return HTSVD_ERR_TIMEOUT;
 }
 
 // Side stream and fork/join events of a workspace, created on first use.
@@ -342,9 +353,9 @@ htsvd_status run_block_match(Workspace* w, const uint8_t* q, const Geo& g, const
                 CK(cudaMallocHost(&w->timeout, sizeof(int)));
                 *w->timeout = 0;
             }
-            if (*w->timeout) return HTSVD_ERR_TIMEOUT;
+            ST(take_timeout(w));
             ProfScope ps_("block_match", s);
-            CK(launch_block_match_tc(a, scratch, w->timeout, s));
+            CK(launch_block_match_tc(a, scratch, w->timeout, w->wait_ns, s));
             return HTSVD_OK;
         }
     }
@@ -401,12 +412,13 @@ htsvd_status run_basis(Workspace* w, const uint8_t* q, const Geo& g, double** b6
 
 // Strict-mode eigen-gap check: waits for the per-slice gaps of the basis solve (queued on s), writes
 // the smallest to p->h_basis_gap_out and fails with DEGENERATE_BASIS below kDegenerateGap when
-// p->strict_basis is set.
-htsvd_status check_basis_gap(const double* d_gap, int C, const htsvd_params* p, cudaStream_t s) {
+// p->strict_basis is set. The grouping queued on s before has run as well.
+htsvd_status check_basis_gap(Workspace* w, const double* d_gap, int C, const htsvd_params* p, cudaStream_t s) {
     const int n = basis_problems(C);
     std::vector<double> h((size_t)n);
     CK(cudaMemcpyAsync(h.data(), d_gap, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
+    ST(take_timeout(w));
     double m = h[0];
     for (int i = 1; i < n; ++i) m = std::min(m, h[i]);
     if (p->h_basis_gap_out) *p->h_basis_gap_out = m;
@@ -719,7 +731,7 @@ htsvd_status denoise_checked(const void* d_in, int is_float, int H, int W, int C
     CK(cudaStreamWaitEvent(s, w->ev_join, 0));
     if (p && p->d_basis_out)
         CK(cudaMemcpyAsync(p->d_basis_out, b64, sizeof(double) * 2 * 2 * C * PS2, cudaMemcpyDeviceToDevice, s));
-    if (r.strict_basis) ST(check_basis_gap((const double*)gap, C, p, s));
+    if (r.strict_basis) ST(check_basis_gap(w, (const double*)gap, C, p, s));
     if (sigma < 0) {
         if (cudaEventSynchronize(hev.ev) != cudaSuccess) return HTSVD_ERR_CUDA;
         ST(finish_sigma(hbuf, g, r, &sigma));
@@ -1036,6 +1048,7 @@ htsvd_status sure_w_eval(Workspace* w, const SureW& c, const float* d_w, double*
     double h[4];
     CK(cudaMemcpyAsync(h, terms, sizeof(h), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
+    ST(take_timeout(w));
     *h_sure = h[0] / (double)c.n - c.sigma * c.sigma + beta * (h[3] - h[1]);
     return HTSVD_OK;
 }
@@ -1063,6 +1076,13 @@ int32_t htsvd_internal_sampled_ranks(const uint8_t* d_img, int32_t H, int32_t W,
     if (launch_group_rank(d_img, g, (const int32_t*)idx2, n, (int32_t*)ranks, nullptr) != cudaSuccess) return -1;
     if (cudaMemcpy(h_ranks, ranks, sizeof(int32_t) * n, cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
     return n;
+}
+
+htsvd_status htsvd_internal_wait_limit(int64_t ns, cudaStream_t s) {
+    Workspace* w = workspace_for(s);
+    if (!w) return HTSVD_ERR_OOM;
+    w->wait_ns = ns < 0 ? kWaitLimitNs : (unsigned long long)ns;
+    return HTSVD_OK;
 }
 
 int32_t htsvd_internal_filter_tile(int32_t H, int32_t W, int32_t C, const htsvd_params* p) {
@@ -1143,6 +1163,12 @@ htsvd_status htsvd_denoise_batch(const htsvd_image* imgs, int32_t n, const htsvd
     Workspace* w = workspace_for(s);
     if (!w) return HTSVD_ERR_OOM;
     const int lanes = std::min(n, kBatchLanes);
+    htsvd_status late = take_timeout(w);     // of an earlier call, on any lane (each reported once, together)
+    for (int l = 0; l < kBatchLanes; ++l) {
+        Workspace* lw = w->lane[l] ? workspace_for(w->lane[l]) : nullptr;
+        if (lw && take_timeout(lw) != HTSVD_OK) late = HTSVD_ERR_TIMEOUT;
+    }
+    ST(late);
     if (!w->ev_batch) CK(cudaEventCreateWithFlags(&w->ev_batch, cudaEventDisableTiming));
     for (int l = 0; l < lanes; ++l) {
         if (!w->lane[l]) CK(cudaStreamCreateWithFlags(&w->lane[l], cudaStreamNonBlocking));
@@ -1151,6 +1177,7 @@ htsvd_status htsvd_denoise_batch(const htsvd_image* imgs, int32_t n, const htsvd
         if (!lw) return HTSVD_ERR_OOM;
         lw->plane_cap = kPlaneBytes / kBatchLanes;
         lw->share = lanes;
+        lw->wait_ns = w->wait_ns;
     }
     // largest images first, each to the lane with the least work so far (a lane's workspace then grows once)
     std::vector<int> order(n);
@@ -1362,6 +1389,7 @@ htsvd_status htsvd_sure(const float* d_y, int32_t H, int32_t W, int32_t C, doubl
     std::vector<double> h(4 * (size_t)n_tau);
     CK(cudaMemcpyAsync(h.data(), terms, sizeof(double) * 4 * n_tau, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
+    ST(take_timeout(w));
     for (int i = 0; i < n_tau; ++i) {
         const double* t = &h[4 * (size_t)i];
         const double div = fd ? (t[3] - t[1]) / eps : t[1];
@@ -1450,7 +1478,7 @@ htsvd_status htsvd_denoise_cube(const uint8_t* d_cube, int32_t H, int32_t W, int
       CK(launch_basis((const unsigned long long*)mom, N, (double*)p64, (float*)p32, s, (double*)gap)); }
     if (p && p->d_basis_out)
         CK(cudaMemcpyAsync(p->d_basis_out, p64, sizeof(double) * 2 * 2 * N * PS2, cudaMemcpyDeviceToDevice, s));
-    if (r.strict_basis) ST(check_basis_gap((const double*)gap, N, p, s));
+    if (r.strict_basis) ST(check_basis_gap(w, (const double*)gap, N, p, s));
     if (p && p->h_sigma_out) *p->h_sigma_out = sigma;
     const double tau = r.tau_mult * sigma;
     CubeArgs a{};

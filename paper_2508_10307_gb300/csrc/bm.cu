@@ -675,7 +675,8 @@ bool bt_plan(const BMArgs& a, BtPlan& p) {
 }
 
 template <int NPL, bool GCP>
-cudaError_t launch_bt(const BMArgs& a, const BtPlan& p, void* scratch, int* timeout, cudaStream_t s) {
+cudaError_t launch_bt(const BMArgs& a, const BtPlan& p, void* scratch, int* timeout, unsigned long long wait_ns,
+                      cudaStream_t s) {
     const Geo& g = a.g;
     BtArgs A{};
     A.b = a;
@@ -689,6 +690,7 @@ cudaError_t launch_bt(const BMArgs& a, const BtPlan& p, void* scratch, int* time
     A.TX = p.TX;
     A.ib = p.ib;
     A.timeout = timeout;
+    A.wait_ns = wait_ns;
     for (int f = 0; f < p.nfr; ++f) {
         BtPrep b{};
         b.img = a.nfr > 0 ? a.vid + (a.f0 + f) * a.fstride : a.img;
@@ -733,11 +735,13 @@ size_t bm_tc_scratch(const BMArgs& a, int share) {
     return ((p.planes + 255) & ~(size_t)255) + p.svv;
 }
 
-cudaError_t launch_block_match_tc(const BMArgs& a, void* scratch, int* timeout, cudaStream_t s) {
+cudaError_t launch_block_match_tc(const BMArgs& a, void* scratch, int* timeout, unsigned long long wait_ns,
+                                  cudaStream_t s) {
     BtPlan p;
     if (!bt_plan(a, p)) return cudaErrorInvalidValue;
-    if (p.npl == 2) return launch_bt<2, true>(a, p, scratch, timeout, s);
-    return p.npl == 3 ? launch_bt<3, false>(a, p, scratch, timeout, s) : launch_bt<1, false>(a, p, scratch, timeout, s);
+    if (p.npl == 2) return launch_bt<2, true>(a, p, scratch, timeout, wait_ns, s);
+    return p.npl == 3 ? launch_bt<3, false>(a, p, scratch, timeout, wait_ns, s)
+                      : launch_bt<1, false>(a, p, scratch, timeout, wait_ns, s);
 }
 
 }  // namespace htsvd

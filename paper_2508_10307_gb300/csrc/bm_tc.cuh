@@ -135,6 +135,7 @@ struct BtArgs {
     int TX;                  // references per tile row (32 or 16)
     int ib;                  // index bits of a key
     int* timeout;            // set (host memory) if a wait for the tensor cores runs out
+    unsigned long long wait_ns;   // limit of such a wait
 };
 
 __device__ __forceinline__ void bt_tmem_ld16(uint32_t taddr, float (&v)[16]) {
@@ -340,6 +341,7 @@ __global__ void __launch_bounds__(BT_THREADS, 2) block_match_tc_kernel(const __g
     const uint32_t LBO_B = (uint32_t)A.XP * 16u;
 
     uint32_t it = 0;                                  // rows of candidates done (accumulator it & 1)
+    uint32_t issued = 0;                              // the issuing lane: rows whose MMAs are committed
     bool ok = true;
     for (int fs = 0; fs < nfr && ok; ++fs) {
         const __half* fp = A.planes + fs * A.fstride_p;
@@ -378,7 +380,8 @@ __global__ void __launch_bounds__(BT_THREADS, 2) block_match_tc_kernel(const __g
                 if (lane == 0) {
                     for (int j = 0; j < rows; ++j) {
                         const uint32_t n = it + j, acc = n & 1;
-                        if (n >= 2 && !mbar_wait_or_abort(smem_u32(&bars[2 + acc]), ((n >> 1) & 1) ^ 1, abort_word)) break;
+                        if (n >= 2 && !mbar_wait_or_abort(smem_u32(&bars[2 + acc]), ((n >> 1) & 1) ^ 1, abort_word, A.wait_ns))
+                            break;
                         tc_fence_after();
                         uint32_t on = 0;
 #pragma unroll
@@ -390,6 +393,7 @@ __global__ void __launch_bounds__(BT_THREADS, 2) block_match_tc_kernel(const __g
                             on = 1;
                         }
                         mma_commit(smem_u32(&bars[acc]));
+                        issued = n + 1;
                     }
                 }
                 __syncwarp();
@@ -397,7 +401,7 @@ __global__ void __launch_bounds__(BT_THREADS, 2) block_match_tc_kernel(const __g
                 // ---- the candidates of this warp's references
                 for (int j = 0; j < rows; ++j) {
                     const uint32_t n = it + j, acc = n & 1;
-                    const bool got = mbar_wait_or_abort(smem_u32(&bars[acc]), (n >> 1) & 1, abort_word);
+                    const bool got = mbar_wait_or_abort(smem_u32(&bars[acc]), (n >> 1) & 1, abort_word, A.wait_ns);
                     if (__any_sync(FULL, !got)) break;
                     tc_fence_after();
                     const int wy = yb + j - wy0;
@@ -438,12 +442,14 @@ __global__ void __launch_bounds__(BT_THREADS, 2) block_match_tc_kernel(const __g
             if (*abort_word) ok = false;
         }
     }
-    if (!ok && tid == 0) {
-        // a wait ran out: report it, and let the MMAs issued last finish (bounded) before the tensor memory
-        // is released; the groups below then hold what was found
-        *A.timeout = 1;
-        mbar_wait_bounded(smem_u32(&bars[it & 1]), (it >> 1) & 1);
-        mbar_wait_bounded(smem_u32(&bars[(it + 1) & 1]), ((it + 1) >> 1) & 1);
+    if (!ok) {
+        // A wait ran out: report it, and let the MMAs in flight finish (bounded) before the tensor memory is
+        // released. The last commit covers all of them, and its barrier is at most that one phase behind: row
+        // issued - 1 was issued after row issued - 3 of the same accumulator had been read. The groups below then
+        // hold what was found, and the reference itself for the rest.
+        if (tid == 0) *A.timeout = 1;
+        if (warp == 4 && lane == 0 && issued > 0)
+            mbar_wait_bounded(smem_u32(&bars[(issued - 1) & 1]), ((issued - 1) >> 1) & 1);
     }
     if (warp < 4) {
         while (__any_sync(FULL, ptr != col)) bt_flush(list, ptr, thr, col, g.K, ib, srr);
@@ -452,6 +458,7 @@ __global__ void __launch_bounds__(BT_THREADS, 2) block_match_tc_kernel(const __g
         const uint32_t imask = mul - 1u;
         const int nw = g.wny * g.wnx;
         const int fo = a.nfr > 0 ? a.f0 * g.H * g.W : 0;
+        const int home = fo + fsref * g.H * g.W + ry * g.W + rx, gi = iy * g.nrx + ix;
         bool past = false, enough = true;
         __syncwarp();
 #pragma unroll
@@ -462,11 +469,10 @@ __global__ void __launch_bounds__(BT_THREADS, 2) block_match_tc_kernel(const __g
             const int w = (int)(k & imask);
             const int fs = w / nw, wr = w - fs * nw;
             const int dy = wr / g.wnx, dx = wr - dy * g.wnx;
-            buf[i * 33 + lane] = (uint32_t)(fo + fs * g.H * g.W + (wy0 + dy) * g.W + wx0 + dx);
+            buf[i * 33 + lane] = k != ~0u ? (uint32_t)(fo + fs * g.H * g.W + (wy0 + dy) * g.W + wx0 + dx) : (uint32_t)home;
         }
         __syncwarp();
         const unsigned wide = __ballot_sync(FULL, mine && !enough), valid = __ballot_sync(FULL, mine);
-        const int home = fo + fsref * g.H * g.W + ry * g.W + rx, gi = iy * g.nrx + ix;
         for (int l = 0; l < 32; ++l) {
             if (!((valid >> l) & 1u)) continue;
             const int h = __shfl_sync(FULL, home, l), gl = __shfl_sync(FULL, gi, l);
