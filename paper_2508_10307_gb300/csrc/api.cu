@@ -174,6 +174,8 @@ struct Workspace {
     cudaStream_t lane[kBatchLanes] = {};
     cudaEvent_t ev_lane[kBatchLanes] = {};
     cudaEvent_t ev_batch = nullptr;
+    std::mutex batch_mu;                  // held while a batch is put on the lanes: host threads that share a stream
+                                          // (every thread's default one, say) take turns
 };
 
 std::mutex g_mu;
@@ -1163,6 +1165,7 @@ htsvd_status htsvd_denoise_batch(const htsvd_image* imgs, int32_t n, const htsvd
     Workspace* w = workspace_for(s);
     if (!w) return HTSVD_ERR_OOM;
     const int lanes = std::min(n, kBatchLanes);
+    std::lock_guard<std::mutex> lk(w->batch_mu);
     htsvd_status late = take_timeout(w);     // of an earlier call, on any lane (each reported once, together)
     for (int l = 0; l < kBatchLanes; ++l) {
         Workspace* lw = w->lane[l] ? workspace_for(w->lane[l]) : nullptr;
