@@ -51,6 +51,11 @@ int32_t htsvd_internal_sampled_ranks(const uint8_t* d_img, int32_t H, int32_t W,
  * library's own, about two seconds; 0: every wait counts as run out at once). Host only. */
 htsvd_status htsvd_internal_wait_limit(int64_t ns, cudaStream_t stream);
 
+/* Limits of the workspace of stream: plane_bytes, the most it takes for projection planes (negative: the library's
+ * own), and room, the bytes that the device is taken to have free for buffers a call can do without (negative: it
+ * is asked). Returns the device allocations that the workspace has made so far, or -1. Host only. */
+int64_t htsvd_internal_scratch_limits(int64_t plane_bytes, int64_t room, cudaStream_t stream);
+
 /* Tile edge (references per tile side) that the forward filter of htsvd_denoise takes for an H x W x C
  * uint8 image with parameters p on the current device (it follows the SM count), or -1 on bad
  * arguments. Host only; launches nothing. */

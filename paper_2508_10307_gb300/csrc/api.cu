@@ -169,6 +169,8 @@ struct Workspace {
     int* timeout = nullptr;               // pinned word a kernel sets when one of its waits runs out
     unsigned long long wait_ns = kWaitLimitNs;   // limit of such a wait
     size_t plane_cap = kPlaneBytes;       // most it may hold as projection planes
+    int64_t room = -1;                    // bytes ws_try takes the device to have free (negative: it asks)
+    int64_t allocations = 0;              // device allocations made so far
     int share = 1;                        // images that run side by side (the lanes of a batch)
     // htsvd_denoise_batch: the streams its images run on (each with a workspace of its own), and their events
     cudaStream_t lane[kBatchLanes] = {};
@@ -204,6 +206,7 @@ htsvd_status ws_get(Workspace* w, int slot, size_t bytes, void** out) {
             w->cap[slot] = 0;
         }
         size_t b = bytes + bytes / 8;
+        ++w->allocations;
         if (cudaMalloc(&w->buf[slot], b) != cudaSuccess) {
             cudaGetLastError();
             return HTSVD_ERR_OOM;
@@ -212,6 +215,26 @@ htsvd_status ws_get(Workspace* w, int slot, size_t bytes, void** out) {
     }
     *out = w->buf[slot];
     return HTSVD_OK;
+}
+
+// A buffer that the call can do without (it then takes smaller bands, or the kernel that needs none): OOM, with
+// the present buffer kept, where the device has no room for a larger one. Without that look first, a call on a
+// nearly full device would free what served the last one, and allocate it again, each time: device
+// synchronisations that a call must not make.
+htsvd_status ws_try(Workspace* w, int slot, size_t bytes, void** out) {
+    const size_t held = w->cap[slot];
+    if (held < bytes) {
+        size_t free_ = 0, total = 0;
+        if (w->room >= 0) free_ = (size_t)w->room;
+        else if (cudaMemGetInfo(&free_, &total) != cudaSuccess) {
+            cudaGetLastError();
+            return HTSVD_ERR_OOM;
+        }
+        if (free_ + held < bytes + bytes / 8) return HTSVD_ERR_OOM;
+    }
+    const htsvd_status st = ws_get(w, slot, bytes, out);
+    if (w->room >= 0) w->room = std::max<int64_t>(0, w->room + (int64_t)held - (int64_t)w->cap[slot]);
+    return st;
 }
 
 // TIMEOUT, once, where a kernel of the workspace's stream that has run by now gave up a wait.
@@ -350,7 +373,7 @@ htsvd_status run_block_match(Workspace* w, const uint8_t* q, const Geo& g, const
     a.idx = idx;
     if (const size_t tcb = bm_tc_scratch(a, w->share)) {
         void* scratch;
-        if (ws_get(w, S_BMTC, tcb, &scratch) == HTSVD_OK) {
+        if (ws_try(w, S_BMTC, tcb, &scratch) == HTSVD_OK) {
             if (!w->timeout) {
                 CK(cudaMallocHost(&w->timeout, sizeof(int)));
                 *w->timeout = 0;
@@ -528,12 +551,12 @@ htsvd_status plane_bands(Workspace* w, const Geo& g, int TR, int nty, int ntiles
         const size_t bytes = (size_t)most * row * PS2 * g.C * sizeof(float);
         if ((bytes > w->plane_cap || most > 65535) && per > 1) continue;
         void *c, *n, *k;
-        const htsvd_status st = ws_get(w, S_PLANE, bytes, &c);
+        htsvd_status st = ws_try(w, S_PLANE, bytes, &c);
+        if (st == HTSVD_OK) st = ws_try(w, S_PNRM, (size_t)most * row * sizeof(float), &n);
         if (st != HTSVD_OK) {
             if (per > 1) continue;
             return st;
         }
-        ST(ws_get(w, S_PNRM, (size_t)most * row * sizeof(float), &n));
         ST(ws_get(w, S_CTR, sizeof(int) * (2 + (size_t)ntiles + 3), &k));
         P.coef = (float*)c;
         P.pn = (float*)n;
@@ -631,12 +654,10 @@ htsvd_status run_forward_filter(Workspace* w, const void* img, int is_float, con
     int per = t.nty, grid = 0;
     bool planes = !cc && g.ngroups() >= kPlaneGroups;
     if (planes) {
-        htsvd_status st = plane_bands(w, g, t.TR, t.nty, t.nty * t.ntx, vc ? vc->nfr : 1, per, P);
-        if (st == HTSVD_OK) {
-            ga.nty_band = per;
-            grid = group_grid(ga);
-            st = ws_get(w, S_SPILL, sizeof(float) * group_spill_floats(ga, grid), &spill);
-        }
+        ga.nty_band = per;
+        grid = group_grid(ga);
+        htsvd_status st = ws_try(w, S_SPILL, sizeof(float) * group_spill_floats(ga, grid), &spill);
+        if (st == HTSVD_OK) st = plane_bands(w, g, t.TR, t.nty, t.nty * t.ntx, vc ? vc->nfr : 1, per, P);
         if (st != HTSVD_OK && st != HTSVD_ERR_OOM) return st;
         planes = st == HTSVD_OK;
     }
@@ -917,12 +938,10 @@ htsvd_status vjp_core(Workspace* w, const float* d_x, const Geo& g, const Resolv
     a.grad_w = d_grad_w;
     Planes P, R;
     int per = t.nty, grid = 0;
-    htsvd_status st = plane_bands(w, g, t.TR, t.nty, t.nty * t.ntx, 2, per, P);       // (two images: as two frames)
-    if (st == HTSVD_OK) {
-        ga.nty_band = per;
-        grid = group_grid(ga);
-        st = ws_get(w, S_SPILL, sizeof(float) * group_spill_floats(ga, grid), &spill);
-    }
+    ga.nty_band = per;
+    grid = group_grid(ga);
+    htsvd_status st = ws_try(w, S_SPILL, sizeof(float) * group_spill_floats(ga, grid), &spill);
+    if (st == HTSVD_OK) st = plane_bands(w, g, t.TR, t.nty, t.nty * t.ntx, 2, per, P);   // (two images: as two frames)
     if (st != HTSVD_OK && st != HTSVD_ERR_OOM) return st;
     if (st != HTSVD_OK) {                          // no room for the planes: the tile kernel alone
         ProfScope ps_("adjoint", s);
@@ -1087,6 +1106,14 @@ htsvd_status htsvd_internal_wait_limit(int64_t ns, cudaStream_t s) {
     return HTSVD_OK;
 }
 
+int64_t htsvd_internal_scratch_limits(int64_t plane_bytes, int64_t room, cudaStream_t s) {
+    Workspace* w = workspace_for(s);
+    if (!w) return -1;
+    w->plane_cap = plane_bytes < 0 ? kPlaneBytes : (size_t)plane_bytes;
+    w->room = room;
+    return w->allocations;
+}
+
 int32_t htsvd_internal_filter_tile(int32_t H, int32_t W, int32_t C, const htsvd_params* p) {
     Resolved r;
     if (resolve(p, C, r) != HTSVD_OK || check_image(H, W, C, r) != HTSVD_OK) return -1;
@@ -1178,7 +1205,8 @@ htsvd_status htsvd_denoise_batch(const htsvd_image* imgs, int32_t n, const htsvd
         if (!w->ev_lane[l]) CK(cudaEventCreateWithFlags(&w->ev_lane[l], cudaEventDisableTiming));
         Workspace* lw = workspace_for(w->lane[l]);
         if (!lw) return HTSVD_ERR_OOM;
-        lw->plane_cap = kPlaneBytes / kBatchLanes;
+        lw->plane_cap = w->plane_cap / kBatchLanes;
+        lw->room = w->room;
         lw->share = lanes;
         lw->wait_ns = w->wait_ns;
     }
@@ -1532,9 +1560,9 @@ htsvd_status run_volume_filter(Workspace* w, const VolFilterArgs& a, int64_t ng,
         htsvd_status st = HTSVD_ERR_OOM;
         if (most <= 65535 && pos * 64 * sizeof(float) <= w->plane_cap &&
             (int64_t)per * volume_tiles_plane(g) < ((int64_t)1 << 31)) {
-            st = ws_get(w, S_PLANE, pos * 64 * sizeof(float), &coef);
-            if (st == HTSVD_OK) st = ws_get(w, S_PNRM, pos * sizeof(float), &pn);
-            if (st == HTSVD_OK) st = ws_get(w, S_SPILL, volume_group_rec_bytes(g, per), &rec);
+            st = ws_try(w, S_PLANE, pos * 64 * sizeof(float), &coef);
+            if (st == HTSVD_OK) st = ws_try(w, S_PNRM, pos * sizeof(float), &pn);
+            if (st == HTSVD_OK) st = ws_try(w, S_SPILL, volume_group_rec_bytes(g, per), &rec);
         }
         if (st == HTSVD_OK) break;
         if (st != HTSVD_ERR_OOM) return st;
