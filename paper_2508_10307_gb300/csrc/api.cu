@@ -535,6 +535,7 @@ struct Planes {
     const int* dense = nullptr;  // its verdict, where it is asked
     long long stride = 0;        // positions per frame
     int y0 = 0, y1 = 0;          // position rows held
+    size_t most = 0;             // positions of the largest band, per frame
 };
 
 // Tile rows per band: as many as fit the workspace's share; where the device cannot give that much, halved until
@@ -562,6 +563,7 @@ htsvd_status plane_bands(Workspace* w, const Geo& g, int TR, int nty, int ntiles
         P.pn = (float*)n;
         P.counter = (int*)k;
         P.sample = P.counter + 2 + ntiles;
+        P.most = (size_t)most * g.npx;
         return HTSVD_OK;
     }
 }
@@ -942,6 +944,7 @@ htsvd_status vjp_core(Workspace* w, const float* d_x, const Geo& g, const Resolv
     grid = group_grid(ga);
     htsvd_status st = ws_try(w, S_SPILL, sizeof(float) * group_spill_floats(ga, grid), &spill);
     if (st == HTSVD_OK) st = plane_bands(w, g, t.TR, t.nty, t.nty * t.ntx, 2, per, P);   // (two images: as two frames)
+    if (st == HTSVD_OK) st = ws_try(w, S_DOT, sizeof(float) * P.most, &dot);
     if (st != HTSVD_OK && st != HTSVD_ERR_OOM) return st;
     if (st != HTSVD_OK) {                          // no room for the planes: the tile kernel alone
         ProfScope ps_("adjoint", s);
@@ -960,7 +963,6 @@ htsvd_status vjp_core(Workspace* w, const float* d_x, const Geo& g, const Resolv
         ST(fill_planes(d_x, 1, g, b32, y0, y1, nullptr, P, s));
         ST(fill_planes(rimg, 1, g, b32, y0, y1, nullptr, R, s));
         rc = R.coef;
-        ST(ws_get(w, S_DOT, sizeof(float) * pos, &dot));
         { ProfScope ps_("patch_dot", s); CK(launch_patch_dot((const float*)rimg, d_out, g.H, g.W, C, y0, y1 - y0, (float*)dot, s)); }
         ga.coef = P.coef;
         ga.pn = P.pn;

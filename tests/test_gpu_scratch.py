@@ -149,3 +149,32 @@ def test_short_of_memory_allocates_once():
         assert torch.equal(H.denoise(x, 20.0, dict()), ref)
     assert H.load_library().htsvd_internal_scratch_limits(-1, -1, s) == made
     assert torch.equal(first, ref)
+
+
+def test_gradients_at_every_amount_of_room():
+    """Whichever buffer of the plane path is the one that finds no room (spilled rows, planes, patch products), the
+    call runs without planes."""
+    x = torch.from_numpy(synth.add_gaussian_float(synth.clean_image(125, 121, 1, 7), 20.0, 7)).cuda()
+    prm = dict(stride=2, window=9, K=16)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    out, info = H.denoise_f32(x, 20.0, prm, return_info=True)
+    g = torch.randn(x.shape, device="cuda", generator=gen)
+    want = H.denoise_vjp(x, 20.0, info["idx"], None, out, g, prm)
+
+    def at(room):
+        torch.cuda.synchronize()
+        H.load_library().htsvd_release_workspace()
+        _limits(room=room)
+        (gx, gw), n = _counted(lambda: H.denoise_vjp(x, 20.0, info["idx"], None, out, g, prm))
+        assert (gx - want[0]).abs().max() <= 1e-4 * want[0].abs().max()
+        assert (gw - want[1]).abs().max() <= 1e-4 * max(1.0, want[1].abs().max().item())
+        return "planes" in n
+
+    lo, hi = 0, 1 << 30
+    assert not at(lo) and at(hi)
+    while hi - lo > 1 << 12:                     # the least room at which the planes are used, to 4 KB
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if at(mid) else (mid, hi)
+    for k in range(12):                          # (the patch products take 54 KB, last of all)
+        at(lo - (k << 13))
