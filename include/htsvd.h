@@ -20,7 +20,12 @@
  *    candidates of its search window by (SSD, linear index) ascending.
  *  - Calls are asynchronous on `stream` except where a host result is
  *    returned (documented per call). The library owns a workspace cached per
- *    (device, stream); it grows with cudaMalloc on first use at a size. Calls
+ *    (device, stream); it grows with cudaMalloc on first use at a size and is
+ *    held until htsvd_release_workspace. Most of it are projection planes, at
+ *    most 8 GiB and an eighth (a 3840 x 2160 RGB image: 7 GiB; a batch: the
+ *    same over its streams) where the device has room for them: calls run
+ *    without them too, and give them back before they fail for want of memory.
+ *    Calls
  *    on different streams may run from different host threads at once; calls
  *    on one stream share its workspace, so host threads that issue them must
  *    serialise them (stream order then keeps their kernels apart).

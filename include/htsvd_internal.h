@@ -56,6 +56,9 @@ htsvd_status htsvd_internal_wait_limit(int64_t ns, cudaStream_t stream);
  * is asked). Returns the device allocations that the workspace has made so far, or -1. Host only. */
 int64_t htsvd_internal_scratch_limits(int64_t plane_bytes, int64_t room, cudaStream_t stream);
 
+/* The next n device allocations of the workspace of stream fail, as on a full device. Host only. */
+htsvd_status htsvd_internal_fail_allocations(int32_t n, cudaStream_t stream);
+
 /* Tile edge (references per tile side) that the forward filter of htsvd_denoise takes for an H x W x C
  * uint8 image with parameters p on the current device (it follows the SM count), or -1 on bad
  * arguments. Host only; launches nothing. */

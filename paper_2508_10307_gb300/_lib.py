@@ -105,6 +105,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.htsvd_internal_wait_limit.argtypes = [ctypes.c_int64, vp]
     lib.htsvd_internal_scratch_limits.argtypes = [ctypes.c_int64, ctypes.c_int64, vp]
     lib.htsvd_internal_scratch_limits.restype = ctypes.c_int64
+    lib.htsvd_internal_fail_allocations.argtypes = [i32, vp]
     lib.htsvd_internal_filter_tile.argtypes = [i32, i32, i32, P]
     lib.htsvd_internal_filter_tile.restype = i32
     lib.htsvd_internal_noalloc_bytes.argtypes = [i32, i32, i32, P]

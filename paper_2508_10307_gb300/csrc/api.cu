@@ -171,6 +171,7 @@ struct Workspace {
     size_t plane_cap = kPlaneBytes;       // most it may hold as projection planes
     int64_t room = -1;                    // bytes ws_try takes the device to have free (negative: it asks)
     int64_t allocations = 0;              // device allocations made so far
+    int fail_next = 0;                    // as many coming allocations fail (tests)
     int share = 1;                        // images that run side by side (the lanes of a batch)
     // htsvd_denoise_batch: the streams its images run on (each with a workspace of its own), and their events
     cudaStream_t lane[kBatchLanes] = {};
@@ -197,7 +198,28 @@ Workspace* workspace_for(cudaStream_t s) {
     return w;
 }
 
-htsvd_status ws_get(Workspace* w, int slot, size_t bytes, void** out) {
+// Frees what the workspace (and those of its lanes, unless a batch is being put on them) holds of the buffers a
+// call can do without (ws_try). No call takes a buffer that it cannot do without after one of these.
+void ws_give_back(Workspace* w) {
+    constexpr int slots[] = {S_PLANE, S_PNRM, S_SPILL, S_DOT, S_BMTC};
+    auto drop = [&](Workspace* v) {
+        for (int k : slots)
+            if (v->buf[k]) {
+                cudaFree(v->buf[k]);           // (waits for the device: nothing in flight uses it)
+                v->buf[k] = nullptr;
+                v->cap[k] = 0;
+            }
+    };
+    drop(w);
+    std::unique_lock<std::mutex> lanes(w->batch_mu, std::try_to_lock);
+    if (!lanes.owns_lock()) return;
+    std::lock_guard<std::mutex> lk(g_mu);
+    for (Workspace* v : g_ws)
+        for (cudaStream_t l : w->lane)
+            if (l && v->device == w->device && v->stream == l) drop(v);
+}
+
+htsvd_status ws_get(Workspace* w, int slot, size_t bytes, void** out, bool optional = false) {
     if (bytes == 0) bytes = 16;
     if (w->cap[slot] < bytes) {
         if (w->buf[slot]) {
@@ -206,10 +228,20 @@ htsvd_status ws_get(Workspace* w, int slot, size_t bytes, void** out) {
             w->cap[slot] = 0;
         }
         size_t b = bytes + bytes / 8;
-        ++w->allocations;
-        if (cudaMalloc(&w->buf[slot], b) != cudaSuccess) {
+        auto get = [&] {
+            ++w->allocations;
+            if (w->fail_next > 0) {
+                --w->fail_next;
+                return false;
+            }
+            if (cudaMalloc(&w->buf[slot], b) == cudaSuccess) return true;
             cudaGetLastError();
-            return HTSVD_ERR_OOM;
+            return false;
+        };
+        if (!get()) {
+            if (optional) return HTSVD_ERR_OOM;
+            ws_give_back(w);
+            if (!get()) return HTSVD_ERR_OOM;
         }
         w->cap[slot] = b;
     }
@@ -232,7 +264,7 @@ htsvd_status ws_try(Workspace* w, int slot, size_t bytes, void** out) {
         }
         if (free_ + held < bytes + bytes / 8) return HTSVD_ERR_OOM;
     }
-    const htsvd_status st = ws_get(w, slot, bytes, out);
+    const htsvd_status st = ws_get(w, slot, bytes, out, true);
     if (w->room >= 0) w->room = std::max<int64_t>(0, w->room + (int64_t)held - (int64_t)w->cap[slot]);
     return st;
 }
@@ -554,11 +586,11 @@ htsvd_status plane_bands(Workspace* w, const Geo& g, int TR, int nty, int ntiles
         void *c, *n, *k;
         htsvd_status st = ws_try(w, S_PLANE, bytes, &c);
         if (st == HTSVD_OK) st = ws_try(w, S_PNRM, (size_t)most * row * sizeof(float), &n);
+        if (st == HTSVD_OK) st = ws_try(w, S_CTR, sizeof(int) * (2 + (size_t)ntiles + 3), &k);
         if (st != HTSVD_OK) {
             if (per > 1) continue;
             return st;
         }
-        ST(ws_get(w, S_CTR, sizeof(int) * (2 + (size_t)ntiles + 3), &k));
         P.coef = (float*)c;
         P.pn = (float*)n;
         P.counter = (int*)k;
@@ -1114,6 +1146,13 @@ int64_t htsvd_internal_scratch_limits(int64_t plane_bytes, int64_t room, cudaStr
     w->plane_cap = plane_bytes < 0 ? kPlaneBytes : (size_t)plane_bytes;
     w->room = room;
     return w->allocations;
+}
+
+htsvd_status htsvd_internal_fail_allocations(int32_t n, cudaStream_t s) {
+    Workspace* w = workspace_for(s);
+    if (!w) return HTSVD_ERR_OOM;
+    w->fail_next = n;
+    return HTSVD_OK;
 }
 
 int32_t htsvd_internal_filter_tile(int32_t H, int32_t W, int32_t C, const htsvd_params* p) {

@@ -178,3 +178,24 @@ def test_gradients_at_every_amount_of_room():
         lo, hi = (lo, mid) if at(mid) else (mid, hi)
     for k in range(12):                          # (the patch products take 54 KB, last of all)
         at(lo - (k << 13))
+
+
+@pytest.mark.parametrize("batch", [False, True])
+def test_planes_are_given_back_before_a_call_fails(batch):
+    """A full device: an allocation the call cannot do without fails once, the buffers it can do without are
+    freed (the caller's own or those of an earlier batch), and the second attempt succeeds."""
+    x = torch.from_numpy(synth.add_gaussian(synth.clean_image(124, 131, 3, 3), 20.0, 3)).cuda()
+    y = torch.from_numpy(synth.add_gaussian(synth.clean_image(224, 231, 3, 3), 20.0, 3)).cuda()
+    prm = dict(stride=2, window=9, K=16)
+    want = H.denoise(y, 20.0, prm)
+    torch.cuda.synchronize()
+    H.load_library().htsvd_release_workspace()
+    H.denoise_batch([x, x], [20.0, 20.0], prm) if batch else H.denoise(x, 20.0, prm)
+    torch.cuda.synchronize()
+    s = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert H.load_library().htsvd_internal_fail_allocations(1, s) == 0
+    assert torch.equal(H.denoise(y, 20.0, prm), want)
+    H.load_library().htsvd_internal_fail_allocations(2, s)
+    with pytest.raises(_lib.HtsvdError, match="OOM"):
+        H.denoise(torch.cat([y, y], 1), 20.0, prm)
+    assert torch.equal(H.denoise(y, 20.0, prm), want)
