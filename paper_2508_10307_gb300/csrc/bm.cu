@@ -664,6 +664,9 @@ bool bt_plan(const BMArgs& a, BtPlan& p) {
     }
     const int64_t nc = (int64_t)p.nfr * g.wny * g.wnx;
     if (nc > 4096) return false;
+    // the rows of blocks of both kernels within a grid's 65,535 (images of a million rows)
+    const int TY = BT_REFS / p.TX;
+    if ((g.H + BP_Y - 1) / BP_Y > 65535 || (g.nry + TY - 1) / TY > 65535) return false;
     p.ib = 8;                // at least 8: the exponent of SSD + 2^23 then falls out of the key
     while (((int64_t)1 << p.ib) < nc) ++p.ib;
     p.pitch = (g.W + 39) & ~7;

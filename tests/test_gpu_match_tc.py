@@ -54,3 +54,11 @@ def test_ties_and_extreme_values(kind):
         noisy[:, n // 2:] = (255, 211, 255)
         noisy[::37, ::5] = rng.integers(0, 256, noisy[::37, ::5].shape, dtype=np.uint8)
     _check(np.ascontiguousarray(noisy), dict(stride=3, window=31, K=32), rows=(30, 60))
+
+
+def test_image_of_a_million_rows():
+    """More rows than a grid of the tensor-core form reaches: the other form groups it, as it did before."""
+    h, w = 1_050_000, 16
+    rng = np.random.default_rng(11)
+    noisy = (np.arange(h)[:, None, None] // 64 % 200 + rng.integers(0, 40, (h, w, 1))).astype(np.uint8)
+    _check(noisy, dict(stride=16, window=9, K=8), rows=(40_000, 65_000))
