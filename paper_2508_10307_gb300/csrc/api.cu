@@ -1219,8 +1219,11 @@ htsvd_status htsvd_denoise_batch(const htsvd_image* imgs, int32_t n, const htsvd
     q.d_coef_out = nullptr;
     q.strict_basis = 0;
     q.h_basis_gap_out = nullptr;
+    const int edge = std::max(q.tile, 0);    // (a batch takes any edge: below 1 automatic, else as large as fits)
+    q.tile = 0;
     Resolved r;
     ST(resolve(&q, imgs[0].C, r));
+    r.tile = edge;
     for (int i = 0; i < n; ++i) {
         const htsvd_image& im = imgs[i];
         if (!im.d_in || !im.d_out || !(im.sigma >= 0) || im.C != imgs[0].C || (im.C != 1 && im.C != 3) || im.H < PS ||

@@ -81,3 +81,11 @@ def test_batch_of_uneven_images_equals_single_calls(n):
     sig = [10.0 + 2 * i for i in range(n)]
     for x, s, o in zip(xs, sig, H.denoise_batch(xs, sig, prm)):
         assert max_abs(o.cpu().numpy(), H.denoise(x, s, prm).cpu().numpy()) <= PIX_TOL
+
+
+@pytest.mark.parametrize("tile", [-1, 17, 20])
+def test_batch_takes_any_tile_edge(tile):
+    x = torch.from_numpy(synth.add_gaussian(synth.clean_image(117, 122, 1, 5), 20.0, 5)).cuda()
+    prm = dict(stride=1, window=5, K=8)
+    out, = H.denoise_batch([x], [20.0], dict(prm, tile=tile))
+    assert max_abs(out.cpu().numpy(), H.denoise(x, 20.0, prm).cpu().numpy()) <= PIX_TOL
