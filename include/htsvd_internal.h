@@ -83,6 +83,9 @@ htsvd_status htsvd_internal_project_simt(const uint8_t* d_img, int32_t H, int32_
  * layout of htsvd_params.d_basis_out. Returns the smallest relative eigen-gap of the slices 0..2. */
 double htsvd_internal_volume_bases(const unsigned long long* mom, double* b64);
 
+/* HOST: 1 if the filter of a D x H x W volume takes projection planes where there is room for them, else 0. */
+int32_t htsvd_internal_volume_planes(int32_t D, int32_t H, int32_t W, int32_t stride, int32_t window, int32_t K);
+
 /* DEVICE probe of an arithmetic pipe's issue rate on the current device: 2 CTAs of 512 threads per
  * SM, each thread running 8 independent chains of one instruction for 32 * iters steps (op 0: FP32
  * fused multiply-add, 1: 32-bit integer multiply-add, 2: 4-way byte dot product with accumulate).

@@ -1585,13 +1585,18 @@ namespace {
 // 173 / 165 at 1,331 references, 181 / 172 at 3,375, 174 / 184 at 6,859, 276 / 401 at 29,791.
 constexpr int64_t kVolPlaneGroups = 5000;
 
+// Whether a volume's filter takes projection planes (where the device has room for them).
+bool volume_takes_planes(const VolGeo& g) {
+    return (int64_t)g.nrz * g.nry * g.nrx >= kVolPlaneGroups && volume_group_fits(g);
+}
+
 // Filter of a volume: bands of tile planes over the projection planes that fit the workspace's share, or
 // volume_filter_kernel where they do not pay or the device has no room for them.
 htsvd_status run_volume_filter(Workspace* w, const VolFilterArgs& a, int64_t ng, cudaStream_t s) {
     const VolGeo& g = a.g;
     const int ntz = volume_tiles_z(g);
     void *coef, *pn, *rec;
-    bool planes = ng >= kVolPlaneGroups && volume_group_fits(g);
+    bool planes = volume_takes_planes(g);
     int per = ntz;
     while (planes) {
         int most = 0;
@@ -1647,6 +1652,10 @@ htsvd_status run_volume_filter(Workspace* w, const VolFilterArgs& a, int64_t ng,
 }
 
 }  // namespace
+
+int32_t htsvd_internal_volume_planes(int32_t D, int32_t H, int32_t W, int32_t stride, int32_t window, int32_t K) {
+    return volume_takes_planes(make_vol_geo(D, H, W, stride, window, K)) ? 1 : 0;
+}
 
 htsvd_status htsvd_denoise_volume(const uint8_t* d_vol, int32_t D, int32_t H, int32_t W, double sigma,
                                   const htsvd_params* p, float* d_out, int32_t* d_idx_out, cudaStream_t s) {

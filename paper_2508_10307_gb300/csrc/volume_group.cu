@@ -570,11 +570,12 @@ __global__ void __launch_bounds__(VG_THREADS, 2) volume_group_kernel(const __gri
     }
 }
 
+// Voxels of a tile's footprint, at most a million (in 64 bits: strides of a few hundred pass 2^31).
 int vol_nvox(const VolGeo& g) {
     const int ext[3] = {g.wnz, g.wny, g.wnx};
-    int n = 1;
-    for (int d = 0; d < 3; ++d) n *= (VT - 1) * g.s + ext[d] + VE - 1;
-    return n;
+    int64_t n = 1;
+    for (int d = 0; d < 3; ++d) n = std::min<int64_t>(n * ((int64_t)(VT - 1) * g.s + ext[d] + VE - 1), 1 << 20);
+    return (int)n;
 }
 
 template <int K>
