@@ -630,6 +630,11 @@ htsvd_status fill_planes(const void* img, int is_float, const Geo& g, const floa
 // call: RGB, K 32: 131 / 123 at 2,704 references, 172 / 182 at 4,225, 261 / 300 at 7,056; gray, K 32: 53 / 41
 // at 1,681, 79 / 81 at 2,704, 103 / 123 at 4,225.
 constexpr int kPlaneGroups = 3000;
+// CTAs of the group filter that must fit an SM: with one, its three warps lose to the tile kernel's eight. us of
+// planes and filter against the tile kernel, RGB, K 32: window 48, stride 5 (85 x 85 pixels a footprint, 6,720
+// references) 338 / 245, window 64, stride 4 (83 x 83, 31,146) 1,198 / 1,100; with two, window 48, stride 3
+// (76 x 76, 18,348 references) 439 / 608.
+constexpr int kGroupCtas = 2;
 
 // Filter + reduce for the forward pass.
 htsvd_status run_forward_filter(Workspace* w, const void* img, int is_float, const Geo& g, const Resolved& r,
@@ -690,7 +695,8 @@ htsvd_status run_forward_filter(Workspace* w, const void* img, int is_float, con
     if (planes) {
         ga.nty_band = per;
         grid = group_grid(ga);
-        htsvd_status st = ws_try(w, S_SPILL, sizeof(float) * group_spill_floats(ga, grid), &spill);
+        htsvd_status st = ga.per_sm < kGroupCtas ? HTSVD_ERR_OOM : HTSVD_OK;
+        if (st == HTSVD_OK) st = ws_try(w, S_SPILL, sizeof(float) * group_spill_floats(ga, grid), &spill);
         if (st == HTSVD_OK) st = plane_bands(w, g, t.TR, t.nty, t.nty * t.ntx, vc ? vc->nfr : 1, per, P);
         if (st != HTSVD_OK && st != HTSVD_ERR_OOM) return st;
         planes = st == HTSVD_OK;
@@ -974,11 +980,12 @@ htsvd_status vjp_core(Workspace* w, const float* d_x, const Geo& g, const Resolv
     int per = t.nty, grid = 0;
     ga.nty_band = per;
     grid = group_grid(ga);
-    htsvd_status st = ws_try(w, S_SPILL, sizeof(float) * group_spill_floats(ga, grid), &spill);
+    htsvd_status st = ga.per_sm < kGroupCtas ? HTSVD_ERR_OOM : HTSVD_OK;
+    if (st == HTSVD_OK) st = ws_try(w, S_SPILL, sizeof(float) * group_spill_floats(ga, grid), &spill);
     if (st == HTSVD_OK) st = plane_bands(w, g, t.TR, t.nty, t.nty * t.ntx, 2, per, P);   // (two images: as two frames)
     if (st == HTSVD_OK) st = ws_try(w, S_DOT, sizeof(float) * P.most, &dot);
     if (st != HTSVD_OK && st != HTSVD_ERR_OOM) return st;
-    if (st != HTSVD_OK) {                          // no room for the planes: the tile kernel alone
+    if (st != HTSVD_OK) {                          // no room for the planes or the CTAs: the tile kernel alone
         ProfScope ps_("adjoint", s);
         CK(launch_filter(a, s));
         per = t.nty + 1;

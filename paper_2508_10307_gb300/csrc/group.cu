@@ -298,13 +298,13 @@ int group_grid(GroupArgs& a) {
     const int rows = a.f.g.K * PS;                        // every row of every slot
     const int row_bytes = GR_WARPS * PS * a.f.g.C * 4;     // all warps
     const int fixed = layout_of(a, 0).total + 1024 + 64;
-    int per_sm = 1;
+    a.per_sm = 1;
     a.cap = std::min(rows, 8);
     for (int n = GR_CTAS; n >= 1; --n) {
         const int room = 228 * 1024 / n - fixed;
         const int cap = std::min(rows, room / row_bytes);
         if (cap >= std::min(rows, 16) || n == 1) {
-            per_sm = n;
+            a.per_sm = n;
             a.cap = std::max(cap, 0);
             break;
         }
@@ -314,7 +314,7 @@ int group_grid(GroupArgs& a) {
     // 860 / 816 / 762 / 764 / 763 at sigma 15 and 4.2, 1,483 / 1,489 / 1,479 / 1,781 / 1,860 at sigma 8 and 2.0. With
     // 8 patches or fewer a group has 64 rows at most and nothing is left.
     a.dense_rows = a.f.g.K <= 8 ? 1 << 20 : 30;
-    return std::min(a.nty_band * a.f.ntx, per_sm * device_sm_count());
+    return std::min(a.nty_band * a.f.ntx, a.per_sm * device_sm_count());
 }
 
 size_t group_spill_floats(const GroupArgs& a, int grid) {

@@ -149,6 +149,7 @@ struct GroupArgs {
     int py0;                 // image row of the planes' first position row
     int ty0, nty_band;
     int cap;                 // rows of kept coefficients a warp holds in shared memory
+    int per_sm;              // CTAs that share an SM
     float* spill;            // rows beyond cap, group_spill_floats(...) in all
     const float* rcoef;      // adjoint: planes of r
     const float* dot;        // adjoint: per position, <patch of r, patch of the output>
@@ -161,7 +162,7 @@ struct GroupArgs {
 // Sets st[2] where the sampled groups of the image keep more rows of coefficients than the group filter is the
 // faster one for (st: three zeroed words); FilterArgs as for the filter. K 16 or 32.
 cudaError_t launch_sample_rows(const FilterArgs& a, int* st, cudaStream_t s);
-// Fills a.cap and returns the grid (persistent CTAs) of a launch.
+// Fills a.cap and a.per_sm and returns the grid (persistent CTAs) of a launch.
 int group_grid(GroupArgs& a);
 size_t group_spill_floats(const GroupArgs& a, int grid);
 cudaError_t launch_group(const GroupArgs& a, int grid, cudaStream_t s);
