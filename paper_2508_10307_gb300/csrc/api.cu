@@ -707,10 +707,11 @@ htsvd_status run_forward_filter(Workspace* w, const void* img, int is_float, con
         return HTSVD_OK;
     }
     ga.spill = (float*)spill;
-    if (r.K > 8) {                             // (with fewer slots the group filter is the faster one at any threshold)
+    const int most = group_rows_limit(a);
+    if (most != kEveryRow) {
         ProfScope ps_("sample_rows", s);
         CK(cudaMemsetAsync(P.sample, 0, 3 * sizeof(int), s));
-        CK(launch_sample_rows(a, P.sample, s));
+        CK(launch_sample_rows(a, most, P.sample, s));
         P.dense = a.dense = P.sample + 2;
     }
     if (a.mask_out)

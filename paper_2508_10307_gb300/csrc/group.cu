@@ -49,15 +49,8 @@ GLayout layout_of(const GroupArgs& a, int cap) {
 // Rows of coefficients that the groups keep, from SR_GROUPS groups spread over the image: one CTA per group
 // projects its patches, takes the Haar transform of every coefficient across them and counts the (slot, basis
 // row) pairs with a coefficient above the threshold. The last CTA compares the mean with the rows up to which
-// the group filter is the faster one (see dense_mean). 15 us, most of it the latency of one group.
+// the group filter is the faster one (group_rows_limit). 15 us, most of it the latency of one group.
 constexpr int SR_GROUPS = 128;
-
-// Mean rows per group at which planes and group filter take as long as filter_tile_fwd alone (us per image, both,
-// by the mean rows). RGB, K 32: tiles of 5 x 5 groups and more (512 x 512, stride 2): 883 / 1,459 at 17, 1,383 /
-// 1,567 at 41, 2,169 / 1,651 at 61; smaller tiles, whose few groups wait for one another longer (512 x 512, stride
-// 3): 611 / 721 at 22, 763 / 750 at 34, 915 / 758 at 39. K 16: 1,102 / 1,284 at 45, 1,582 / 1,370 at 60. Gray,
-// K 32: 763 / 809 at 34, 859 / 818 at 40.
-int dense_mean(const FilterArgs& a) { return a.g.K == 16 ? 48 : a.g.C == 1 ? 36 : a.TR >= 5 ? 42 : 32; }
 
 template <int K, int C, typename Tin, bool MF>
 __global__ void __launch_bounds__(K * PS) sample_rows_kernel(FilterArgs a, int* __restrict__ st, int most) {
@@ -171,9 +164,9 @@ __global__ void __launch_bounds__(K * PS) sample_rows_kernel(FilterArgs a, int* 
 }
 
 template <int K>
-cudaError_t sample_rows(const FilterArgs& a, int* st, cudaStream_t s) {
+cudaError_t sample_rows(const FilterArgs& a, int most, int* st, cudaStream_t s) {
     const bool mf = a.mode == FM_VIDEO;
-    const int most = dense_mean(a) * SR_GROUPS;
+    most *= SR_GROUPS;
     if (a.g.C == 3) {
         if (mf) sample_rows_kernel<K, 3, uint8_t, true><<<SR_GROUPS, K * PS, 0, s>>>(a, st, most);
         else if (a.img_is_float) sample_rows_kernel<K, 3, float, false><<<SR_GROUPS, K * PS, 0, s>>>(a, st, most);
@@ -275,8 +268,29 @@ __global__ void __launch_bounds__(256) patch_dot_kernel(const float* __restrict_
 
 }  // namespace
 
-cudaError_t launch_sample_rows(const FilterArgs& a, int* st, cudaStream_t s) {
-    return a.g.K == 32 ? sample_rows<32>(a, st, s) : a.g.K == 16 ? sample_rows<16>(a, st, s) : cudaErrorInvalidValue;
+// Where planes and group filter (with the sampling) take as long as the tile kernel alone, us, both, by the mean rows.
+// The fewer groups a tile holds, the fewer warps work on it (with one, a third of them), and the earlier that is.
+// RGB, K 32: tiles of one group (256 x 264, stride 3) 283 / 305 at 13, 317 / 311 at 17, 359 / 315 at 25; 2 x 2
+// (350 x 358) 344 / 367 at 18, 391 / 376 at 26; 3 x 3 (512 x 512) 611 / 721 at 22, 763 / 750 at 34; 5 x 5 and more
+// (512 x 512, stride 2) 883 / 1,459 at 17, 1,383 / 1,567 at 41, 2,169 / 1,651 at 61. K 16: one group 249 / 270 at 19,
+// 285 / 276 at 28; 2 x 2 285 / 307 at 29, 331 / 321 at 43; 5 x 5 1,102 / 1,284 at 45, 1,582 / 1,370 at 60. Gray, K 32:
+// one group 183 / 201 at 14, 206 / 205 at 21; 2 x 2 192 / 215 at 14, 214 / 217 at 21; 3 x 3 281 / 310 at 20,
+// 383 / 319 at 30; 5 x 5 763 / 809 at 34, 859 / 818 at 40. Gray, K 16: one group 114 / 109 at 15 (4,420 references),
+// 161 / 174 at 15 (7,308). Below 4,000 references a third of that: RGB, K 32, 3,599 references 151 / 150 at 6,
+// K 16 132 / 134 at 9. With 8 slots or fewer the group filter is the faster one at any threshold.
+int group_rows_limit(const FilterArgs& a) {
+    constexpr int rgb32[] = {15, 20, 32, 36, 42}, gray32[] = {15, 20, 24, 30, 36};
+    constexpr int rgb16[] = {22, 32, 44, 48, 48}, gray16[] = {14, 24, 32, 44, 48};
+    const int K = a.g.K, t = std::min(a.TR, 5) - 1;
+    if (K <= 8) return kEveryRow;
+    if (a.g.ngroups() < 4000) return K == 32 ? 6 : 8;
+    return K == 32 ? (a.g.C == 3 ? rgb32 : gray32)[t] : (a.g.C == 3 ? rgb16 : gray16)[t];
+}
+
+cudaError_t launch_sample_rows(const FilterArgs& a, int most, int* st, cudaStream_t s) {
+    return a.g.K == 32   ? sample_rows<32>(a, most, st, s)
+           : a.g.K == 16 ? sample_rows<16>(a, most, st, s)
+                         : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_denom(const FilterArgs& a, cudaStream_t s) {

@@ -159,9 +159,12 @@ struct GroupArgs {
     int dense_rows;
     unsigned wrec;           // 2^32 / W, rounded down (filled by the launch)
 };
-// Sets st[2] where the sampled groups of the image keep more rows of coefficients than the group filter is the
-// faster one for (st: three zeroed words); FilterArgs as for the filter. K 16 or 32.
-cudaError_t launch_sample_rows(const FilterArgs& a, int* st, cudaStream_t s);
+// Mean rows of coefficients a group keeps up to which planes and group filter are the faster way; kEveryRow: at any.
+constexpr int kEveryRow = 1 << 20;
+int group_rows_limit(const FilterArgs& a);
+// Sets st[2] where the sampled groups of the image keep more rows than most in the mean (st: three zeroed words);
+// FilterArgs as for the filter.
+cudaError_t launch_sample_rows(const FilterArgs& a, int most, int* st, cudaStream_t s);
 // Fills a.cap and a.per_sm and returns the grid (persistent CTAs) of a launch.
 int group_grid(GroupArgs& a);
 size_t group_spill_floats(const GroupArgs& a, int grid);
