@@ -965,14 +965,6 @@ htsvd_status vjp_core(Workspace* w, const float* d_x, const Geo& g, const Resolv
     void *part, *spill = nullptr, *rc, *dot;
     ST(ws_get(w, S_PART, sizeof(float) * (size_t)t.ntx * t.nty * t.FHmax * t.FWmax * acc, &part));
     a.partials = (float*)part;
-    Geo g1 = g;
-    g1.C = 1;
-    { ProfScope ps_("denom", s); CK(launch_denom(a, s)); }
-    { ProfScope ps_("reduce", s); CK(launch_reduce((float*)part, g1, t.TR, t.ntx, t.nty, t.FHmax, t.FWmax, (float*)tmp, (float*)den, 0,
-                     nullptr, s)); }
-    { ProfScope ps_("div", s); CK(launch_div(d_grad_out, (const float*)den, npix, C, (float*)rimg, s)); }
-
-    // adjoint filter on r = gout / D with the masks of x: the planes of both images in the same bands
     a.mode = FM_ADJOINT;
     a.r_img = (const float*)rimg;
     a.out_img = d_out;
@@ -981,12 +973,33 @@ htsvd_status vjp_core(Workspace* w, const float* d_x, const Geo& g, const Resolv
     int per = t.nty, grid = 0;
     ga.nty_band = per;
     grid = group_grid(ga);
-    htsvd_status st = ga.per_sm < kGroupCtas ? HTSVD_ERR_OOM : HTSVD_OK;
+    const int most = group_rows_limit(a);
+    htsvd_status st = ga.per_sm < kGroupCtas || most < 0 ? HTSVD_ERR_OOM : HTSVD_OK;
     if (st == HTSVD_OK) st = ws_try(w, S_SPILL, sizeof(float) * group_spill_floats(ga, grid), &spill);
     if (st == HTSVD_OK) st = plane_bands(w, g, t.TR, t.nty, t.nty * t.ntx, 2, per, P);   // (two images: as two frames)
     if (st == HTSVD_OK) st = ws_try(w, S_DOT, sizeof(float) * P.most, &dot);
     if (st != HTSVD_OK && st != HTSVD_ERR_OOM) return st;
-    if (st != HTSVD_OK) {                          // no room for the planes or the CTAs: the tile kernel alone
+    const bool planes = st == HTSVD_OK, ask = planes && most != kEveryRow;
+    if (ask) {                                     // the sampled groups, beside the denominators
+        ST(ws_side(w));
+        CK(cudaEventRecord(w->ev_fork, s));
+        CK(cudaStreamWaitEvent(w->side, w->ev_fork, 0));
+        ProfScope ps_("sample_rows", w->side);
+        CK(cudaMemsetAsync(P.sample, 0, 3 * sizeof(int), w->side));
+        CK(launch_sample_rows(a, most, P.sample, w->side));
+        CK(cudaEventRecord(w->ev_join, w->side));
+        P.dense = R.dense = a.dense = P.sample + 2;
+    }
+    Geo g1 = g;
+    g1.C = 1;
+    { ProfScope ps_("denom", s); CK(launch_denom(a, s)); }
+    { ProfScope ps_("reduce", s); CK(launch_reduce((float*)part, g1, t.TR, t.ntx, t.nty, t.FHmax, t.FWmax, (float*)tmp, (float*)den, 0,
+                     nullptr, s)); }
+    { ProfScope ps_("div", s); CK(launch_div(d_grad_out, (const float*)den, npix, C, (float*)rimg, s)); }
+    if (ask) CK(cudaStreamWaitEvent(s, w->ev_join, 0));
+
+    // adjoint filter on r = gout / D with the masks of x: the planes of both images in the same bands
+    if (!planes) {                                 // they do not pay, or there is no room for them: the tile kernel alone
         ProfScope ps_("adjoint", s);
         CK(launch_filter(a, s));
         per = t.nty + 1;
@@ -1015,8 +1028,9 @@ htsvd_status vjp_core(Workspace* w, const float* d_x, const Geo& g, const Resolv
         ga.nty_band = t1 - t0;
         ProfScope ps_("adjoint", s);
         CK(launch_group(ga, std::min(grid, (t1 - t0) * t.ntx), s));
-        if (r.K > 8) {
+        if (ask || r.K > 8) {
             a.left = P.counter;
+            a.left_first = t0 * t.ntx;
             a.left_tiles = (t1 - t0) * t.ntx;
             CK(launch_filter(a, s));
             a.left = nullptr;

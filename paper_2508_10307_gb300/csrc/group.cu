@@ -278,7 +278,27 @@ __global__ void __launch_bounds__(256) patch_dot_kernel(const float* __restrict_
 // 383 / 319 at 30; 5 x 5 763 / 809 at 34, 859 / 818 at 40. Gray, K 16: one group 114 / 109 at 15 (4,420 references),
 // 161 / 174 at 15 (7,308). Below 4,000 references a third of that: RGB, K 32, 3,599 references 151 / 150 at 6,
 // K 16 132 / 134 at 9. With 8 slots or fewer the group filter is the faster one at any threshold.
+//
+// The backward pass, whose tiles are smaller at a size (two images are staged), RGB: K 32, one group 346 / 495 at 6,
+// 455 / 530 at 17, 611 / 553 at 38 (7,056 references); two and more 1,010 / 1,117 at 59, 1,258 / 1,168 at 88. K 16: one
+// group 332 / 342 at 19, 376 / 350 at 29; more 743 / 1,105 at 44, 748 / 755 at 84. Gray, K 32: one group 238 / 287
+// at 21, 275 / 287 at 32; more 484 / 565 at 70, 687 / 606 at 158. K 16: one group 171 / 185 at 11, 203 / 189 at 23.
+// K 8, one group: RGB 240 / 278 at 7, 319 / 302 at 41, gray 117 / 145 at 2, 153 / 148 at 17; more: the group filter
+// at any threshold. Below 3,000 references (K 32: 1,500; 961: 139 / 96 at 5, 1,681: 135 / 149 at 5, 344 / 276 at 245;
+// K 16, 1,681: 101 / 88 at 3) the tile kernel, but for images of so few
+// references that its tiles are the largest and fewer than the SMs (289: 344 / 580 at 5, 225: 1,143 / 1,085 at 173).
 int group_rows_limit(const FilterArgs& a) {
+    if (a.mode == FM_ADJOINT) {
+        const int K = a.g.K, ng = a.g.ngroups();
+        if (ng < (K == 32 ? 1500 : 3000)) {
+            if (a.ntx * a.nty >= device_sm_count()) return -1;
+            return K == 32 ? 60 : K >= 8 ? 40 : kEveryRow;
+        }
+        if (K == 32 && ng < 4000) return 14;
+        if (a.TR > 1) return K == 32 ? (a.g.C == 3 ? 80 : 110) : K == 16 ? (a.g.C == 3 ? 84 : 100) : kEveryRow;
+        if (a.g.C == 3) return K == 32 ? 20 : K == 8 ? (ng < 4000 ? 14 : 24) : ng < 4000 ? 9 : 16;
+        return ng < 4000 ? 3 : K == 32 ? 24 : K == 16 ? 10 : 8;
+    }
     constexpr int rgb32[] = {15, 20, 32, 36, 42}, gray32[] = {15, 20, 24, 30, 36};
     constexpr int rgb16[] = {22, 32, 44, 48, 48}, gray16[] = {14, 24, 32, 44, 48};
     const int K = a.g.K, t = std::min(a.TR, 5) - 1;
@@ -288,9 +308,14 @@ int group_rows_limit(const FilterArgs& a) {
 }
 
 cudaError_t launch_sample_rows(const FilterArgs& a, int most, int* st, cudaStream_t s) {
-    return a.g.K == 32   ? sample_rows<32>(a, most, st, s)
-           : a.g.K == 16 ? sample_rows<16>(a, most, st, s)
-                         : cudaErrorInvalidValue;
+    switch (a.g.K) {
+        case 2: return sample_rows<2>(a, most, st, s);
+        case 4: return sample_rows<4>(a, most, st, s);
+        case 8: return sample_rows<8>(a, most, st, s);
+        case 16: return sample_rows<16>(a, most, st, s);
+        case 32: return sample_rows<32>(a, most, st, s);
+    }
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_denom(const FilterArgs& a, cudaStream_t s) {

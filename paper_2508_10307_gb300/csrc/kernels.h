@@ -159,7 +159,8 @@ struct GroupArgs {
     int dense_rows;
     unsigned wrec;           // 2^32 / W, rounded down (filled by the launch)
 };
-// Mean rows of coefficients a group keeps up to which planes and group filter are the faster way; kEveryRow: at any.
+// Mean rows of coefficients a group keeps up to which planes and group filter are the faster way; kEveryRow: at
+// any, -1: at none.
 constexpr int kEveryRow = 1 << 20;
 int group_rows_limit(const FilterArgs& a);
 // Sets st[2] where the sampled groups of the image keep more rows than most in the mean (st: three zeroed words);

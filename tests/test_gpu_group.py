@@ -89,3 +89,25 @@ def test_batch_takes_any_tile_edge(tile):
     prm = dict(stride=1, window=5, K=8)
     out, = H.denoise_batch([x], [20.0], dict(prm, tile=tile))
     assert max_abs(out.cpu().numpy(), H.denoise(x, 20.0, prm).cpu().numpy()) <= PIX_TOL
+
+
+@pytest.mark.parametrize("shape,K,mult", [
+    ((118, 121, 3), 2, 0.0), ((118, 121, 3), 2, 0.5), ((118, 121, 1), 4, 0.0), ((118, 121, 1), 4, 0.7),
+    ((118, 121, 3), 8, 0.0), ((118, 121, 1), 8, 0.7),          # tiles of one group, few rows and many
+    ((260, 263, 1), 16, 0.0), ((260, 263, 1), 16, 0.5),        # larger tiles
+    ((34, 37, 3), 32, 0.0), ((34, 37, 3), 32, 1.0), ((60, 52, 3), 16, 0.0),
+])
+def test_gradients_by_size_and_rows_kept(shape, K, mult):
+    """The backward pass samples how many rows its groups keep and takes one kernel or the other."""
+    x = synth.add_gaussian_float(synth.clean_image(*shape, 7), 20.0, 7)
+    prm = dict(stride=2, window=9, K=K, tau_mult=mult)
+    rng = np.random.default_rng(4)
+    r = O.denoise(x.astype(np.float64), 20.0, prm, keep_masks=True)
+    w = rng.uniform(0.5, 1.5, size=len(r.idx))
+    gout = rng.standard_normal(x.shape)
+    gx_o, gw_o = O.denoise_fixed_vjp(x.astype(np.float64), gout, r.idx, r.masks, r.U, r.V, w, 8)
+    xt, wt = torch.from_numpy(x).cuda(), torch.from_numpy(w.astype(np.float32)).cuda()
+    out, info = H.denoise_f32(xt, 20.0, prm, w=wt, return_info=True)
+    gx, gw = H.denoise_vjp(xt, 20.0, info["idx"], wt, out, torch.from_numpy(gout.astype(np.float32)).cuda(), prm)
+    assert np.abs(gx.cpu().numpy() - gx_o).max() <= 1e-4 * np.abs(gx_o).max()
+    assert np.abs(gw.cpu().numpy() - gw_o).max() <= 1e-4 * max(1.0, np.abs(gw_o).max())
