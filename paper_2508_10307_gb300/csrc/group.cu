@@ -283,7 +283,8 @@ __global__ void __launch_bounds__(256) patch_dot_kernel(const float* __restrict_
 // 455 / 530 at 17, 611 / 553 at 38 (7,056 references); two and more 1,010 / 1,117 at 59, 1,258 / 1,168 at 88. K 16: one
 // group 332 / 342 at 19, 376 / 350 at 29; more 743 / 1,105 at 44, 748 / 755 at 84. Gray, K 32: one group 238 / 287
 // at 21, 275 / 287 at 32; more 484 / 565 at 70, 687 / 606 at 158. K 16: one group 171 / 185 at 11, 203 / 189 at 23.
-// K 8, one group: RGB 240 / 278 at 7, 319 / 302 at 41, gray 117 / 145 at 2, 153 / 148 at 17; more: the group filter
+// K 8, one group: RGB 240 / 278 at 7, 319 / 302 at 41, gray 117 / 145 at 2, 153 / 148 at 17
+// (K 2, 4,225 references: 83 / 74 at 1); more: the group filter
 // at any threshold. Below 3,000 references (K 32: 1,500; 961: 139 / 96 at 5, 1,681: 135 / 149 at 5, 344 / 276 at 245;
 // K 16, 1,681: 101 / 88 at 3) the tile kernel, but for images of so few
 // references that its tiles are the largest and fewer than the SMs (289: 344 / 580 at 5, 225: 1,143 / 1,085 at 173).
@@ -295,6 +296,7 @@ int group_rows_limit(const FilterArgs& a) {
             return K == 32 ? 60 : K >= 8 ? 40 : kEveryRow;
         }
         if (K == 32 && ng < 4000) return 14;
+        if (K <= 8 && a.g.C == 1 && ng < 5000) return -1;
         if (a.TR > 1) return K == 32 ? (a.g.C == 3 ? 80 : 110) : K == 16 ? (a.g.C == 3 ? 84 : 100) : kEveryRow;
         if (a.g.C == 3) return K == 32 ? 20 : K == 8 ? (ng < 4000 ? 14 : 24) : ng < 4000 ? 9 : 16;
         return ng < 4000 ? 3 : K == 32 ? 24 : K == 16 ? 10 : 8;
