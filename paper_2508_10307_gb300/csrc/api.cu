@@ -1617,7 +1617,7 @@ bool volume_takes_planes(const VolGeo& g) {
 htsvd_status run_volume_filter(Workspace* w, const VolFilterArgs& a, int64_t ng, cudaStream_t s) {
     const VolGeo& g = a.g;
     const int ntz = volume_tiles_z(g);
-    void *coef, *pn, *rec;
+    void *coef, *pn, *rec, *ctr;
     bool planes = volume_takes_planes(g);
     int per = ntz;
     while (planes) {
@@ -1634,6 +1634,7 @@ htsvd_status run_volume_filter(Workspace* w, const VolFilterArgs& a, int64_t ng,
             st = ws_try(w, S_PLANE, pos * 64 * sizeof(float), &coef);
             if (st == HTSVD_OK) st = ws_try(w, S_PNRM, pos * sizeof(float), &pn);
             if (st == HTSVD_OK) st = ws_try(w, S_SPILL, volume_group_rec_bytes(g, per), &rec);
+            if (st == HTSVD_OK) st = ws_try(w, S_CTR, 3 * sizeof(int), &ctr);
         }
         if (st == HTSVD_OK) break;
         if (st != HTSVD_ERR_OOM) return st;
@@ -1644,6 +1645,18 @@ htsvd_status run_volume_filter(Workspace* w, const VolFilterArgs& a, int64_t ng,
         ProfScope ps_("volume_filter", s);
         CK(launch_volume_filter(a, s));
         return HTSVD_OK;
+    }
+    VolFilterArgs f = a;
+    const int most = volume_rows_limit(g);
+    if (most != kEveryRow) {                       // the sampled groups, beside the first planes
+        ST(ws_side(w));
+        CK(cudaEventRecord(w->ev_fork, s));
+        CK(cudaStreamWaitEvent(w->side, w->ev_fork, 0));
+        ProfScope ps_("volume_sample", w->side);
+        CK(cudaMemsetAsync(ctr, 0, 3 * sizeof(int), w->side));
+        CK(launch_volume_sample(a, most, (int*)ctr, w->side));
+        CK(cudaEventRecord(w->ev_join, w->side));
+        f.dense = (const int*)ctr + 2;
     }
     if (a.mask_out) CK(cudaMemsetAsync(a.mask_out, 0, sizeof(uint32_t) * 2 * g.K * (size_t)ng, s));
     for (int t = 0; t < ntz; t += per) {
@@ -1660,8 +1673,9 @@ htsvd_status run_volume_filter(Workspace* w, const VolFilterArgs& a, int64_t ng,
         pa.coef = (float*)coef;
         pa.pn = (float*)pn;
         { ProfScope ps_("volume_planes", s); CK(launch_volume_plane(pa, z1 - z0, s)); }
+        if (t == 0 && f.dense) CK(cudaStreamWaitEvent(s, w->ev_join, 0));
         VolGroupArgs ga{};
-        ga.f = a;
+        ga.f = f;
         ga.coef = (const float*)coef;
         ga.pn = (const float*)pn;
         ga.pz0 = z0;
@@ -1669,6 +1683,10 @@ htsvd_status run_volume_filter(Workspace* w, const VolFilterArgs& a, int64_t ng,
         ga.rec = rec;
         ProfScope ps_("volume_filter", s);
         CK(launch_volume_group(ga, tz, s));
+    }
+    if (f.dense) {                                 // every tile, where the sampled groups keep too much for the above
+        ProfScope ps_("volume_filter", s);
+        CK(launch_volume_filter(f, s));
     }
     return HTSVD_OK;
 }

@@ -246,8 +246,9 @@ struct VolFilterArgs {
     float* den;
     uint32_t* mask_out;      // optional, 2 K words per group (bit m * 64 + (i * 4 + j) * 4 + k)
     float* weights_out;      // optional
+    const int* dense;        // optional: volume_filter_kernel works only where it is set, volume_group_kernel where not
 };
-size_t volume_filter_smem_bytes(const VolGeo& g);
+bool volume_filter_fits(const VolGeo& g);
 cudaError_t launch_volume_filter(const VolFilterArgs& a, cudaStream_t s);
 cudaError_t launch_volume_finalize(const float* num, const float* den, long long n, float* out, cudaStream_t s);
 
@@ -271,6 +272,10 @@ struct VolGroupArgs {
     void* rec;               // volume_group_rec_bytes(g, tile planes)
 };
 bool volume_group_fits(const VolGeo& g);
+// Mean rows of coefficients a group keeps up to which planes and group filter are the faster way (kEveryRow: at any),
+// and whether the sampled groups of the volume keep more than most: st[2] of three zeroed words is set. K 16 or 32.
+int volume_rows_limit(const VolGeo& g);
+cudaError_t launch_volume_sample(const VolFilterArgs& a, int most, int* st, cudaStream_t s);
 int volume_tiles_z(const VolGeo& g);
 int volume_tiles_plane(const VolGeo& g);
 // Position planes [z0, z1) that the tile planes [t0, t1) gather from.

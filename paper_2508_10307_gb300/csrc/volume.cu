@@ -442,6 +442,7 @@ __device__ __forceinline__ void load_cube(const uint8_t* fb, int fy, int FXp, in
 template <int K>
 __global__ void __launch_bounds__(kVolWarps * 32, 2)
 volume_filter_kernel(VolFilterArgs A) {
+    if (A.dense && !*A.dense) return;
     const VolGeo g = A.g;
     __shared__ VolSmem sm;
     extern __shared__ __align__(16) unsigned char dyn[];
@@ -951,6 +952,8 @@ double volume_bases_host(const unsigned long long* mom, double* b64) {
     return gap;
 }
 
+namespace {
+constexpr size_t kVolSmem = 160 * 1024;
 size_t volume_filter_smem_bytes(const VolGeo& g) {
     const int ext[3] = {g.wnz, g.wny, g.wnx};
     int fn[3];
@@ -959,6 +962,9 @@ size_t volume_filter_smem_bytes(const VolGeo& g) {
     const size_t nfb = (size_t)fn[0] * fn[1] * FXp;
     return kHcBytes + ((nfb + 15) & ~(size_t)15) + sizeof(float) * 3 * (size_t)fn[0] * fn[1] * fn[2];
 }
+}  // namespace
+
+bool volume_filter_fits(const VolGeo& g) { return volume_filter_smem_bytes(g) <= kVolSmem; }
 
 template <int K>
 static cudaError_t launch_volume_filter_k(const VolFilterArgs& a, int ntiles, size_t smem, cudaStream_t s) {
@@ -967,7 +973,7 @@ static cudaError_t launch_volume_filter_k(const VolFilterArgs& a, int ntiles, si
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (configured != dev) {
-        e = cudaFuncSetAttribute(volume_filter_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+        e = cudaFuncSetAttribute(volume_filter_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVolSmem);
         if (e != cudaSuccess) return e;
         configured = dev;
     }

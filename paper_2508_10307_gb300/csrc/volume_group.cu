@@ -307,6 +307,7 @@ __global__ void __launch_bounds__(VG_THREADS, 2) volume_group_kernel(const __gri
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ VolSm sm;
     const VolFilterArgs& A = G.f;
+    if (A.dense && *A.dense) return;
     const VolGeo& g = A.g;
     const int tid = threadIdx.x, warp = __shfl_sync(ALL, tid >> 5, 0), lane = tid & 31;
     // tile of references and its footprint
@@ -570,6 +571,88 @@ __global__ void __launch_bounds__(VG_THREADS, 2) volume_group_kernel(const __gri
     }
 }
 
+// Rows of coefficients that VS_GROUPS groups spread over the volume keep, as sample_rows_kernel counts them for
+// images: thread (cube k, basis row i) projects its row, 64 threads take the Haar transform of a coefficient each.
+// It runs beside the first band's planes.
+constexpr int VS_GROUPS = 128;
+
+template <int K>
+__global__ void __launch_bounds__(K * VE) volume_sample_kernel(VolFilterArgs A, int* __restrict__ st, int most) {
+    __shared__ float sm[K * 64];                                       // [k][i][j][tube]
+    __shared__ unsigned mask[VE];
+    const VolGeo& g = A.g;
+    const int tid = threadIdx.x;
+    const long long ng = (long long)g.nrz * g.nry * g.nrx;
+    const long long grp = (2ll * blockIdx.x + 1) * ng / (2 * VS_GROUPS);
+    if (tid < VE) mask[tid] = 0u;
+    {
+        const int k = tid >> 2, i = tid & 3;
+        const uint8_t* cube = A.vol + A.idx[grp * K + k];
+        const size_t plane = (size_t)g.H * g.W;
+        const double *U = A.basis64, *V = A.basis64 + 4 * 16 * 2;      // [slice][a * 4 + i][re, im]
+        float y0[VE] = {}, y2[VE] = {}, yr[VE] = {}, yi[VE] = {};
+#pragma unroll
+        for (int a = 0; a < VE; ++a) {
+            const float u0 = (float)U[(a * 4 + i) * 2], u2 = (float)U[(32 + a * 4 + i) * 2];
+            const float ur = (float)U[(16 + a * 4 + i) * 2], ui = (float)U[(16 + a * 4 + i) * 2 + 1];
+#pragma unroll
+            for (int b = 0; b < VE; ++b) {
+                const uint8_t* p = cube + (size_t)a * g.W + b;
+                const float p0 = p[0], p1 = p[plane], p2 = p[2 * plane], p3 = p[3 * plane];
+                const float Xr = p0 - p2, Xi = p3 - p1;
+                y0[b] = fmaf(u0, (p0 + p1) + (p2 + p3), y0[b]);
+                y2[b] = fmaf(u2, (p0 - p1) + (p2 - p3), y2[b]);
+                yr[b] = fmaf(ur, Xr, fmaf(ui, Xi, yr[b]));
+                yi[b] = fmaf(ur, Xi, fmaf(-ui, Xr, yi[b]));
+            }
+        }
+        float* d = sm + tid * 16;
+#pragma unroll
+        for (int j = 0; j < VE; ++j) {
+            float z0 = 0.f, z2 = 0.f, zr = 0.f, zi = 0.f;
+#pragma unroll
+            for (int b = 0; b < VE; ++b) {
+                const float vr = (float)V[(16 + b * 4 + j) * 2], vi = (float)V[(16 + b * 4 + j) * 2 + 1];
+                z0 = fmaf(y0[b], (float)V[(b * 4 + j) * 2], z0);
+                z2 = fmaf(y2[b], (float)V[(32 + b * 4 + j) * 2], z2);
+                zr = fmaf(yr[b], vr, fmaf(-yi[b], vi, zr));
+                zi = fmaf(yr[b], vi, fmaf(yi[b], vr, zi));
+            }
+            d[j * 4] = 0.25f * fmaf(2.f, zr, z0 + z2);
+            d[j * 4 + 1] = 0.25f * fmaf(-2.f, zi, z0 - z2);
+            d[j * 4 + 2] = 0.25f * fmaf(-2.f, zr, z0 + z2);
+            d[j * 4 + 3] = 0.25f * fmaf(2.f, zi, z0 - z2);
+        }
+    }
+    __syncthreads();
+    if (tid < 64) {
+        float p[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) p[k] = sm[k * 64 + tid];
+#pragma unroll
+        for (int d = 1; d < K; d <<= 1)
+#pragma unroll
+            for (int m = 0; m < K; m += 2 * d) {
+                const float x = p[m], y = p[m + d];
+                p[m + d] = x - y;
+                p[m] = x + y;
+            }
+        unsigned keep = 0u;
+#pragma unroll
+        for (int l = 0; l < K; ++l)
+            if (fabsf(p[l]) >= A.tau32 * v_root(l == 0 ? v_log2(K) : v_ctz(l) + 1)) keep |= 1u << l;
+        atomicOr(&mask[tid >> 4], keep);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        int rows = 0;
+        for (int i = 0; i < VE; ++i) rows += __popc(mask[i]);
+        atomicAdd(st, rows);
+        __threadfence();
+        if (atomicAdd(st + 1, 1) == VS_GROUPS - 1) st[2] = atomicAdd(st, 0) > most * VS_GROUPS;
+    }
+}
+
 // Voxels of a tile's footprint, at most a million (in 64 bits: strides of a few hundred pass 2^31).
 int vol_nvox(const VolGeo& g) {
     const int ext[3] = {g.wnz, g.wny, g.wnx};
@@ -593,6 +676,26 @@ cudaError_t launch_vg(const VolGroupArgs& a, int tiles, cudaStream_t s) {
 
 bool volume_group_fits(const VolGeo& g) {
     return vol_layout(vol_nvox(g), g.K * 4).total <= 110 * 1024 && g.H / VP_NY <= 65535;
+}
+
+// us of the filter with its planes against volume_filter_kernel, window 5, K 32, by the rows kept per group: 7,600
+// references 178 / 198 at 10, 215 / 205 at 17, 408 / 333 at 64; 31,744: 484 / 540 at 26, 581 / 583 at 38, 1,386 / 1,068
+// at 112; 120,050: 1,782 / 1,978 at 38, 2,363 / 2,314 at 64, 7,124 / 5,253 at 127. K 16: 165 / 166 at 18, 393 / 412 at
+// 30, 604 / 540 at 55; 1,214 / 1,380 at 30, 1,801 / 1,732 at 54. (Leaving single tiles to the other kernel, as images
+// do, took 447 us at 7,600 references and 26 rows, since each kernel waits for its last tiles, and the registers it
+// needed cost 7 % everywhere.) With 8 slots or fewer: at any.
+int volume_rows_limit(const VolGeo& g) {
+    const int64_t ng = (int64_t)g.nrz * g.nry * g.nrx;
+    if (g.K <= 8 || !volume_filter_fits(g)) return kEveryRow;
+    if (g.K == 32) return ng < 15000 ? 14 : ng < 60000 ? 38 : 62;
+    return ng < 15000 ? 18 : ng < 60000 ? 36 : 47;
+}
+
+cudaError_t launch_volume_sample(const VolFilterArgs& a, int most, int* st, cudaStream_t s) {
+    if (a.g.K == 32) volume_sample_kernel<32><<<VS_GROUPS, 32 * VE, 0, s>>>(a, st, most);
+    else if (a.g.K == 16) volume_sample_kernel<16><<<VS_GROUPS, 16 * VE, 0, s>>>(a, st, most);
+    else return cudaErrorInvalidValue;
+    return cudaGetLastError();
 }
 
 int volume_tiles_z(const VolGeo& g) { return (g.nrz + VT - 1) / VT; }

@@ -106,7 +106,7 @@ def test_gradients(C, K, mult):
             assert (a - r).abs().max() <= 1e-4 * max(1.0, a.abs().max().item())
 
 
-@pytest.mark.parametrize("K,mult", [(32, 0.0), (8, 1.0)])
+@pytest.mark.parametrize("K,mult", [(32, 0.0), (8, 1.0), (16, 1.0)])
 def test_volume(K, mult):
     v = torch.from_numpy(synth.add_gaussian(synth.clean_volume(48, 39, 40, 6), 11.5, 6)).cuda()
 

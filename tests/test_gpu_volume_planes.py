@@ -23,8 +23,10 @@ pytestmark = pytest.mark.gpu
     ((56, 57, 58), dict(stride=3, window=7, K=32, tau_mult=40.0), 11.5),         # hardly a coefficient kept
 ])
 def test_volume_filter_matches_oracle(shape, prm, sigma):
-    prm = dict(ps=4, **prm)
-    v = synth.add_gaussian(synth.clean_volume(*shape, 6), sigma, 6)
+    _check(synth.add_gaussian(synth.clean_volume(*shape, 6), sigma, 6), dict(ps=4, **prm), sigma)
+
+
+def _check(v, prm, sigma):
     r = O.denoise_volume(v, sigma, prm, keep_masks=True)
     out, info = H.denoise_volume(torch.from_numpy(v).cuda(), sigma, prm, return_info=True, masks=True, weights=True)
     assert len(r.idx) >= 5000
@@ -37,3 +39,12 @@ def test_volume_filter_matches_oracle(shape, prm, sigma):
         assert all((int(g), int(wd) * 32 + b) in amb for b in range(32) if (d >> b) & 1)
     np.testing.assert_allclose(info["weights"].cpu().numpy(), r.weights, rtol=1e-6)
     assert max_abs(out.cpu().numpy(), r.out) <= PIX_TOL
+
+
+@pytest.mark.parametrize("K,agg,half", [(32, "uniform", 20), (16, "sparsity", 8), (16, "uniform", 39)])
+def test_dense_volumes(K, agg, half):
+    """Noise above the threshold in a part: the groups sampled decide which kernel filters the volume."""
+    v = synth.add_gaussian(synth.clean_volume(44, 39, 38, 6), 4.0, 6)
+    rng = np.random.default_rng(3)
+    v[:, half:] = rng.integers(0, 256, v[:, half:].shape)
+    _check(np.ascontiguousarray(v), dict(ps=4, stride=2, window=4, K=K, agg_mode=agg), 15.0)
