@@ -816,6 +816,122 @@ htsvd_status denoise_impl(const void* d_in, int is_float, int H, int W, int C, d
     return denoise_checked(d_in, is_float, H, W, C, sigma, p, r, d_w, d_out, d_idx_out, s);
 }
 
+// References below which the images of a batch share their launches: those that a filter alone takes without
+// planes. us per batch of 2 / 8 / 64 images, so and on the lanes, RGB, window 18, K 32: 64 x 64 185 / 286 / 1,333
+// and 218 / 385 / 2,383; 96 x 96 215 / 432 / 2,377 and 213 / 609 / 4,241; 150 x 150 297 / 763 / 5,425 and 381 / 824 /
+// 5,707. Gray, 64 x 64 153 / 220 / 728 and 189 / 325 / 1,844; 150 x 150 210 / 451 / 2,840 and 322 / 557 / 3,597.
+constexpr int kSmallGroups = kPlaneGroups;
+
+// Alg. 1 on n small images, checked, in one launch a phase; the bases on the side stream beside the grouping, as
+// for one image.
+htsvd_status denoise_small(Workspace* w, const htsvd_image* imgs, const int* which, int n, const Resolved& r,
+                           cudaStream_t s) {
+    SmallBatch B;
+    std::memset(&B, 0, sizeof(B));
+    const int C = imgs[which[0]].C;
+    B.n = n;
+    B.C = C;
+    B.s = r.s;
+    B.win = r.win;
+    B.K = r.K;
+    B.mode = resolve_mode(r, C);
+    B.agg_mode = r.agg_mode;
+    B.gamma2 = r.gamma * r.gamma;
+    int64_t refs = 0;
+    for (int i = 0; i < n; ++i) refs += make_geo(imgs[which[i]].H, imgs[which[i]].W, C, r.s, r.win, r.K).ngroups();
+    const int64_t want = 2 * (int64_t)device_sm_count();        // as launch_moments cuts one image
+    B.per = (int)std::min<int64_t>(256, ((refs + want - 1) / want + 31) / 32 * 32);
+    int mom = 0, bm = 0, flt = 0, red = 0;
+    size_t idx_ints = 0, part = 0, smem_bm = 0, smem_f = 0;
+    const int acc = C == 3 ? 4 : 2;
+    for (int i = 0; i < n; ++i) {
+        const htsvd_image& im = imgs[which[i]];
+        const Geo g = make_geo(im.H, im.W, C, r.s, r.win, r.K);
+        BMArgs ba{};
+        ba.g = g;
+        ba.mode = B.mode;
+        ba.rstep = 1;
+        choose_bm_tiles(g, 1, ba.TRy, ba.TRx);
+        bm_fit_tiles(ba);
+        // tile edge: us of filter and reduction at 2 / 3 / 4, window 18, RGB, K 32: 53 / 68 / 100 on 450 references of the
+        // set, 92 / 91 / 106 on 1,800, 247 / 236 / 238 on 7,688, 478 / 425 / 427 on 14,400, 909 / 811 / 777 on 30,752
+        // (1: 76, 139, 395, 782, 1,492); smaller where two CTAs would not share an SM
+        FilterTiling t{};
+        FilterArgs fa{};
+        fa.g = g;
+        fa.mode = FM_FORWARD;
+        for (int e = refs < 1200 ? 2 : refs < 10000 ? 3 : 4; r.tile == 0 && e > 0; --e) {
+            t = choose_filter_tiling(g, 1, FM_FORWARD, e);
+            fa.FHmax = t.FHmax;
+            fa.FWmax = t.FWmax;
+            if (t.TR > 0 && filter_smem_bytes(fa) <= 112 * 1024) break;
+            t.TR = 0;
+        }
+        if (t.TR == 0) t = choose_filter_tiling(g, 1, FM_FORWARD, r.tile);
+        if (t.TR == 0) return HTSVD_ERR_UNSUPPORTED;
+        fa.FHmax = t.FHmax;
+        fa.FWmax = t.FWmax;
+        SmallImage& m = B.im[i];
+        m.in = im.d_in;
+        m.out = im.d_out;
+        m.idx = im.d_idx_out;
+        m.tau = r.tau_mult * im.sigma;
+        m.part = (long long)part;
+        m.H = im.H;
+        m.W = im.W;
+        m.TR = t.TR;
+        m.TRy = ba.TRy;
+        m.TRx = ba.TRx;
+        m.mom0 = mom;
+        m.bm0 = bm;
+        m.flt0 = flt;
+        m.red0 = red;
+        mom += (g.ngroups() + B.per - 1) / B.per;
+        bm += ((g.nrx + ba.TRx - 1) / ba.TRx) * ((g.nry + ba.TRy - 1) / ba.TRy);
+        flt += t.ntx * t.nty;
+        red += (int)(((int64_t)im.H * im.W + 255) / 256);
+        part += ((size_t)t.ntx * t.nty * t.FHmax * t.FWmax * acc + 63) & ~(size_t)63;
+        if (!im.d_idx_out) idx_ints += ((size_t)g.ngroups() * r.K + 63) & ~(size_t)63;
+        smem_bm = std::max(smem_bm, bm_smem_bytes(ba));
+        smem_f = std::max(smem_f, filter_smem_bytes(fa));
+    }
+    if (smem_bm > 227 * 1024 || smem_f > 227 * 1024) return HTSVD_ERR_UNSUPPORTED;
+    void *p_mom, *p64, *p32, *p_idx, *p_part;
+    ST(ws_get(w, S_MOM, sizeof(unsigned long long) * 2 * PS2 * C * C * n, &p_mom));
+    ST(ws_get(w, S_B64, sizeof(double) * 4 * C * PS2 * n, &p64));
+    ST(ws_get(w, S_B32, sizeof(float) * 512 * n, &p32));
+    ST(ws_get(w, S_IDX, sizeof(int32_t) * idx_ints, &p_idx));
+    ST(ws_get(w, S_PART, sizeof(float) * part, &p_part));
+    B.mom = (unsigned long long*)p_mom;
+    B.b64 = (double*)p64;
+    B.b32 = (float*)p32;
+    B.part = (float*)p_part;
+    int32_t* own = (int32_t*)p_idx;
+    for (int i = 0; i < n; ++i)
+        if (!B.im[i].idx) {
+            B.im[i].idx = own;
+            own += ((size_t)make_geo(B.im[i].H, B.im[i].W, C, r.s, r.win, r.K).ngroups() * r.K + 63) & ~(size_t)63;
+        }
+    ST(ws_side(w));
+    CK(cudaEventRecord(w->ev_fork, s));
+    CK(cudaStreamWaitEvent(w->side, w->ev_fork, 0));
+    { ProfScope ps_("moments", w->side); CK(launch_moments_small(B, mom, w->side)); }
+    // The bases are FP64 chains of a warp each, 85 us alone on an SM and up to 400 beside the grouping or each other.
+    // Where there is an SM for each and the grouping is short, it starts after the moments, on the other SMs.
+    const bool alone = n * basis_problems(C) <= device_sm_count() && bm <= 10 * device_sm_count();
+    if (alone) {
+        CK(cudaEventRecord(w->ev_join, w->side));
+        CK(cudaStreamWaitEvent(s, w->ev_join, 0));
+    }
+    { ProfScope ps_("basis", w->side); CK(launch_basis_small(B, alone, w->side)); }
+    CK(cudaEventRecord(w->ev_join, w->side));
+    { ProfScope ps_("block_match", s); CK(launch_block_match_small(B, bm, smem_bm, s)); }
+    CK(cudaStreamWaitEvent(s, w->ev_join, 0));
+    { ProfScope ps_("filter", s); CK(launch_filter_small(B, flt, smem_f, s)); }
+    { ProfScope ps_("reduce", s); CK(launch_reduce_small(B, red, s)); }
+    return HTSVD_OK;
+}
+
 // A clip, frame by frame (real-world color video denoising, Sec. IV): output frame t is Alg. 1 on
 // frame t (its own sigma, estimated or given, and its own global bases), except that grouping
 // searches the spatial window in frames t - T .. t + T and only the patches lying in frame t are
@@ -1257,7 +1373,19 @@ htsvd_status htsvd_denoise_batch(const htsvd_image* imgs, int32_t n, const htsvd
     }
     Workspace* w = workspace_for(s);
     if (!w) return HTSVD_ERR_OOM;
-    const int lanes = std::min(n, kBatchLanes);
+    // largest images first; the small ones in sets that share their launches
+    std::vector<int> order(n);
+    for (int i = 0; i < n; ++i) order[i] = i;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        return (int64_t)imgs[a].H * imgs[a].W > (int64_t)imgs[b].H * imgs[b].W;
+    });
+    int large = n;
+    while (large > 0 &&
+           (int64_t)ref_count(imgs[order[large - 1]].H, r.s) * ref_count(imgs[order[large - 1]].W, r.s) < kSmallGroups)
+        --large;
+    if (n - large < 2) large = n;
+    const int jobs = large + (n - large + kSmallImages - 1) / kSmallImages;
+    const int lanes = std::min(jobs, kBatchLanes);
     std::lock_guard<std::mutex> lk(w->batch_mu);
     htsvd_status late = take_timeout(w);     // of an earlier call, on any lane (each reported once, together)
     for (int l = 0; l < kBatchLanes; ++l) {
@@ -1276,21 +1404,22 @@ htsvd_status htsvd_denoise_batch(const htsvd_image* imgs, int32_t n, const htsvd
         lw->share = lanes;
         lw->wait_ns = w->wait_ns;
     }
-    // largest images first, each to the lane with the least work so far (a lane's workspace then grows once)
-    std::vector<int> order(n);
-    for (int i = 0; i < n; ++i) order[i] = i;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-        return (int64_t)imgs[a].H * imgs[a].W > (int64_t)imgs[b].H * imgs[b].W;
-    });
+    // each to the lane with the least work so far (a lane's workspace then grows once)
     int64_t load[kBatchLanes] = {};
     CK(cudaEventRecord(w->ev_batch, s));
     for (int l = 0; l < lanes; ++l) CK(cudaStreamWaitEvent(w->lane[l], w->ev_batch, 0));
     htsvd_status st = HTSVD_OK;
-    for (int k = 0; k < n && st == HTSVD_OK; ++k) {
+    for (int k = 0; k < large && st == HTSVD_OK; ++k) {
         const htsvd_image& im = imgs[order[k]];
         const int l = (int)(std::min_element(load, load + lanes) - load);
         load[l] += (int64_t)im.H * im.W;
         st = denoise_checked(im.d_in, 0, im.H, im.W, im.C, im.sigma, &q, r, nullptr, im.d_out, im.d_idx_out, w->lane[l]);
+    }
+    for (int k = large; k < n && st == HTSVD_OK; k += kSmallImages) {
+        const int m = std::min(kSmallImages, n - k), l = (int)(std::min_element(load, load + lanes) - load);
+        for (int i = 0; i < m; ++i) load[l] += (int64_t)imgs[order[k + i]].H * imgs[order[k + i]].W;
+        Workspace* lw = workspace_for(w->lane[l]);
+        st = lw ? denoise_small(lw, imgs, order.data() + k, m, r, w->lane[l]) : HTSVD_ERR_OOM;
     }
     for (int l = 0; l < lanes; ++l) {          // joined on every path: the caller's stream covers the lanes' work
         CK(cudaEventRecord(w->ev_lane[l], w->lane[l]));

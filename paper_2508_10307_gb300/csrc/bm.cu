@@ -22,6 +22,7 @@
 
 #include "kernels.h"
 #include "lane_sort.cuh"
+#include "small_batch.cuh"
 #include "tc.cuh"
 
 namespace htsvd {
@@ -601,6 +602,28 @@ __global__ void __launch_bounds__(BM_THREADS, 2) block_match_video_kernel(BMArgs
     bm_tile<true>(a, blockIdx.y, blockIdx.x, bsm);
 }
 
+__global__ void __launch_bounds__(BM_THREADS, 2) block_match_small_kernel(const __grid_constant__ SmallBatch B) {
+    extern __shared__ __align__(16) unsigned char bsm[];
+    __shared__ BMArgs a;
+    const SmallImage& m = B.im[small_find<&SmallImage::bm0>(B, blockIdx.x)];
+    if (threadIdx.x == 0) {
+        a = BMArgs{};
+        a.img = m.in;
+        a.g = small_geo(B, m);
+        a.mode = B.mode;
+        a.gamma2 = B.gamma2;
+        a.rstep = 1;
+        a.nry_s = a.g.nry;
+        a.nrx_s = a.g.nrx;
+        a.TRy = m.TRy;
+        a.TRx = m.TRx;
+        a.idx = m.idx;
+    }
+    __syncthreads();
+    const int t = blockIdx.x - m.bm0, ntx = (a.nrx_s + a.TRx - 1) / a.TRx;
+    bm_tile<false>(a, t / ntx, t % ntx, bsm);
+}
+
 #include "bm_tc.cuh"
 
 constexpr size_t BM_SMEM_TARGET = 100 * 1024;    // leaves room for two CTAs per SM
@@ -638,6 +661,17 @@ cudaError_t launch_block_match(const BMArgs& a, cudaStream_t s) {
     }
     dim3 grid((a.nrx_s + a.TRx - 1) / a.TRx, (a.nry_s + a.TRy - 1) / a.TRy);
     fn<<<grid, BM_THREADS, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_block_match_small(const SmallBatch& b, int items, size_t smem, cudaStream_t s) {
+    if (smem > BM_SMEM_MAX) return cudaErrorInvalidValue;
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(block_match_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    block_match_small_kernel<<<items, BM_THREADS, smem, s>>>(b);
     return cudaGetLastError();
 }
 

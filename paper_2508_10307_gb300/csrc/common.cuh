@@ -38,7 +38,7 @@ struct Geo {
     __host__ __device__ int ngroups() const { return nry * nrx; }
 };
 
-__host__ inline Geo make_geo(int H, int W, int C, int s, int win, int K) {
+__host__ __device__ inline Geo make_geo(int H, int W, int C, int s, int win, int K) {
     Geo g;
     g.H = H; g.W = W; g.C = C; g.s = s; g.win = win; g.K = K;
     g.nry = ref_count(H, s); g.nrx = ref_count(W, s);

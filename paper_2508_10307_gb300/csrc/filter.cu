@@ -1,6 +1,7 @@
 // Dispatch of the group filter, the deterministic reduction of tile partials, and the small kernels
 // of the SURE path (perturbed image, FP64 sums).
 #include "filter_impl.cuh"
+#include "small_batch.cuh"
 
 namespace htsvd {
 
@@ -38,6 +39,53 @@ cudaError_t dispatch_k(const FilterArgs& a, cudaStream_t s) {
         case 32: return dispatch_mode<32, C>(a, s);
     }
     return cudaErrorInvalidValue;
+}
+
+// Filter arguments of a small image of a batch.
+__device__ __forceinline__ void small_filter_args(const SmallBatch& B, int i, FilterArgs& a) {
+    const SmallImage& m = B.im[i];
+    a = FilterArgs{};
+    a.img = m.in;
+    a.g = small_geo(B, m);
+    a.TR = m.TR;
+    a.ntx = (a.g.nrx + m.TR - 1) / m.TR;
+    a.nty = (a.g.nry + m.TR - 1) / m.TR;
+    a.FHmax = min(a.g.H, (m.TR - 1) * B.s + a.g.wny + PS - 1);
+    a.FWmax = min(a.g.W, (m.TR - 1) * B.s + a.g.wnx + PS - 1);
+    a.idx = m.idx;
+    a.basis64 = B.b64 + (size_t)i * 4 * B.C * PS2;
+    a.basis32 = B.b32 + (size_t)i * 512;
+    a.tau64 = m.tau;
+    a.tau32 = (float)m.tau;
+    a.band_rel = kBandRel;
+    a.band_abs = (float)(m.tau * kBandTau) + 1e-6f;
+    a.agg_mode = B.agg_mode;
+    a.partials = B.part + m.part;
+    a.mode = FM_FORWARD;
+}
+
+template <int K, int C>
+__global__ void __launch_bounds__(FT_THREADS, 2) filter_small_kernel(const __grid_constant__ SmallBatch B) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ FilterArgs a;
+    const int i = small_find<&SmallImage::flt0>(B, blockIdx.x);
+    if (threadIdx.x == 0) small_filter_args(B, i, a);
+    __syncthreads();
+    filter_tile<K, C, uint8_t, FM_FORWARD>(a, blockIdx.x - B.im[i].flt0, smem);
+}
+
+template <int C>
+cudaError_t launch_filter_small_k(const SmallBatch& b, int items, size_t smem, cudaStream_t s) {
+    auto fn = b.K == 2   ? filter_small_kernel<2, C>
+              : b.K == 4 ? filter_small_kernel<4, C>
+              : b.K == 8 ? filter_small_kernel<8, C>
+              : b.K == 16 ? filter_small_kernel<16, C>
+                          : filter_small_kernel<32, C>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e != cudaSuccess) return e;
+    fn<<<items, FT_THREADS, smem, s>>>(b);
+    return cudaGetLastError();
 }
 
 // First tile (along one axis) whose footprint ends after p, and last tile whose footprint starts at or before p.
@@ -107,6 +155,17 @@ __global__ void reduce_kernel(const float* __restrict__ partials, Geo g, int TR,
     const int64_t npix = (int64_t)g.H * g.W;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < npix; p += (int64_t)gridDim.x * blockDim.x)
         reduce_pixel<C>(p, partials, g, TR, ntx, nty, FHmax, FWmax, out, den_out, num_only, den_in);
+}
+
+template <int C>
+__global__ void __launch_bounds__(256) reduce_small_kernel(const __grid_constant__ SmallBatch B) {
+    __shared__ FilterArgs a;
+    const int i = small_find<&SmallImage::red0>(B, blockIdx.x);
+    if (threadIdx.x == 0) small_filter_args(B, i, a);
+    __syncthreads();
+    const int64_t p = (int64_t)(blockIdx.x - B.im[i].red0) * 256 + threadIdx.x;
+    if (p < (int64_t)a.g.H * a.g.W)
+        reduce_pixel<C>(p, a.partials, a.g, a.TR, a.ntx, a.nty, a.FHmax, a.FWmax, B.im[i].out, nullptr, 0, nullptr);
 }
 
 __global__ void div_kernel(const float* __restrict__ gout, const float* __restrict__ den, int64_t npix, int C,
@@ -277,6 +336,16 @@ size_t filter_smem_bytes(const FilterArgs& a) {
 
 cudaError_t launch_filter(const FilterArgs& a, cudaStream_t s) {
     return a.g.C == 3 ? dispatch_k<3>(a, s) : dispatch_k<1>(a, s);
+}
+
+cudaError_t launch_filter_small(const SmallBatch& b, int items, size_t smem, cudaStream_t s) {
+    return b.C == 3 ? launch_filter_small_k<3>(b, items, smem, s) : launch_filter_small_k<1>(b, items, smem, s);
+}
+
+cudaError_t launch_reduce_small(const SmallBatch& b, int items, cudaStream_t s) {
+    if (b.C == 3) reduce_small_kernel<3><<<items, 256, 0, s>>>(b);
+    else reduce_small_kernel<1><<<items, 256, 0, s>>>(b);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_reduce(const float* partials, const Geo& g, int TR, int ntx, int nty, int FHmax, int FWmax,

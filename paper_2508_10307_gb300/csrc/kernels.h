@@ -199,6 +199,35 @@ cudaError_t launch_sure_terms(const float* out, const float* x, const float* b, 
 // Adjoint helper: r = gout / den.
 cudaError_t launch_div(const float* gout, const float* den, int64_t npix, int C, float* r, cudaStream_t s);
 
+// ---- small images of a batch, one launch a phase (small_batch.cuh)
+constexpr int kSmallImages = 128;        // images a launch describes at most (its parameter: 9 KB)
+struct SmallImage {
+    const uint8_t* in;
+    float* out;
+    int32_t* idx;
+    double tau;
+    long long part;          // first float of its tile partials
+    int H, W;
+    int TR, TRy, TRx;        // filter tile edge, grouping tile
+    int mom0, bm0, flt0, red0;   // work items of the images before it, per phase
+};
+struct SmallBatch {
+    int n, C, s, win, K, mode, agg_mode;
+    int per;                 // references per chunk of the moments
+    double gamma2;
+    unsigned long long* mom; // [n][2][64][C][C], zeroed
+    double* b64;             // [n][2][C][64][2]
+    float* b32;              // [n][512]
+    float* part;
+    SmallImage im[kSmallImages];
+};
+cudaError_t launch_moments_small(const SmallBatch& b, int items, cudaStream_t s);
+// alone: each problem has an SM to itself (they take one by their shared memory).
+cudaError_t launch_basis_small(const SmallBatch& b, bool alone, cudaStream_t s);
+cudaError_t launch_block_match_small(const SmallBatch& b, int items, size_t smem, cudaStream_t s);
+cudaError_t launch_filter_small(const SmallBatch& b, int items, size_t smem, cudaStream_t s);
+cudaError_t launch_reduce_small(const SmallBatch& b, int items, cudaStream_t s);
+
 // ---- batched patch projection (project.cu): S = U^T * P * V per patch, 64 C coefficients in the
 // order n = (i * 8 + j) * C + c; positions are linear top-left indices y * W + x (outside: NaN).
 // Bytes of the split BF16 basis matrix (three pieces, both halves) that launch_project_split writes.

@@ -11,6 +11,7 @@
 // as A_f[a][a'] = sum_{c,c'} w^{f(c-c')} R[a][a'][c][c'] and
 //    B_f[b][b'] = sum_{c,c'} w^{f(c'-c)} Q[b][b'][c][c'],   w = exp(-2 pi i / C).
 #include "kernels.h"
+#include "small_batch.cuh"
 
 namespace htsvd {
 
@@ -132,6 +133,13 @@ template <int C>
 __global__ void __launch_bounds__(256) moments_kernel(const uint8_t* __restrict__ img, Geo g, int per,
                                                       unsigned long long* __restrict__ out) {
     moments_chunk<C>(img, g, blockIdx.x, per, out);
+}
+
+template <int C>
+__global__ void __launch_bounds__(256) moments_small_kernel(const __grid_constant__ SmallBatch B) {
+    const int i = small_find<&SmallImage::mom0>(B, blockIdx.x);
+    const SmallImage& m = B.im[i];
+    moments_chunk<C>(m.in, small_geo(B, m), blockIdx.x - m.mom0, B.per, B.mom + (size_t)i * 2 * PS2 * C * C);
 }
 
 // Row and column moments of the reference patches of a cube with any number of bands C, in the
@@ -836,6 +844,13 @@ __global__ void basis_kernel(const unsigned long long* __restrict__ mom, int C, 
     basis_problem(mom, C, blockIdx.x, b64, b32, gap);
 }
 
+// Block b: problem b % (2 (C / 2 + 1)) of image b / (2 (C / 2 + 1)).
+__global__ void basis_small_kernel(const __grid_constant__ SmallBatch B) {
+    const int np = 2 * (B.C / 2 + 1), i = blockIdx.x / np;
+    basis_problem(B.mom + (size_t)i * 2 * PS2 * B.C * B.C, B.C, blockIdx.x % np, B.b64 + (size_t)i * 4 * B.C * PS2,
+                  B.b32 + (size_t)i * 512, nullptr);
+}
+
 __global__ void quantize_kernel(const float* __restrict__ x, int64_t n, uint8_t* __restrict__ q) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         float v = rintf(x[i]);
@@ -975,6 +990,24 @@ extern "C" int htsvd_internal_moments(const uint8_t* d_img, int H, int W, int C,
 extern "C" int htsvd_internal_basis(const unsigned long long* d_mom, int C, double* d_b64, float* d_b32) {
     if (launch_basis(d_mom, C, d_b64, d_b32, 0) != cudaSuccess) return 1;
     return cudaDeviceSynchronize() == cudaSuccess ? 0 : 1;
+}
+
+cudaError_t launch_moments_small(const SmallBatch& b, int items, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(b.mom, 0, sizeof(unsigned long long) * 2 * PS2 * b.C * b.C * b.n, s);
+    if (e != cudaSuccess) return e;
+    if (b.C == 3) moments_small_kernel<3><<<items, 256, 0, s>>>(b);
+    else moments_small_kernel<1><<<items, 256, 0, s>>>(b);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_basis_small(const SmallBatch& b, bool alone, cudaStream_t s) {
+    const int smem = alone ? 200 * 1024 : 0;
+    if (alone) {
+        cudaError_t e = cudaFuncSetAttribute(basis_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    basis_small_kernel<<<b.n * basis_problems(b.C), 32, smem, s>>>(b);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_moments(const uint8_t* img, const Geo& g, unsigned long long* d_mom, cudaStream_t s) {

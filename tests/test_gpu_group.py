@@ -111,3 +111,36 @@ def test_gradients_by_size_and_rows_kept(shape, K, mult):
     gx, gw = H.denoise_vjp(xt, 20.0, info["idx"], wt, out, torch.from_numpy(gout.astype(np.float32)).cuda(), prm)
     assert np.abs(gx.cpu().numpy() - gx_o).max() <= 1e-4 * np.abs(gx_o).max()
     assert np.abs(gw.cpu().numpy() - gw_o).max() <= 1e-4 * max(1.0, np.abs(gw_o).max())
+
+
+@pytest.mark.parametrize("C,K,sizes", [
+    (3, 8, [(33, 40), (125, 130), (64, 33), (20, 90), (48, 48)]),              # a larger one among them
+    (1, 32, [(40 + i % 7, 41 + i % 5) for i in range(131)]),                   # more than one launch describes
+    (3, 16, [(36, 37)] * 2),
+    (1, 2, [(8, 8), (9, 31), (8, 60)]),                                        # one reference row
+])
+def test_small_images_of_a_batch(C, K, sizes):
+    """They share their launches: groupings equal those of single calls, pixels to rounding (other filter tiles)."""
+    prm = dict(stride=3, window=9, K=K, agg_mode="sparsity" if K == 16 else "uniform")
+    sizes = [(h, w) for h, w in sizes if min(9, h - 7) * min(9, w - 7) >= K]
+    xs = [torch.from_numpy(synth.add_gaussian(synth.clean_image(h, w, C, 5 + i), 20.0, i)).cuda()
+          for i, (h, w) in enumerate(sizes)]
+    sig = [10.0 + i % 9 for i in range(len(xs))]
+    idx = [torch.empty((H.num_groups(h, w, prm), K), dtype=torch.int32, device="cuda") for h, w in sizes]
+    outs = H.denoise_batch(xs, sig, prm, idx_outs=idx)
+    again = H.denoise_batch(xs, sig, prm)
+    for x, s, o, o2, ix in zip(xs, sig, outs, again, idx):
+        want, info = H.denoise(x, s, prm, return_info=True)
+        assert torch.equal(ix, info["idx"])
+        assert torch.equal(o, o2) and max_abs(o.cpu().numpy(), want.cpu().numpy()) <= PIX_TOL
+
+
+def test_images_of_a_batch_are_grouped_as_single_ones():
+    """Side by side, images take the tensor-core grouping at sizes where one alone does not."""
+    prm = dict(stride=3, window=18, K=32)
+    xs = [torch.from_numpy(synth.add_gaussian(synth.clean_image(150 + 9 * i, 170, 3, i), 20.0, i)).cuda() for i in range(8)]
+    idx = [torch.empty((H.num_groups(*x.shape[:2], prm), 32), dtype=torch.int32, device="cuda") for x in xs]
+    outs = H.denoise_batch(xs, [20.0] * 8, prm, idx_outs=idx)
+    for x, o, ix in zip(xs, outs, idx):
+        want, info = H.denoise(x, 20.0, prm, return_info=True)
+        assert torch.equal(ix, info["idx"]) and max_abs(o.cpu().numpy(), want.cpu().numpy()) <= PIX_TOL
