@@ -751,10 +751,10 @@ struct HostEvent {
     }
 };
 
-// Alg. 1 with the arguments checked.
-htsvd_status denoise_checked(const void* d_in, int is_float, int H, int W, int C, double sigma, const htsvd_params* p,
-                             const Resolved& r, const float* d_w, float* d_out, int32_t* d_idx_out, cudaStream_t s) {
-    Workspace* w = workspace_for(s);
+// Alg. 1 with the arguments checked, in workspace w.
+htsvd_status denoise_checked(Workspace* w, const void* d_in, int is_float, int H, int W, int C, double sigma,
+                             const htsvd_params* p, const Resolved& r, const float* d_w, float* d_out,
+                             int32_t* d_idx_out, cudaStream_t s) {
     if (!w) return HTSVD_ERR_OOM;
     const Geo g = make_geo(H, W, C, r.s, r.win, r.K);
     const int64_t N = g.ngroups();
@@ -813,7 +813,7 @@ htsvd_status denoise_impl(const void* d_in, int is_float, int H, int W, int C, d
     ST(resolve(p, C, r));
     ST(check_image(H, W, C, r));
     if (std::isnan(sigma)) return HTSVD_ERR_INVALID_ARG;
-    return denoise_checked(d_in, is_float, H, W, C, sigma, p, r, d_w, d_out, d_idx_out, s);
+    return denoise_checked(workspace_for(s), d_in, is_float, H, W, C, sigma, p, r, d_w, d_out, d_idx_out, s);
 }
 
 // References below which the images of a batch share their launches: those that a filter alone takes without
@@ -1406,6 +1406,15 @@ htsvd_status htsvd_denoise_batch(const htsvd_image* imgs, int32_t n, const htsvd
     }
     // each to the lane with the least work so far (a lane's workspace then grows once)
     int64_t load[kBatchLanes] = {};
+    // one image or one set: on the caller's stream itself, in the first lane's workspace (whose other work is either
+    // joined into this stream already or waits for it)
+    if (jobs == 1) {
+        Workspace* lw = workspace_for(w->lane[0]);
+        if (!lw) return HTSVD_ERR_OOM;
+        if (large == 0) return denoise_small(lw, imgs, order.data(), n, r, s);
+        return denoise_checked(lw, imgs[0].d_in, 0, imgs[0].H, imgs[0].W, imgs[0].C, imgs[0].sigma, &q, r, nullptr,
+                               imgs[0].d_out, imgs[0].d_idx_out, s);
+    }
     CK(cudaEventRecord(w->ev_batch, s));
     for (int l = 0; l < lanes; ++l) CK(cudaStreamWaitEvent(w->lane[l], w->ev_batch, 0));
     htsvd_status st = HTSVD_OK;
@@ -1413,7 +1422,8 @@ htsvd_status htsvd_denoise_batch(const htsvd_image* imgs, int32_t n, const htsvd
         const htsvd_image& im = imgs[order[k]];
         const int l = (int)(std::min_element(load, load + lanes) - load);
         load[l] += (int64_t)im.H * im.W;
-        st = denoise_checked(im.d_in, 0, im.H, im.W, im.C, im.sigma, &q, r, nullptr, im.d_out, im.d_idx_out, w->lane[l]);
+        st = denoise_checked(workspace_for(w->lane[l]), im.d_in, 0, im.H, im.W, im.C, im.sigma, &q, r, nullptr, im.d_out,
+                             im.d_idx_out, w->lane[l]);
     }
     for (int k = large; k < n && st == HTSVD_OK; k += kSmallImages) {
         const int m = std::min(kSmallImages, n - k), l = (int)(std::min_element(load, load + lanes) - load);
