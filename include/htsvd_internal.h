@@ -47,9 +47,8 @@ double htsvd_internal_sigma_from_moments(const unsigned long long* M, const unsi
 int32_t htsvd_internal_sampled_ranks(const uint8_t* d_img, int32_t H, int32_t W, int32_t C, const htsvd_params* p,
                                      int32_t* h_ranks, int32_t max_ranks);
 
-/* Limit of a kernel's wait for the tensor cores in the later calls on stream, in nanoseconds (negative: the
- * library's own, about two seconds; 0: every wait counts as run out at once). Host only. */
-htsvd_status htsvd_internal_wait_limit(int64_t ns, cudaStream_t stream);
+/* on: in the later calls on stream, a kernel that waits for the tensor cores ends as if a wait had run out. Host only. */
+htsvd_status htsvd_internal_give_up_waits(int32_t on, cudaStream_t stream);
 
 /* Limits of the workspace of stream: plane_bytes, the most it takes for projection planes (negative: the library's
  * own), and room, the bytes that the device is taken to have free for buffers a call can do without (negative: it

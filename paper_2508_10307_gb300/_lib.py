@@ -102,7 +102,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.htsvd_internal_volume_bases.restype = ctypes.c_double
     lib.htsvd_internal_alu_probe.argtypes = [i32, i32]
     lib.htsvd_internal_alu_probe.restype = ctypes.c_double
-    lib.htsvd_internal_wait_limit.argtypes = [ctypes.c_int64, vp]
+    lib.htsvd_internal_give_up_waits.argtypes = [i32, vp]
     lib.htsvd_internal_scratch_limits.argtypes = [ctypes.c_int64, ctypes.c_int64, vp]
     lib.htsvd_internal_scratch_limits.restype = ctypes.c_int64
     lib.htsvd_internal_fail_allocations.argtypes = [i32, vp]

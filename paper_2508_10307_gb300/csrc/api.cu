@@ -154,8 +154,6 @@ constexpr size_t kPlaneBytes = (size_t)8 << 30;
 // and last tiles leave most of the chip idle); planes are limited to kPlaneBytes over all lanes.
 constexpr int kBatchLanes = 8;
 
-constexpr unsigned long long kWaitLimitNs = 2000000000ull;
-
 struct Workspace {
     int device = -1;
     cudaStream_t stream = nullptr;
@@ -167,7 +165,7 @@ struct Workspace {
                                           // block matching
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int* timeout = nullptr;               // pinned word a kernel sets when one of its waits runs out
-    unsigned long long wait_ns = kWaitLimitNs;   // limit of such a wait
+    bool give_up = false;                 // its waits count as run out (tests)
     size_t plane_cap = kPlaneBytes;       // most it may hold as projection planes
     int64_t room = -1;                    // bytes ws_try takes the device to have free (negative: it asks)
     int64_t allocations = 0;              // device allocations made so far
@@ -412,7 +410,7 @@ htsvd_status run_block_match(Workspace* w, const uint8_t* q, const Geo& g, const
             }
             ST(take_timeout(w));
             ProfScope ps_("block_match", s);
-            CK(launch_block_match_tc(a, scratch, w->timeout, w->wait_ns, s));
+            CK(launch_block_match_tc(a, scratch, w->timeout, w->give_up, s));
             return HTSVD_OK;
         }
     }
@@ -1271,10 +1269,10 @@ int32_t htsvd_internal_sampled_ranks(const uint8_t* d_img, int32_t H, int32_t W,
     return n;
 }
 
-htsvd_status htsvd_internal_wait_limit(int64_t ns, cudaStream_t s) {
+htsvd_status htsvd_internal_give_up_waits(int32_t on, cudaStream_t s) {
     Workspace* w = workspace_for(s);
     if (!w) return HTSVD_ERR_OOM;
-    w->wait_ns = ns < 0 ? kWaitLimitNs : (unsigned long long)ns;
+    w->give_up = on != 0;
     return HTSVD_OK;
 }
 
@@ -1402,7 +1400,7 @@ htsvd_status htsvd_denoise_batch(const htsvd_image* imgs, int32_t n, const htsvd
         lw->plane_cap = w->plane_cap / kBatchLanes;
         lw->room = w->room;
         lw->share = lanes;
-        lw->wait_ns = w->wait_ns;
+        lw->give_up = w->give_up;
     }
     // each to the lane with the least work so far (a lane's workspace then grows once)
     int64_t load[kBatchLanes] = {};

@@ -712,8 +712,7 @@ bool bt_plan(const BMArgs& a, BtPlan& p) {
 }
 
 template <int NPL, bool GCP>
-cudaError_t launch_bt(const BMArgs& a, const BtPlan& p, void* scratch, int* timeout, unsigned long long wait_ns,
-                      cudaStream_t s) {
+cudaError_t launch_bt(const BMArgs& a, const BtPlan& p, void* scratch, int* timeout, bool give_up, cudaStream_t s) {
     const Geo& g = a.g;
     BtArgs A{};
     A.b = a;
@@ -727,7 +726,7 @@ cudaError_t launch_bt(const BMArgs& a, const BtPlan& p, void* scratch, int* time
     A.TX = p.TX;
     A.ib = p.ib;
     A.timeout = timeout;
-    A.wait_ns = wait_ns;
+    A.give_up = give_up;
     for (int f = 0; f < p.nfr; ++f) {
         BtPrep b{};
         b.img = a.nfr > 0 ? a.vid + (a.f0 + f) * a.fstride : a.img;
@@ -772,13 +771,12 @@ size_t bm_tc_scratch(const BMArgs& a, int share) {
     return ((p.planes + 255) & ~(size_t)255) + p.svv;
 }
 
-cudaError_t launch_block_match_tc(const BMArgs& a, void* scratch, int* timeout, unsigned long long wait_ns,
-                                  cudaStream_t s) {
+cudaError_t launch_block_match_tc(const BMArgs& a, void* scratch, int* timeout, bool give_up, cudaStream_t s) {
     BtPlan p;
     if (!bt_plan(a, p)) return cudaErrorInvalidValue;
-    if (p.npl == 2) return launch_bt<2, true>(a, p, scratch, timeout, wait_ns, s);
-    return p.npl == 3 ? launch_bt<3, false>(a, p, scratch, timeout, wait_ns, s)
-                      : launch_bt<1, false>(a, p, scratch, timeout, wait_ns, s);
+    if (p.npl == 2) return launch_bt<2, true>(a, p, scratch, timeout, give_up, s);
+    return p.npl == 3 ? launch_bt<3, false>(a, p, scratch, timeout, give_up, s)
+                      : launch_bt<1, false>(a, p, scratch, timeout, give_up, s);
 }
 
 }  // namespace htsvd

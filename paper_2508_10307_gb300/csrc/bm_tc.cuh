@@ -135,7 +135,7 @@ struct BtArgs {
     int TX;                  // references per tile row (32 or 16)
     int ib;                  // index bits of a key
     int* timeout;            // set (host memory) if a wait for the tensor cores runs out
-    unsigned long long wait_ns;   // limit of such a wait
+    int give_up;             // every wait counts as run out (tests)
 };
 
 __device__ __forceinline__ void bt_tmem_ld16(uint32_t taddr, float (&v)[16]) {
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(BT_THREADS, 2) block_match_tc_kernel(const __g
             mbar_init(smem_u32(&bars[i]), 1);
             mbar_init(smem_u32(&bars[2 + i]), 4);
         }
-        *abort_word = 0;
+        *abort_word = A.give_up;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 4) {
@@ -380,8 +380,7 @@ __global__ void __launch_bounds__(BT_THREADS, 2) block_match_tc_kernel(const __g
                 if (lane == 0) {
                     for (int j = 0; j < rows; ++j) {
                         const uint32_t n = it + j, acc = n & 1;
-                        if (n >= 2 && !mbar_wait_or_abort(smem_u32(&bars[2 + acc]), ((n >> 1) & 1) ^ 1, abort_word, A.wait_ns))
-                            break;
+                        if (n >= 2 && !mbar_wait_or_abort(smem_u32(&bars[2 + acc]), ((n >> 1) & 1) ^ 1, abort_word)) break;
                         tc_fence_after();
                         uint32_t on = 0;
 #pragma unroll
@@ -401,7 +400,7 @@ __global__ void __launch_bounds__(BT_THREADS, 2) block_match_tc_kernel(const __g
                 // ---- the candidates of this warp's references
                 for (int j = 0; j < rows; ++j) {
                     const uint32_t n = it + j, acc = n & 1;
-                    const bool got = mbar_wait_or_abort(smem_u32(&bars[acc]), (n >> 1) & 1, abort_word, A.wait_ns);
+                    const bool got = mbar_wait_or_abort(smem_u32(&bars[acc]), (n >> 1) & 1, abort_word);
                     if (__any_sync(FULL, !got)) break;
                     tc_fence_after();
                     const int wy = yb + j - wy0;
@@ -445,8 +444,8 @@ __global__ void __launch_bounds__(BT_THREADS, 2) block_match_tc_kernel(const __g
     if (!ok) {
         // A wait ran out: report it, and let the MMAs in flight finish (bounded) before the tensor memory is
         // released. The last commit covers all of them, and its barrier is at most that one phase behind: row
-        // issued - 1 was issued after row issued - 3 of the same accumulator had been read. The groups below then
-        // hold what was found, and the reference itself for the rest.
+        // issued - 1 was issued after row issued - 3 of the same accumulator had been read. The groups below
+        // hold what was found, or the reference alone.
         if (tid == 0) *A.timeout = 1;
         if (warp == 4 && lane == 0 && issued > 0)
             mbar_wait_bounded(smem_u32(&bars[(issued - 1) & 1]), ((issued - 1) >> 1) & 1);
@@ -458,7 +457,6 @@ __global__ void __launch_bounds__(BT_THREADS, 2) block_match_tc_kernel(const __g
         const uint32_t imask = mul - 1u;
         const int nw = g.wny * g.wnx;
         const int fo = a.nfr > 0 ? a.f0 * g.H * g.W : 0;
-        const int home = fo + fsref * g.H * g.W + ry * g.W + rx, gi = iy * g.nrx + ix;
         bool past = false, enough = true;
         __syncwarp();
 #pragma unroll
@@ -469,14 +467,16 @@ __global__ void __launch_bounds__(BT_THREADS, 2) block_match_tc_kernel(const __g
             const int w = (int)(k & imask);
             const int fs = w / nw, wr = w - fs * nw;
             const int dy = wr / g.wnx, dx = wr - dy * g.wnx;
-            buf[i * 33 + lane] = k != ~0u ? (uint32_t)(fo + fs * g.H * g.W + (wy0 + dy) * g.W + wx0 + dx) : (uint32_t)home;
+            buf[i * 33 + lane] = (uint32_t)(fo + fs * g.H * g.W + (wy0 + dy) * g.W + wx0 + dx);
         }
         __syncwarp();
         const unsigned wide = __ballot_sync(FULL, mine && !enough), valid = __ballot_sync(FULL, mine);
+        const int home = fo + fsref * g.H * g.W + ry * g.W + rx, gi = iy * g.nrx + ix;
+        const unsigned none = ok ? 0u : wide;           // given up before the group was full: the reference alone
         for (int l = 0; l < 32; ++l) {
             if (!((valid >> l) & 1u)) continue;
             const int h = __shfl_sync(FULL, home, l), gl = __shfl_sync(FULL, gi, l);
-            if (lane < g.K) a.idx[(size_t)gl * g.K + lane] = lane == 0 ? h : (int32_t)buf[(lane - 1) * 33 + l];
+            if (lane < g.K) a.idx[(size_t)gl * g.K + lane] = lane == 0 || ((none >> l) & 1u) ? h : (int32_t)buf[(lane - 1) * 33 + l];
         }
         __syncwarp();
         for (unsigned m = ok ? wide : 0u; m; m &= m - 1) {              // warp-uniform

@@ -34,11 +34,10 @@ size_t bm_smem_bytes(const BMArgs& a);
 void bm_fit_tiles(BMArgs& a);
 cudaError_t launch_block_match(const BMArgs& a, cudaStream_t s);
 // Tensor-core form: bytes of device scratch it needs (0: not for this geometry, or not faster there), and
-// its launch. timeout: host-readable word set if a wait inside the kernel takes more than wait_ns; the groups
-// then hold positions of the search windows that may not be the nearest.
+// its launch. timeout: host-readable word set if a wait inside the kernel runs out (give_up: as if one had); the
+// groups then hold positions of the search windows that may not be the nearest.
 size_t bm_tc_scratch(const BMArgs& a, int share);
-cudaError_t launch_block_match_tc(const BMArgs& a, void* scratch, int* timeout, unsigned long long wait_ns,
-                                  cudaStream_t s);
+cudaError_t launch_block_match_tc(const BMArgs& a, void* scratch, int* timeout, bool give_up, cudaStream_t s);
 
 // ---- second moments and bases (moments.cu)
 // Row/column second moments of the reference patches, exact:

@@ -84,20 +84,15 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
     for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-constexpr uint64_t kWaitNs = 2000000000ull;          // limit of a wait for the tensor cores
-
 // Waits for the phase of `parity` of an mbarrier, giving up when the CTA's abort word is set or after
-// limit_ns (then it sets the abort word; at 0 without looking at the barrier). Returns false on giving up.
-__device__ inline bool mbar_wait_or_abort(uint32_t bar, uint32_t parity, volatile int* abort_word,
-                                          uint64_t limit_ns = kWaitNs) {
-    if (limit_ns > 0) {
+// about two seconds (then it sets the abort word). Returns false on giving up.
+__device__ inline bool mbar_wait_or_abort(uint32_t bar, uint32_t parity, volatile int* abort_word) {
+    if (mbar_try_wait(bar, parity)) return true;
+    const uint64_t t0 = global_ns();
+    for (int i = 0; i < (1 << 28); ++i) {
         if (mbar_try_wait(bar, parity)) return true;
-        const uint64_t t0 = global_ns();
-        for (int i = 0; i < (1 << 28); ++i) {
-            if (mbar_try_wait(bar, parity)) return true;
-            if (*abort_word) return false;
-            if (global_ns() - t0 > limit_ns) break;
-        }
+        if (*abort_word) return false;
+        if (global_ns() - t0 > 2000000000ull) break;
     }
     *abort_word = 1;
     return false;

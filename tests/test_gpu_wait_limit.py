@@ -1,4 +1,4 @@
-"""Waits for the tensor cores that run out (the limit set to nothing): the call's groups hold positions inside
+"""Waits for the tensor cores that run out (by a switch of the stream's workspace): the call's groups hold positions inside
 the image, the status comes once, from the next call or from the call itself where it waits for the device, and
 the call after it groups as ever. Images of at least 76 tiles of 128 references, which the tensor cores group."""
 import ctypes
@@ -16,16 +16,16 @@ pytestmark = pytest.mark.gpu
 PRM = dict(stride=3, window=18, K=32)
 
 
-def _limit(ns):
+def _give_up(on):
     s = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-    assert H.load_library().htsvd_internal_wait_limit(ns, s) == 0
+    assert H.load_library().htsvd_internal_give_up_waits(on, s) == 0
 
 
 @pytest.fixture
 def no_waiting():
-    _limit(0)
+    _give_up(1)
     yield
-    _limit(-1)
+    _give_up(0)
 
 
 def _noisy(C, seed=3):
@@ -42,7 +42,7 @@ def test_status_comes_once_and_indices_stay_inside(C, no_waiting):
     assert idx.min() >= 0 and y.max() <= 330 - 8 and xx.max() <= 331 - 8
     rows, cols = O.reference_positions(330, 8, 3), O.reference_positions(331, 8, 3)
     assert np.array_equal(idx[:, 0], (np.asarray(rows)[:, None] * 331 + np.asarray(cols)[None, :]).ravel())
-    _limit(-1)
+    _give_up(0)
     with pytest.raises(_lib.HtsvdError, match="TIMEOUT"):
         H.denoise(x, 20.0, PRM)
     ref, good = H.denoise(x, 20.0, PRM, return_info=True)
@@ -56,7 +56,7 @@ def test_a_call_that_waits_for_the_device_reports_its_own(no_waiting):
     x = _noisy(3)
     with pytest.raises(_lib.HtsvdError, match="TIMEOUT"):
         H.denoise(x, 20.0, PRM, basis_gap=True, return_info=True)
-    _limit(-1)
+    _give_up(0)
     H.denoise(x, 20.0, PRM, basis_gap=True, return_info=True)
 
 
@@ -64,7 +64,7 @@ def test_a_batch_reports_the_lanes_of_the_one_before(no_waiting):
     xs = [_noisy(3, 3 + i) for i in range(3)]
     H.denoise_batch(xs, [20.0] * 3, PRM)
     torch.cuda.synchronize()
-    _limit(-1)
+    _give_up(0)
     with pytest.raises(_lib.HtsvdError, match="TIMEOUT"):
         H.denoise_batch(xs[:1], [20.0], PRM)         # (one lane: the others' words count as well)
     for x, o in zip(xs, H.denoise_batch(xs, [20.0] * 3, PRM)):
