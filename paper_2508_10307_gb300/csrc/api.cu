@@ -140,7 +140,7 @@ enum Slot {
     S_CSCR, S_CNUM, S_CDEN,          // hyperspectral cubes: per-CTA Haar slots, numerator, denominator
     S_BMTC,                          // planes and box sums of the tensor-core grouping
     S_PROJ,                          // split BF16 basis matrix of htsvd_project_patches
-    S_VMOM, S_VB64, S_VNUM, S_VDEN,  // MRI volumes: moments, bases, numerator, denominator
+    S_VMOM, S_VB64, S_VNUM,          // MRI volumes: moments, bases, numerator and denominator
     S_NSLOT
 };
 
@@ -598,8 +598,10 @@ htsvd_status plane_bands(Workspace* w, const Geo& g, int TR, int nty, int ntiles
     }
 }
 
+// sample: also the groups sampled for P.dense, against most rows.
 htsvd_status fill_planes(const void* img, int is_float, const Geo& g, const float* b32, int y0, int y1,
-                         const VideoCtx* vc, Planes& P, cudaStream_t s) {
+                         const VideoCtx* vc, Planes& P, cudaStream_t s, const FilterArgs* sample = nullptr,
+                         int most = 0) {
     const int nfr = vc ? vc->nfr : 1;
     P.y0 = y0;
     P.y1 = y1;
@@ -619,7 +621,7 @@ htsvd_status fill_planes(const void* img, int is_float, const Geo& g, const floa
         pa.counter = P.counter;
         pa.dense = P.dense;
         ProfScope ps_("planes", s);
-        CK(launch_plane(pa, s));
+        CK(launch_plane(pa, s, sample, most, P.sample));
     }
     return HTSVD_OK;
 }
@@ -1094,23 +1096,13 @@ htsvd_status vjp_core(Workspace* w, const float* d_x, const Geo& g, const Resolv
     if (st == HTSVD_OK) st = ws_try(w, S_DOT, sizeof(float) * P.most, &dot);
     if (st != HTSVD_OK && st != HTSVD_ERR_OOM) return st;
     const bool planes = st == HTSVD_OK, ask = planes && most != kEveryRow;
-    if (ask) {                                     // the sampled groups, beside the denominators
-        ST(ws_side(w));
-        CK(cudaEventRecord(w->ev_fork, s));
-        CK(cudaStreamWaitEvent(w->side, w->ev_fork, 0));
-        ProfScope ps_("sample_rows", w->side);
-        CK(cudaMemsetAsync(P.sample, 0, 3 * sizeof(int), w->side));
-        CK(launch_sample_rows(a, most, P.sample, w->side));
-        CK(cudaEventRecord(w->ev_join, w->side));
-        P.dense = R.dense = a.dense = P.sample + 2;
-    }
+    if (ask) P.dense = R.dense = a.dense = P.sample + 2;       // (sampled beside the first planes)
     Geo g1 = g;
     g1.C = 1;
-    { ProfScope ps_("denom", s); CK(launch_denom(a, s)); }
+    { ProfScope ps_("denom", s); CK(launch_denom(a, ask ? P.sample : nullptr, s)); }
     { ProfScope ps_("reduce", s); CK(launch_reduce((float*)part, g1, t.TR, t.ntx, t.nty, t.FHmax, t.FWmax, (float*)tmp, (float*)den, 0,
                      nullptr, s)); }
     { ProfScope ps_("div", s); CK(launch_div(d_grad_out, (const float*)den, npix, C, (float*)rimg, s)); }
-    if (ask) CK(cudaStreamWaitEvent(s, w->ev_join, 0));
 
     // adjoint filter on r = gout / D with the masks of x: the planes of both images in the same bands
     if (!planes) {                                 // they do not pay, or there is no room for them: the tile kernel alone
@@ -1127,7 +1119,7 @@ htsvd_status vjp_core(Workspace* w, const float* d_x, const Geo& g, const Resolv
         R.coef = P.coef + pos * PS2 * C;
         R.pn = P.pn + pos;                                 // (not used)
         R.counter = P.counter;
-        ST(fill_planes(d_x, 1, g, b32, y0, y1, nullptr, P, s));
+        ST(fill_planes(d_x, 1, g, b32, y0, y1, nullptr, P, s, ask && t0 == 0 ? &a : nullptr, most));
         ST(fill_planes(rimg, 1, g, b32, y0, y1, nullptr, R, s));
         rc = R.coef;
         { ProfScope ps_("patch_dot", s); CK(launch_patch_dot((const float*)rimg, d_out, g.H, g.W, C, y0, y1 - y0, (float*)dot, s)); }
@@ -1751,10 +1743,11 @@ bool volume_takes_planes(const VolGeo& g) {
 
 // Filter of a volume: bands of tile planes over the projection planes that fit the workspace's share, or
 // volume_filter_kernel where they do not pay or the device has no room for them.
-htsvd_status run_volume_filter(Workspace* w, const VolFilterArgs& a, int64_t ng, cudaStream_t s) {
+// (sample: three zeroed words, device).
+htsvd_status run_volume_filter(Workspace* w, const VolFilterArgs& a, int64_t ng, int* sample, cudaStream_t s) {
     const VolGeo& g = a.g;
     const int ntz = volume_tiles_z(g);
-    void *coef, *pn, *rec, *ctr;
+    void *coef, *pn, *rec;
     bool planes = volume_takes_planes(g);
     int per = ntz;
     while (planes) {
@@ -1766,12 +1759,11 @@ htsvd_status run_volume_filter(Workspace* w, const VolFilterArgs& a, int64_t ng,
         }
         const size_t pos = (size_t)most * g.npy * g.npx;
         htsvd_status st = HTSVD_ERR_OOM;
-        if (most <= 65535 && pos * 64 * sizeof(float) <= w->plane_cap &&
+        if (most <= 65535 - 128 && pos * 64 * sizeof(float) <= w->plane_cap &&
             (int64_t)per * volume_tiles_plane(g) < ((int64_t)1 << 31)) {
             st = ws_try(w, S_PLANE, pos * 64 * sizeof(float), &coef);
             if (st == HTSVD_OK) st = ws_try(w, S_PNRM, pos * sizeof(float), &pn);
             if (st == HTSVD_OK) st = ws_try(w, S_SPILL, volume_group_rec_bytes(g, per), &rec);
-            if (st == HTSVD_OK) st = ws_try(w, S_CTR, 3 * sizeof(int), &ctr);
         }
         if (st == HTSVD_OK) break;
         if (st != HTSVD_ERR_OOM) return st;
@@ -1785,16 +1777,7 @@ htsvd_status run_volume_filter(Workspace* w, const VolFilterArgs& a, int64_t ng,
     }
     VolFilterArgs f = a;
     const int most = volume_rows_limit(g);
-    if (most != kEveryRow) {                       // the sampled groups, beside the first planes
-        ST(ws_side(w));
-        CK(cudaEventRecord(w->ev_fork, s));
-        CK(cudaStreamWaitEvent(w->side, w->ev_fork, 0));
-        ProfScope ps_("volume_sample", w->side);
-        CK(cudaMemsetAsync(ctr, 0, 3 * sizeof(int), w->side));
-        CK(launch_volume_sample(a, most, (int*)ctr, w->side));
-        CK(cudaEventRecord(w->ev_join, w->side));
-        f.dense = (const int*)ctr + 2;
-    }
+    if (most != kEveryRow) f.dense = sample + 2;
     if (a.mask_out) CK(cudaMemsetAsync(a.mask_out, 0, sizeof(uint32_t) * 2 * g.K * (size_t)ng, s));
     for (int t = 0; t < ntz; t += per) {
         const int tz = std::min(per, ntz - t);
@@ -1809,8 +1792,8 @@ htsvd_status run_volume_filter(Workspace* w, const VolFilterArgs& a, int64_t ng,
         pa.basis64 = a.basis64;
         pa.coef = (float*)coef;
         pa.pn = (float*)pn;
-        { ProfScope ps_("volume_planes", s); CK(launch_volume_plane(pa, z1 - z0, s)); }
-        if (t == 0 && f.dense) CK(cudaStreamWaitEvent(s, w->ev_join, 0));
+        pa.sample = f.dense ? sample : nullptr;
+        { ProfScope ps_("volume_planes", s); CK(launch_volume_plane(pa, z1 - z0, t == 0 && f.dense ? &a : nullptr, most, s)); }
         VolGroupArgs ga{};
         ga.f = f;
         ga.coef = (const float*)coef;
@@ -1861,11 +1844,11 @@ htsvd_status htsvd_denoise_volume(const uint8_t* d_vol, int32_t D, int32_t H, in
         ST(ws_get(w, S_IDX, sizeof(int32_t) * ng * K, &ib));
         idx = (int32_t*)ib;
     }
-    void *mom, *b64, *num, *den, *hbuf;
+    void *mom, *b64, *num, *hbuf;
     ST(ws_get(w, S_VMOM, sizeof(unsigned long long) * 512, &mom));
     ST(ws_get(w, S_VB64, sizeof(double) * 256, &b64));
-    ST(ws_get(w, S_VNUM, sizeof(float) * nvox, &num));
-    ST(ws_get(w, S_VDEN, sizeof(float) * nvox, &den));
+    const size_t acc_bytes = sizeof(float) * 2 * (size_t)nvox + 3 * sizeof(int);   // numerator, denominator, sample
+    ST(ws_get(w, S_VNUM, acc_bytes, &num));
     const bool estimate = sigma < 0;
     const size_t fm_words = estimate ? 64 * 64 + 64 : 0;
     ST(ws_host(w, sizeof(unsigned long long) * (512 + fm_words) + sizeof(double) * 256, &hbuf));
@@ -1914,13 +1897,12 @@ htsvd_status htsvd_denoise_volume(const uint8_t* d_vol, int32_t D, int32_t H, in
     a.w_in = nullptr;
     a.agg_mode = q.agg_mode;
     a.num = (float*)num;
-    a.den = (float*)den;
+    a.den = (float*)num + nvox;
     a.mask_out = p ? p->d_mask_out : nullptr;
     a.weights_out = p ? p->d_weights_out : nullptr;
-    CK(cudaMemsetAsync(num, 0, sizeof(float) * nvox, s));
-    CK(cudaMemsetAsync(den, 0, sizeof(float) * nvox, s));
-    ST(run_volume_filter(w, a, ng, s));
-    { ProfScope ps_("volume_finalize", s); CK(launch_volume_finalize((const float*)num, (const float*)den, nvox, d_out, s)); }
+    CK(cudaMemsetAsync(num, 0, acc_bytes, s));
+    ST(run_volume_filter(w, a, ng, (int*)((float*)num + 2 * nvox), s));
+    { ProfScope ps_("volume_finalize", s); CK(launch_volume_finalize(a.num, a.den, nvox, d_out, s)); }
     return HTSVD_OK;
 }
 

@@ -3,6 +3,7 @@
 #include <type_traits>
 
 #include "group_impl.cuh"
+#include "sample_rows.cuh"
 
 namespace htsvd {
 
@@ -46,121 +47,11 @@ GLayout layout_of(const GroupArgs& a, int cap) {
                         : group_layout<1>(a.f.FHmax, a.f.FWmax, cap, adj);
 }
 
-// Rows of coefficients that the groups keep, from SR_GROUPS groups spread over the image: one CTA per group
-// projects its patches, takes the Haar transform of every coefficient across them and counts the (slot, basis
-// row) pairs with a coefficient above the threshold. The last CTA compares the mean with the rows up to which
-// the group filter is the faster one (group_rows_limit). 15 us, most of it the latency of one group.
-constexpr int SR_GROUPS = 128;
-
 template <int K, int C, typename Tin, bool MF>
 __global__ void __launch_bounds__(K * PS) sample_rows_kernel(FilterArgs a, int* __restrict__ st, int most) {
-    constexpr int NC = C == 3 ? 3 : 1, NF = PS2 * NC;              // floats of a patch
-    __shared__ float sm[K * NF];                                    // [k][i][b or j][NC]
+    __shared__ float sm[K * PS2 * C];
     __shared__ unsigned mask[PS];
-    const Geo& g = a.g;
-    const int tid = threadIdx.x, ng = g.nry * g.nrx;
-    const int grp = (int)((2ll * blockIdx.x + 1) * ng / (2 * SR_GROUPS));
-    if (tid < PS) mask[tid] = 0u;
-    {
-        // column b of patch k: Y[i][b] = sum_a conj(U[a][i]) X(a, b)
-        const int k = tid >> 3, b = tid & 7;
-        int v = max(a.idx[(size_t)grp * K + k], 0);
-        const Tin* img = reinterpret_cast<const Tin*>(a.img);
-        if constexpr (MF) {
-            const int hw = g.H * g.W, f = v / hw;
-            img = reinterpret_cast<const Tin*>(a.vid) + (size_t)min(f, a.f0 + a.nfr - 1) * a.fstride;
-            v -= f * hw;
-        }
-        const int y = min(v / g.W, g.H - PS), x = min(v % g.W, g.W - PS);
-        float s0[PS] = {}, sr[PS] = {}, si[PS] = {};
-#pragma unroll 2
-        for (int r = 0; r < PS; ++r) {
-            const Tin* p = img + ((size_t)(y + r) * g.W + x + b) * C;
-            if constexpr (C == 3) {
-                const float v0 = (float)p[0], v1 = (float)p[1], v2 = (float)p[2];
-                const float X0 = v0 + v1 + v2, Xr = v0 - 0.5f * (v1 + v2), Xi = G_S3H * (v2 - v1);
-#pragma unroll
-                for (int i = 0; i < PS; ++i) {
-                    const float ur = a.basis32[64 + r * PS + i], ui = a.basis32[128 + r * PS + i];
-                    s0[i] = fmaf(a.basis32[r * PS + i], X0, s0[i]);
-                    sr[i] = fmaf(ur, Xr, fmaf(ui, Xi, sr[i]));
-                    si[i] = fmaf(ur, Xi, fmaf(-ui, Xr, si[i]));
-                }
-            } else {
-                const float X0 = (float)p[0];
-#pragma unroll
-                for (int i = 0; i < PS; ++i) s0[i] = fmaf(a.basis32[r * PS + i], X0, s0[i]);
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < PS; ++i) {
-            float* d = sm + k * NF + (i * PS + b) * NC;
-            d[0] = s0[i];
-            if constexpr (C == 3) {
-                d[1] = sr[i];
-                d[2] = si[i];
-            }
-        }
-    }
-    __syncthreads();
-    {
-        // row i of patch k: S[i][j] = sum_b Y[i][b] V[b][j] and the inverse channel DFT, over its own floats
-        float* row = sm + (tid >> 3) * NF + (tid & 7) * PS * NC;
-        float s0[PS] = {}, sr[PS] = {}, si[PS] = {};
-        const float* V = a.basis32 + (C == 3 ? 192 : 64);
-#pragma unroll 2
-        for (int b = 0; b < PS; ++b) {
-            const float y0 = row[b * NC], yr = C == 3 ? row[b * NC + (C == 3 ? 1 : 0)] : 0.f;
-            const float yi = C == 3 ? row[b * NC + (C == 3 ? 2 : 0)] : 0.f;
-#pragma unroll
-            for (int j = 0; j < PS; ++j) {
-                s0[j] = fmaf(y0, V[b * PS + j], s0[j]);
-                if constexpr (C == 3) {
-                    const float vr = V[64 + b * PS + j], vi = V[128 + b * PS + j];
-                    sr[j] = fmaf(yr, vr, fmaf(-yi, vi, sr[j]));
-                    si[j] = fmaf(yr, vi, fmaf(yi, vr, si[j]));
-                }
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < PS; ++j) {
-            if constexpr (C == 3) {
-                row[j * 3] = (s0[j] + 2.f * sr[j]) * G_THIRD;
-                row[j * 3 + 1] = (s0[j] - sr[j] - G_SQ3 * si[j]) * G_THIRD;
-                row[j * 3 + 2] = (s0[j] - sr[j] + G_SQ3 * si[j]) * G_THIRD;
-            } else {
-                row[j] = s0[j];
-            }
-        }
-    }
-    __syncthreads();
-    for (int t = tid; t < NF; t += K * PS) {
-        // coefficient t across the patches (unnormalised: the threshold grows with the support)
-        float p[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) p[k] = sm[k * NF + t];
-#pragma unroll
-        for (int d = 1; d < K; d <<= 1)
-#pragma unroll
-            for (int m = 0; m < K; m += 2 * d) {
-                const float x = p[m], y = p[m + d];
-                p[m + d] = x - y;
-                p[m] = x + y;
-            }
-        unsigned keep = 0u;
-#pragma unroll
-        for (int l = 0; l < K; ++l)
-            if (fabsf(p[l]) >= a.tau32 * g_root(l == 0 ? g_ctz(K) : g_ctz(l) + 1)) keep |= 1u << l;
-        atomicOr(&mask[t / (PS * NC)], keep);
-    }
-    __syncthreads();
-    if (tid == 0) {
-        int rows = 0;
-        for (int i = 0; i < PS; ++i) rows += __popc(mask[i]);
-        atomicAdd(st, rows);
-        __threadfence();
-        if (atomicAdd(st + 1, 1) == SR_GROUPS - 1) st[2] = atomicAdd(st, 0) > most;
-    }
+    sample_group<K, C, Tin, MF, K * PS>(a, blockIdx.x, sm, mask, st, most);
 }
 
 template <int K>
@@ -185,10 +76,12 @@ cudaError_t sample_rows(const FilterArgs& a, int most, int* st, cudaStream_t s) 
 // filter's for one channel, (0, denominator). 32 adds per group in place of 2,048 weights.
 constexpr int DN_THREADS = 128;
 
-__global__ void __launch_bounds__(DN_THREADS) denom_kernel(FilterArgs a) {
+__global__ void __launch_bounds__(DN_THREADS) denom_kernel(const __grid_constant__ FilterArgs a, int* __restrict__ st) {
     extern __shared__ float dsm[];
+    const int tile = blockIdx.x;
+    if (st && tile == 0 && threadIdx.x < 3) st[threadIdx.x] = 0;
     const Geo& g = a.g;
-    const int tid = threadIdx.x, ty = blockIdx.x / a.ntx, tx = blockIdx.x - ty * a.ntx;
+    const int tid = threadIdx.x, ty = tile / a.ntx, tx = tile - ty * a.ntx;
     int FY0, FY1, FX0, FX1;
     tile_span(ty, a.TR, g.nry, g.s, g.H, g.npy, g.wny, g.win, FY0, FY1);
     tile_span(tx, a.TR, g.nrx, g.s, g.W, g.npx, g.wnx, g.win, FX0, FX1);
@@ -221,7 +114,7 @@ __global__ void __launch_bounds__(DN_THREADS) denom_kernel(FilterArgs a) {
         row[t] = s;
     }
     __syncthreads();
-    float2* dst = reinterpret_cast<float2*>(a.partials) + (size_t)blockIdx.x * a.FHmax * a.FWmax;
+    float2* dst = reinterpret_cast<float2*>(a.partials) + (size_t)tile * a.FHmax * a.FWmax;
     for (int t = tid; t < FH * FW; t += DN_THREADS) {
         const int y = t / FW, x = t - y * FW;
         float s = 0.f;
@@ -283,23 +176,23 @@ __global__ void __launch_bounds__(256) patch_dot_kernel(const float* __restrict_
 // 455 / 530 at 17, 611 / 553 at 38 (7,056 references); two and more 1,010 / 1,117 at 59, 1,258 / 1,168 at 88. K 16: one
 // group 332 / 342 at 19, 376 / 350 at 29; more 743 / 1,105 at 44, 748 / 755 at 84. Gray, K 32: one group 238 / 287
 // at 21, 275 / 287 at 32; more 484 / 565 at 70, 687 / 606 at 158. K 16: one group 171 / 185 at 11, 203 / 189 at 23.
-// K 8, one group: RGB 240 / 278 at 7, 319 / 302 at 41, gray 117 / 145 at 2, 153 / 148 at 17
-// (K 2, 4,225 references: 83 / 74 at 1); more: the group filter
-// at any threshold. Below 3,000 references (K 32: 1,500; 961: 139 / 96 at 5, 1,681: 135 / 149 at 5, 344 / 276 at 245;
-// K 16, 1,681: 101 / 88 at 3) the tile kernel, but for images of so few
-// references that its tiles are the largest and fewer than the SMs (289: 344 / 580 at 5, 225: 1,143 / 1,085 at 173).
+// K 8, one group: RGB 240 / 278 at 7, 319 / 302 at 41, gray 117 / 145 at 2, 153 / 148 at 17 (K 2, 4,225 references:
+// 83 / 74 at 1), which a sample would not earn back; more: the group filter at any threshold. Below 3,000 references
+// (K 32: 1,500; 961: 139 / 96 at 5, 1,681: 135 / 149 at 5, 344 / 276 at 245; K 16, 1,681: 101 / 88 at 3) the tile
+// kernel, but for images of so few references that its tiles are the largest and fewer than the SMs (289: 344 / 580
+// at 5, 225: 1,143 / 1,085 at 173).
 int group_rows_limit(const FilterArgs& a) {
     if (a.mode == FM_ADJOINT) {
         const int K = a.g.K, ng = a.g.ngroups();
         if (ng < (K == 32 ? 1500 : 3000)) {
             if (a.ntx * a.nty >= device_sm_count()) return -1;
-            return K == 32 ? 60 : K >= 8 ? 40 : kEveryRow;
+            return K == 32 ? 60 : K == 16 ? 40 : kEveryRow;
         }
+        if (K <= 8) return a.g.C == 1 && ng < 5000 ? -1 : kEveryRow;
         if (K == 32 && ng < 4000) return 14;
-        if (K <= 8 && a.g.C == 1 && ng < 5000) return -1;
-        if (a.TR > 1) return K == 32 ? (a.g.C == 3 ? 80 : 110) : K == 16 ? (a.g.C == 3 ? 84 : 100) : kEveryRow;
-        if (a.g.C == 3) return K == 32 ? 20 : K == 8 ? (ng < 4000 ? 14 : 24) : ng < 4000 ? 9 : 16;
-        return ng < 4000 ? 3 : K == 32 ? 24 : K == 16 ? 10 : 8;
+        if (a.TR > 1) return a.g.C == 3 ? (K == 32 ? 80 : 84) : K == 32 ? 110 : 100;
+        if (a.g.C == 3) return K == 32 ? 20 : ng < 4000 ? 9 : 16;
+        return K == 32 ? 24 : ng < 4000 ? 3 : 10;
     }
     constexpr int rgb32[] = {15, 20, 32, 36, 42}, gray32[] = {15, 20, 24, 30, 36};
     constexpr int rgb16[] = {22, 32, 44, 48, 48}, gray16[] = {14, 24, 32, 44, 48};
@@ -310,21 +203,16 @@ int group_rows_limit(const FilterArgs& a) {
 }
 
 cudaError_t launch_sample_rows(const FilterArgs& a, int most, int* st, cudaStream_t s) {
-    switch (a.g.K) {
-        case 2: return sample_rows<2>(a, most, st, s);
-        case 4: return sample_rows<4>(a, most, st, s);
-        case 8: return sample_rows<8>(a, most, st, s);
-        case 16: return sample_rows<16>(a, most, st, s);
-        case 32: return sample_rows<32>(a, most, st, s);
-    }
-    return cudaErrorInvalidValue;
+    return a.g.K == 32   ? sample_rows<32>(a, most, st, s)
+           : a.g.K == 16 ? sample_rows<16>(a, most, st, s)
+                         : cudaErrorInvalidValue;
 }
 
-cudaError_t launch_denom(const FilterArgs& a, cudaStream_t s) {
+cudaError_t launch_denom(const FilterArgs& a, int* st, cudaStream_t s) {
     const size_t smem = 2 * sizeof(float) * a.FHmax * a.FWmax;
     cudaError_t e = cudaFuncSetAttribute(denom_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    denom_kernel<<<a.ntx * a.nty, DN_THREADS, smem, s>>>(a);
+    denom_kernel<<<a.ntx * a.nty, DN_THREADS, smem, s>>>(a, st);
     return cudaGetLastError();
 }
 

@@ -28,6 +28,7 @@
 #include <type_traits>
 
 #include "kernels.h"
+#include "sample_rows.cuh"
 
 namespace htsvd {
 
@@ -35,10 +36,6 @@ constexpr int GR_WARPS = 3;                  // warps per CTA (and tile)
 constexpr int GR_THREADS = GR_WARPS * 32;
 constexpr int GR_CTAS = 16 / GR_WARPS;       // CTAs per SM that the registers allow (16 warps of 128 registers)
 constexpr int GR_RAW = 4;                    // slots' raw coefficients that fit behind a full row list
-constexpr float G_S3H = 0.866025403784438646763723170752936183f;   // sqrt(3)/2
-constexpr float G_SQ3 = 1.73205080756887729352744634150587237f;    // sqrt(3)
-constexpr float G_THIRD = 0.333333333333333333333333333333333333f;
-
 template <int C>
 struct GCfg {
     static constexpr int ACC = (C == 3) ? 4 : 2;      // floats per footprint pixel
@@ -107,15 +104,6 @@ __device__ __forceinline__ void stage_slot(uint32_t mask, const uint32_t bit, ui
 }
 
 __host__ __device__ constexpr int g_log2(int k) { return k <= 1 ? 0 : 1 + g_log2(k / 2); }
-// Trailing zeros of 1 <= x < 32 (an expression that folds in unrolled loops; a recursion stays a call there).
-__host__ __device__ constexpr int g_ctz(int x) {
-    return (x & 1) ? 0 : (x & 2) ? 1 : (x & 4) ? 2 : (x & 8) ? 3 : 4;
-}
-// sqrt(2^e), the FP32 value (a literal: the square root of a constant is not folded in unrolled loops).
-__host__ __device__ constexpr float g_root(int e) {
-    return (e & 1) ? 1.41421356237309504880f * (float)(1 << (e >> 1)) : (float)(1 << (e >> 1));
-}
-
 // Floats of global scratch per warp.
 __host__ __device__ constexpr size_t group_spill_warp(int K, int C) {
     return (size_t)K * PS * PS * C + (size_t)2 * K * (4 + 3 * 32);

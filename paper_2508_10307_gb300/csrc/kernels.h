@@ -81,7 +81,9 @@ struct PlaneArgs {
     int* counter;            // optional: two words zeroed (the group filter's counters)
     const int* dense;        // optional: nothing else is done where it is set
 };
-cudaError_t launch_plane(const PlaneArgs& a, cudaStream_t s);
+// With f (float images, K 16 or 32), the sample of launch_sample_rows as well, into three zeroed words at st.
+struct FilterArgs;
+cudaError_t launch_plane(const PlaneArgs& a, cudaStream_t s, const FilterArgs* f = nullptr, int most = 0, int* st = nullptr);
 
 // ---- group filter and aggregation (filter.cu)
 enum FilterMode { FM_FORWARD = 0, FM_ADJOINT = 2, FM_VIDEO = 3, FM_ANALYZE = 4, FM_SYNTH = 5 };
@@ -170,8 +172,9 @@ int group_grid(GroupArgs& a);
 size_t group_spill_floats(const GroupArgs& a, int grid);
 cudaError_t launch_group(const GroupArgs& a, int grid, cudaStream_t s);
 
-// Denominator partials of a tiling (two floats per footprint pixel, (0, sum of the covering patches' weights)).
-cudaError_t launch_denom(const FilterArgs& a, cudaStream_t s);
+// Denominator partials of a tiling (two floats per footprint pixel, (0, sum of the covering patches' weights)). Zeroes
+// the three words at st, if given.
+cudaError_t launch_denom(const FilterArgs& a, int* st, cudaStream_t s);
 // dot[position] = <patch of u, patch of v> of two float images, position rows py0 .. py0 + rows - 1.
 cudaError_t launch_patch_dot(const float* u, const float* v, int H, int W, int C, int py0, int rows, float* dot,
                              cudaStream_t s);
@@ -289,8 +292,11 @@ struct VolPlaneArgs {
     const double* basis64;
     float* coef;             // [nz][H - 3][W - 3][64]
     float* pn;               // [nz][H - 3][W - 3]
+    int* sample;             // optional: three words, zeroed before the first band; nothing is done where [2] is set
 };
-cudaError_t launch_volume_plane(const VolPlaneArgs& a, int nz, cudaStream_t s);
+// With f, 128 sampled groups of it (K 16 or 32) set a.sample[2] if they keep more rows of coefficients than most in
+// the mean.
+cudaError_t launch_volume_plane(const VolPlaneArgs& a, int nz, const VolFilterArgs* f, int most, cudaStream_t s);
 struct VolGroupArgs {
     VolFilterArgs f;
     const float* coef;
@@ -300,10 +306,8 @@ struct VolGroupArgs {
     void* rec;               // volume_group_rec_bytes(g, tile planes)
 };
 bool volume_group_fits(const VolGeo& g);
-// Mean rows of coefficients a group keeps up to which planes and group filter are the faster way (kEveryRow: at any),
-// and whether the sampled groups of the volume keep more than most: st[2] of three zeroed words is set. K 16 or 32.
+// Mean rows of coefficients a group keeps up to which planes and group filter are the faster way (kEveryRow: at any).
 int volume_rows_limit(const VolGeo& g);
-cudaError_t launch_volume_sample(const VolFilterArgs& a, int most, int* st, cudaStream_t s);
 int volume_tiles_z(const VolGeo& g);
 int volume_tiles_plane(const VolGeo& g);
 // Position planes [z0, z1) that the tile planes [t0, t1) gather from.

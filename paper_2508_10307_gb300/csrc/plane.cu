@@ -17,6 +17,7 @@
 // lane l at 2 l, 2 l + 1.
 #include "f32x2.cuh"
 #include "kernels.h"
+#include "sample_rows.cuh"
 
 namespace htsvd {
 
@@ -44,10 +45,22 @@ __host__ __device__ constexpr int plane_smem() {
     return PCfg<C>::U_BYTES + PCfg<C>::Y_BYTES + PCfg<C>::Q_BYTES + (PL_NY + PS - 1) * PL_COLS * C * (int)sizeof(Tin);
 }
 
-template <int C, typename Tin>
-__global__ void __launch_bounds__(PL_THREADS, 3) plane_kernel(PlaneArgs a) {
+// SK: slots of the groups that the first zs slices of blocks sample (0: no such slices).
+template <int C, typename Tin, int SK>
+__global__ void __launch_bounds__(PL_THREADS, 3) plane_kernel(const __grid_constant__ PlaneArgs a,
+                                                              const __grid_constant__ FilterArgs f, int zs, int most,
+                                                              int* __restrict__ st) {
     using P = PCfg<C>;
     extern __shared__ __align__(16) unsigned char sm[];
+    if constexpr (SK > 0) {
+        __shared__ unsigned mask[PS];
+        if ((int)blockIdx.z < zs) {
+            const int b = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+            if (b < SR_GROUPS)
+                sample_group<SK, C, Tin, false, PL_THREADS>(f, b, reinterpret_cast<float*>(sm), mask, st, most);
+            return;
+        }
+    }
     float* ut = reinterpret_cast<float*>(sm);
     float* yb = reinterpret_cast<float*>(sm + P::U_BYTES);
     float* qs = reinterpret_cast<float*>(sm + P::U_BYTES + P::Y_BYTES);
@@ -57,8 +70,12 @@ __global__ void __launch_bounds__(PL_THREADS, 3) plane_kernel(PlaneArgs a) {
     const int x0 = blockIdx.x * PL_NX, yr0 = blockIdx.y * PL_NY;       // yr0: row within the band
     const int y0 = a.py0 + yr0;
     const Tin* img = reinterpret_cast<const Tin*>(a.img);
-    if (a.counter && blockIdx.x == 0 && blockIdx.y == 0 && tid < 2) a.counter[tid] = 0;
-    if (a.dense && *a.dense) return;
+    if (a.counter && blockIdx.x == 0 && blockIdx.y == 0 && (int)blockIdx.z == zs && tid < 2) a.counter[tid] = 0;
+    if constexpr (SK > 0) {                            // (by now known to be dense: nobody reads the planes)
+        if (__syncthreads_or(tid == 0 && *(volatile const int*)a.dense)) return;
+    } else {
+        if (a.dense && *a.dense) return;
+    }
 
     for (int t = tid; t < PS * 4; t += PL_THREADS) {
         const int r = t >> 2, i = t & 3;
@@ -232,22 +249,32 @@ __global__ void __launch_bounds__(PL_THREADS, 3) plane_kernel(PlaneArgs a) {
     }
 }
 
-template <int C, typename Tin>
-cudaError_t launch_plane_t(const PlaneArgs& a, cudaStream_t s) {
+template <int C, typename Tin, int SK = 0>
+cudaError_t launch_plane_t(const PlaneArgs& a, cudaStream_t s, const FilterArgs* f = nullptr, int most = 0,
+                           int* st = nullptr) {
     constexpr int smem = plane_smem<C, Tin>();
-    auto fn = plane_kernel<C, Tin>;
+    static_assert(smem >= SK * PS2 * C * 4, "the sample's patches");
+    auto fn = plane_kernel<C, Tin, SK>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
     }
-    const dim3 grid((a.W - PS + PL_NX) / PL_NX, (a.rows + PL_NY - 1) / PL_NY);
-    fn<<<grid, PL_THREADS, smem, s>>>(a);
+    dim3 grid((a.W - PS + PL_NX) / PL_NX, (a.rows + PL_NY - 1) / PL_NY);
+    const int per = grid.x * grid.y, zs = SK > 0 ? (SR_GROUPS + per - 1) / per : 0;
+    grid.z = zs + 1;
+    fn<<<grid, PL_THREADS, smem, s>>>(a, f ? *f : FilterArgs{}, zs, most * SR_GROUPS, st);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_plane(const PlaneArgs& a, cudaStream_t s) {
+cudaError_t launch_plane(const PlaneArgs& a, cudaStream_t s, const FilterArgs* f, int most, int* st) {
+    if (f) {
+        if (!a.is_float || !a.dense || (f->g.K != 32 && f->g.K != 16)) return cudaErrorInvalidValue;
+        if (f->g.K == 32)
+            return a.C == 3 ? launch_plane_t<3, float, 32>(a, s, f, most, st) : launch_plane_t<1, float, 32>(a, s, f, most, st);
+        return a.C == 3 ? launch_plane_t<3, float, 16>(a, s, f, most, st) : launch_plane_t<1, float, 16>(a, s, f, most, st);
+    }
     if (a.C == 3) return a.is_float ? launch_plane_t<3, float>(a, s) : launch_plane_t<3, uint8_t>(a, s);
     return a.is_float ? launch_plane_t<1, float>(a, s) : launch_plane_t<1, uint8_t>(a, s);
 }

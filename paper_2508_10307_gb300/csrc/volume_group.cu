@@ -44,17 +44,119 @@ __host__ __device__ inline int vpos(int i, int s, int n) {
 
 // ------------------------------------------------------------------------------ planes
 
+__host__ __device__ constexpr int v_log2(int k) { return k <= 1 ? 0 : 1 + v_log2(k / 2); }
+__host__ __device__ constexpr int v_ctz(int x) {
+    return (x & 1) ? 0 : (x & 2) ? 1 : (x & 4) ? 2 : (x & 8) ? 3 : 4;
+}
+__host__ __device__ constexpr float v_root(int e) {
+    return (e & 1) ? 1.41421356237309504880f * (float)(1 << (e >> 1)) : (float)(1 << (e >> 1));
+}
+
+// Rows of coefficients that VS_GROUPS groups spread over the volume keep, as sample_rows_kernel counts them for
+// images: thread (cube k, basis row i) projects its row, 64 threads take the Haar transform of a coefficient each.
+// The blocks of the first band's planes that come first do it, so that it costs no time of its own.
+constexpr int VS_GROUPS = 128;
+
+// Group b of the sample, by a block of 128 threads; sm: K * 64 floats, [k][i][j][tube].
+template <int K>
+__device__ __forceinline__ void volume_sample(const VolFilterArgs& A, int b, float* sm, unsigned* mask, int* st, int most) {
+    const VolGeo& g = A.g;
+    const int tid = threadIdx.x;
+    const long long ng = (long long)g.nrz * g.nry * g.nrx;
+    const long long grp = (2ll * b + 1) * ng / (2 * VS_GROUPS);
+    if (tid < VE) mask[tid] = 0u;
+    if (tid < K * VE) {
+        const int k = tid >> 2, i = tid & 3;
+        const uint8_t* cube = A.vol + A.idx[grp * K + k];
+        const size_t plane = (size_t)g.H * g.W;
+        const double *U = A.basis64, *V = A.basis64 + 4 * 16 * 2;      // [slice][a * 4 + i][re, im]
+        float y0[VE] = {}, y2[VE] = {}, yr[VE] = {}, yi[VE] = {};
+#pragma unroll
+        for (int a = 0; a < VE; ++a) {
+            const float u0 = (float)U[(a * 4 + i) * 2], u2 = (float)U[(32 + a * 4 + i) * 2];
+            const float ur = (float)U[(16 + a * 4 + i) * 2], ui = (float)U[(16 + a * 4 + i) * 2 + 1];
+#pragma unroll
+            for (int b = 0; b < VE; ++b) {
+                const uint8_t* p = cube + (size_t)a * g.W + b;
+                const float p0 = p[0], p1 = p[plane], p2 = p[2 * plane], p3 = p[3 * plane];
+                const float Xr = p0 - p2, Xi = p3 - p1;
+                y0[b] = fmaf(u0, (p0 + p1) + (p2 + p3), y0[b]);
+                y2[b] = fmaf(u2, (p0 - p1) + (p2 - p3), y2[b]);
+                yr[b] = fmaf(ur, Xr, fmaf(ui, Xi, yr[b]));
+                yi[b] = fmaf(ur, Xi, fmaf(-ui, Xr, yi[b]));
+            }
+        }
+        float* d = sm + tid * 16;
+#pragma unroll
+        for (int j = 0; j < VE; ++j) {
+            float z0 = 0.f, z2 = 0.f, zr = 0.f, zi = 0.f;
+#pragma unroll
+            for (int b = 0; b < VE; ++b) {
+                const float vr = (float)V[(16 + b * 4 + j) * 2], vi = (float)V[(16 + b * 4 + j) * 2 + 1];
+                z0 = fmaf(y0[b], (float)V[(b * 4 + j) * 2], z0);
+                z2 = fmaf(y2[b], (float)V[(32 + b * 4 + j) * 2], z2);
+                zr = fmaf(yr[b], vr, fmaf(-yi[b], vi, zr));
+                zi = fmaf(yr[b], vi, fmaf(yi[b], vr, zi));
+            }
+            d[j * 4] = 0.25f * fmaf(2.f, zr, z0 + z2);
+            d[j * 4 + 1] = 0.25f * fmaf(-2.f, zi, z0 - z2);
+            d[j * 4 + 2] = 0.25f * fmaf(-2.f, zr, z0 + z2);
+            d[j * 4 + 3] = 0.25f * fmaf(2.f, zi, z0 - z2);
+        }
+    }
+    __syncthreads();
+    if (tid < 64) {
+        float p[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) p[k] = sm[k * 64 + tid];
+#pragma unroll
+        for (int d = 1; d < K; d <<= 1)
+#pragma unroll
+            for (int m = 0; m < K; m += 2 * d) {
+                const float x = p[m], y = p[m + d];
+                p[m + d] = x - y;
+                p[m] = x + y;
+            }
+        unsigned keep = 0u;
+#pragma unroll
+        for (int l = 0; l < K; ++l)
+            if (fabsf(p[l]) >= A.tau32 * v_root(l == 0 ? v_log2(K) : v_ctz(l) + 1)) keep |= 1u << l;
+        atomicOr(&mask[tid >> 4], keep);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        int rows = 0;
+        for (int i = 0; i < VE; ++i) rows += __popc(mask[i]);
+        atomicAdd(st, rows);
+        __threadfence();
+        if (atomicAdd(st + 1, 1) == VS_GROUPS - 1) st[2] = atomicAdd(st, 0) > most * VS_GROUPS;
+    }
+}
+
 constexpr int VP_NX = 61;               // positions per CTA row (64 columns)
 constexpr int VP_NY = 4;
 
-__global__ void __launch_bounds__(128) volume_plane_kernel(VolPlaneArgs a) {
+// SK: slots of the groups that the first zs slices of blocks sample (0: no such slices).
+template <int SK>
+__global__ void __launch_bounds__(128, 4) volume_plane_kernel(const __grid_constant__ VolPlaneArgs a,
+                                                           const __grid_constant__ VolFilterArgs f, int zs, int most) {
     __shared__ __align__(16) float ub[3][2][16];                      // [slice][re, im][a * 4 + i]
     __shared__ __align__(16) float yb[VP_NY][64][4][4];               // [y][x][i][Y_0, Y_2, Re Y_1, Im Y_1]
     __shared__ float qs[VP_NY][64];
     __shared__ uint8_t px[VE][VP_NY + VE - 1][64];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int npx = a.W - VE + 1, npy = a.H - VE + 1;
-    const int x0 = blockIdx.x * VP_NX, y0 = blockIdx.y * VP_NY, z = a.pz0 + blockIdx.z;
+    if constexpr (SK > 0) {
+        if ((int)blockIdx.z < zs) {
+            const int b = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+            if (b < VS_GROUPS) volume_sample<SK>(f, b, &yb[0][0][0][0], reinterpret_cast<unsigned*>(qs), a.sample, most);
+            return;
+        }
+    }
+    // (by now known to be dense: nobody reads the planes)
+    if (a.sample && __syncthreads_or(threadIdx.x == 0 && *(volatile int*)(a.sample + 2))) return;
+    const int zb = blockIdx.z - zs;
+    const int x0 = blockIdx.x * VP_NX, y0 = blockIdx.y * VP_NY, z = a.pz0 + zb;
     if (tid < 96) {
         const int f = tid / 32, ri = (tid >> 4) & 1, ai = tid & 15;
         ub[f][ri][ai] = (float)a.basis64[((size_t)f * 16 + ai) * 2 + ri];
@@ -92,7 +194,7 @@ __global__ void __launch_bounds__(128) volume_plane_kernel(VolPlaneArgs a) {
     }
     __syncthreads();
     const int nx = min(VP_NX, npx - x0), ny = min(VP_NY, npy - y0);
-    const size_t row0 = ((size_t)blockIdx.z * npy + y0) * npx + x0;
+    const size_t row0 = ((size_t)zb * npy + y0) * npx + x0;
     for (int t = tid; t < ny * VP_NX; t += 128) {
         const int y = t / VP_NX, x = t - y * VP_NX;
         if (x < nx) a.pn[row0 + (size_t)y * npx + x] = (qs[y][x] + qs[y][x + 1]) + (qs[y][x + 2] + qs[y][x + 3]);
@@ -200,14 +302,6 @@ __device__ __noinline__ void vol_band(const VolFilterArgs& A, const VolSm& sm, V
         }
     }
     __syncwarp();
-}
-
-__host__ __device__ constexpr int v_log2(int k) { return k <= 1 ? 0 : 1 + v_log2(k / 2); }
-__host__ __device__ constexpr int v_ctz(int x) {
-    return (x & 1) ? 0 : (x & 2) ? 1 : (x & 4) ? 2 : (x & 8) ? 3 : 4;
-}
-__host__ __device__ constexpr float v_root(int e) {
-    return (e & 1) ? 1.41421356237309504880f * (float)(1 << (e >> 1)) : (float)(1 << (e >> 1));
 }
 
 // The inverse of one group from its row list (rows already through V^H).
@@ -571,88 +665,6 @@ __global__ void __launch_bounds__(VG_THREADS, 2) volume_group_kernel(const __gri
     }
 }
 
-// Rows of coefficients that VS_GROUPS groups spread over the volume keep, as sample_rows_kernel counts them for
-// images: thread (cube k, basis row i) projects its row, 64 threads take the Haar transform of a coefficient each.
-// It runs beside the first band's planes.
-constexpr int VS_GROUPS = 128;
-
-template <int K>
-__global__ void __launch_bounds__(K * VE) volume_sample_kernel(VolFilterArgs A, int* __restrict__ st, int most) {
-    __shared__ float sm[K * 64];                                       // [k][i][j][tube]
-    __shared__ unsigned mask[VE];
-    const VolGeo& g = A.g;
-    const int tid = threadIdx.x;
-    const long long ng = (long long)g.nrz * g.nry * g.nrx;
-    const long long grp = (2ll * blockIdx.x + 1) * ng / (2 * VS_GROUPS);
-    if (tid < VE) mask[tid] = 0u;
-    {
-        const int k = tid >> 2, i = tid & 3;
-        const uint8_t* cube = A.vol + A.idx[grp * K + k];
-        const size_t plane = (size_t)g.H * g.W;
-        const double *U = A.basis64, *V = A.basis64 + 4 * 16 * 2;      // [slice][a * 4 + i][re, im]
-        float y0[VE] = {}, y2[VE] = {}, yr[VE] = {}, yi[VE] = {};
-#pragma unroll
-        for (int a = 0; a < VE; ++a) {
-            const float u0 = (float)U[(a * 4 + i) * 2], u2 = (float)U[(32 + a * 4 + i) * 2];
-            const float ur = (float)U[(16 + a * 4 + i) * 2], ui = (float)U[(16 + a * 4 + i) * 2 + 1];
-#pragma unroll
-            for (int b = 0; b < VE; ++b) {
-                const uint8_t* p = cube + (size_t)a * g.W + b;
-                const float p0 = p[0], p1 = p[plane], p2 = p[2 * plane], p3 = p[3 * plane];
-                const float Xr = p0 - p2, Xi = p3 - p1;
-                y0[b] = fmaf(u0, (p0 + p1) + (p2 + p3), y0[b]);
-                y2[b] = fmaf(u2, (p0 - p1) + (p2 - p3), y2[b]);
-                yr[b] = fmaf(ur, Xr, fmaf(ui, Xi, yr[b]));
-                yi[b] = fmaf(ur, Xi, fmaf(-ui, Xr, yi[b]));
-            }
-        }
-        float* d = sm + tid * 16;
-#pragma unroll
-        for (int j = 0; j < VE; ++j) {
-            float z0 = 0.f, z2 = 0.f, zr = 0.f, zi = 0.f;
-#pragma unroll
-            for (int b = 0; b < VE; ++b) {
-                const float vr = (float)V[(16 + b * 4 + j) * 2], vi = (float)V[(16 + b * 4 + j) * 2 + 1];
-                z0 = fmaf(y0[b], (float)V[(b * 4 + j) * 2], z0);
-                z2 = fmaf(y2[b], (float)V[(32 + b * 4 + j) * 2], z2);
-                zr = fmaf(yr[b], vr, fmaf(-yi[b], vi, zr));
-                zi = fmaf(yr[b], vi, fmaf(yi[b], vr, zi));
-            }
-            d[j * 4] = 0.25f * fmaf(2.f, zr, z0 + z2);
-            d[j * 4 + 1] = 0.25f * fmaf(-2.f, zi, z0 - z2);
-            d[j * 4 + 2] = 0.25f * fmaf(-2.f, zr, z0 + z2);
-            d[j * 4 + 3] = 0.25f * fmaf(2.f, zi, z0 - z2);
-        }
-    }
-    __syncthreads();
-    if (tid < 64) {
-        float p[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) p[k] = sm[k * 64 + tid];
-#pragma unroll
-        for (int d = 1; d < K; d <<= 1)
-#pragma unroll
-            for (int m = 0; m < K; m += 2 * d) {
-                const float x = p[m], y = p[m + d];
-                p[m + d] = x - y;
-                p[m] = x + y;
-            }
-        unsigned keep = 0u;
-#pragma unroll
-        for (int l = 0; l < K; ++l)
-            if (fabsf(p[l]) >= A.tau32 * v_root(l == 0 ? v_log2(K) : v_ctz(l) + 1)) keep |= 1u << l;
-        atomicOr(&mask[tid >> 4], keep);
-    }
-    __syncthreads();
-    if (tid == 0) {
-        int rows = 0;
-        for (int i = 0; i < VE; ++i) rows += __popc(mask[i]);
-        atomicAdd(st, rows);
-        __threadfence();
-        if (atomicAdd(st + 1, 1) == VS_GROUPS - 1) st[2] = atomicAdd(st, 0) > most * VS_GROUPS;
-    }
-}
-
 // Voxels of a tile's footprint, at most a million (in 64 bits: strides of a few hundred pass 2^31).
 int vol_nvox(const VolGeo& g) {
     const int ext[3] = {g.wnz, g.wny, g.wnx};
@@ -691,13 +703,6 @@ int volume_rows_limit(const VolGeo& g) {
     return ng < 15000 ? 18 : ng < 60000 ? 36 : 47;
 }
 
-cudaError_t launch_volume_sample(const VolFilterArgs& a, int most, int* st, cudaStream_t s) {
-    if (a.g.K == 32) volume_sample_kernel<32><<<VS_GROUPS, 32 * VE, 0, s>>>(a, st, most);
-    else if (a.g.K == 16) volume_sample_kernel<16><<<VS_GROUPS, 16 * VE, 0, s>>>(a, st, most);
-    else return cudaErrorInvalidValue;
-    return cudaGetLastError();
-}
-
 int volume_tiles_z(const VolGeo& g) { return (g.nrz + VT - 1) / VT; }
 
 int volume_tiles_plane(const VolGeo& g) { return ((g.nry + VT - 1) / VT) * ((g.nrx + VT - 1) / VT); }
@@ -711,9 +716,14 @@ size_t volume_group_rec_bytes(const VolGeo& g, int tz) {
     return sizeof(VolRec) * 32 * VG_WARPS * (size_t)tz * volume_tiles_plane(g);
 }
 
-cudaError_t launch_volume_plane(const VolPlaneArgs& a, int nz, cudaStream_t s) {
-    const dim3 grid((a.W - VE + VP_NX) / VP_NX, (a.H - VE + VP_NY) / VP_NY, nz);
-    volume_plane_kernel<<<grid, 128, 0, s>>>(a);
+cudaError_t launch_volume_plane(const VolPlaneArgs& a, int nz, const VolFilterArgs* f, int most, cudaStream_t s) {
+    dim3 grid((a.W - VE + VP_NX) / VP_NX, (a.H - VE + VP_NY) / VP_NY, nz);
+    const int per = grid.x * grid.y, zs = f ? (VS_GROUPS + per - 1) / per : 0;
+    grid.z += zs;
+    if (!f) volume_plane_kernel<0><<<grid, 128, 0, s>>>(a, VolFilterArgs{}, zs, 0);
+    else if (f->g.K == 32) volume_plane_kernel<32><<<grid, 128, 0, s>>>(a, *f, zs, most);
+    else if (f->g.K == 16) volume_plane_kernel<16><<<grid, 128, 0, s>>>(a, *f, zs, most);
+    else return cudaErrorInvalidValue;
     return cudaGetLastError();
 }
 
