@@ -161,45 +161,46 @@ __global__ void __launch_bounds__(256) patch_dot_kernel(const float* __restrict_
 
 }  // namespace
 
-// Where planes and group filter (with the sampling) take as long as the tile kernel alone, us, both, by the mean rows.
-// The fewer groups a tile holds, the fewer warps work on it (with one, a third of them), and the earlier that is.
-// RGB, K 32: tiles of one group (256 x 264, stride 3) 283 / 305 at 13, 317 / 311 at 17, 359 / 315 at 25; 2 x 2
-// (350 x 358) 344 / 367 at 18, 391 / 376 at 26; 3 x 3 (512 x 512) 611 / 721 at 22, 763 / 750 at 34; 5 x 5 and more
-// (512 x 512, stride 2) 883 / 1,459 at 17, 1,383 / 1,567 at 41, 2,169 / 1,651 at 61. K 16: one group 249 / 270 at 19,
-// 285 / 276 at 28; 2 x 2 285 / 307 at 29, 331 / 321 at 43; 5 x 5 1,102 / 1,284 at 45, 1,582 / 1,370 at 60. Gray, K 32:
-// one group 183 / 201 at 14, 206 / 205 at 21; 2 x 2 192 / 215 at 14, 214 / 217 at 21; 3 x 3 281 / 310 at 20,
-// 383 / 319 at 30; 5 x 5 763 / 809 at 34, 859 / 818 at 40. Gray, K 16: one group 114 / 109 at 15 (4,420 references),
-// 161 / 174 at 15 (7,308). Below 4,000 references a third of that: RGB, K 32, 3,599 references 151 / 150 at 6,
-// K 16 132 / 134 at 9. With 8 slots or fewer the group filter is the faster one at any threshold.
+// Where planes and group filter take as long as the tile kernel alone. The fewer groups a tile holds, the fewer warps
+// work on it (with one, a third of them), and the earlier that is. us of both, stride 3, window 18, by the mean rows,
+// on pictures at the universal threshold (tile edge, references): RGB, K 32: 1, 4,030: 171 / 176 at 19, 196 / 180 at
+// 32; 1, 7,308: 271 / 307 at 17, 323 / 315 at 31; 2, 10,395: 267 / 292 at 30, 348 / 306 at 47; 2, 16,854: 397 / 464 at
+// 30, 488 / 484 at 46; 3, 31,265: 786 / 805 at 45, 880 / 819 at 63; 4, 52,735: 1,147 / 1,293 at 45, 1,517 / 1,316 at 63.
+// Gray, K 32: 1, 7,308: 186 / 204 at 21, 242 / 213 at 46; 2, 10,395: 151 / 168 at 20, 203 / 174 at 41; 3, 22,499: 318 /
+// 317 at 39. RGB, K 16: 1, 4,030: 137 / 155 at 24, 160 / 161 at 39; more: 221 / 250 at 39 (10,395). Gray, K 16: 1,
+// 4,030: 97 / 103 at 19, 113 / 104 at 32; 2, 10,395: 119 / 131 at 20, 140 / 133 at 31. At lower thresholds, where every
+// group keeps a few coefficients in most of its slots, the lines lie a third lower (RGB, K 32, 3 x 3: 763 / 750 at 34),
+// and the sample's 15 us count in smaller images: the limits lie between. With 8 slots or fewer the group filter is
+// the faster one at any threshold.
 //
-// The backward pass, whose tiles are smaller at a size (two images are staged), RGB: K 32, one group 346 / 495 at 6,
-// 455 / 530 at 17, 611 / 553 at 38 (7,056 references); two and more 1,010 / 1,117 at 59, 1,258 / 1,168 at 88. K 16: one
-// group 332 / 342 at 19, 376 / 350 at 29; more 743 / 1,105 at 44, 748 / 755 at 84. Gray, K 32: one group 238 / 287
-// at 21, 275 / 287 at 32; more 484 / 565 at 70, 687 / 606 at 158. K 16: one group 171 / 185 at 11, 203 / 189 at 23.
-// K 8, one group: RGB 240 / 278 at 7, 319 / 302 at 41, gray 117 / 145 at 2, 153 / 148 at 17 (K 2, 4,225 references:
-// 83 / 74 at 1), which a sample would not earn back; more: the group filter at any threshold. Below 3,000 references
-// (K 32: 1,500; 961: 139 / 96 at 5, 1,681: 135 / 149 at 5, 344 / 276 at 245; K 16, 1,681: 101 / 88 at 3) the tile
-// kernel, but for images of so few references that its tiles are the largest and fewer than the SMs (289: 344 / 580
-// at 5, 225: 1,143 / 1,085 at 173).
+// The backward pass: RGB, K 32: one group a tile, 4,030 references, ratio of the tile kernel's time 1.05 at 19, 0.99 at 32;
+// 7,308: 1.08 at 31, 0.95 at 48; more groups: 1.23 at 63, 0.95 at 77. Gray, K 32: one group, 4,030: 1.12 at 22, 0.83 at
+// 43; 7,308: 1.23 at 21, 0.98 at 46; more: 1.26 at 70, 0.84 at 158. RGB, K 16: one group, 4,030: 1.06 at 15, 1.00 at 24;
+// 7,308: 1.06 at 30, 1.00 at 38; more: 1.01 at 84. Gray, K 16: one group, 4,030: 0.98 at 8; 7,308: 1.11 at 9, 1.00 at 18;
+// more: 1.04 at 77. K 8: at any, but for small gray images (K 2, 4,225 references: 0.89). Below 3,000 references (K 32:
+// 1,500; us: 961 139 / 96 at 5, 1,681 135 / 149 at 5, 344 / 276 at 245; K 16, 1,681 101 / 88 at 3) the tile kernel, but
+// for images of so few references that its tiles are the largest and fewer than the SMs (289: 344 / 580 at 5, 225:
+// 1,143 / 1,085 at 173).
 int group_rows_limit(const FilterArgs& a) {
+    const int K = a.g.K, ng = a.g.ngroups();
+    const bool rgb = a.g.C == 3;
     if (a.mode == FM_ADJOINT) {
-        const int K = a.g.K, ng = a.g.ngroups();
         if (ng < (K == 32 ? 1500 : 3000)) {
             if (a.ntx * a.nty >= device_sm_count()) return -1;
             return K == 32 ? 60 : K == 16 ? 40 : kEveryRow;
         }
-        if (K <= 8) return a.g.C == 1 && ng < 5000 ? -1 : kEveryRow;
+        if (K <= 8) return !rgb && ng < 5000 ? -1 : kEveryRow;
         if (K == 32 && ng < 4000) return 14;
-        if (a.TR > 1) return a.g.C == 3 ? (K == 32 ? 80 : 84) : K == 32 ? 110 : 100;
-        if (a.g.C == 3) return K == 32 ? 20 : ng < 4000 ? 9 : 16;
-        return K == 32 ? 24 : ng < 4000 ? 3 : 10;
+        if (a.TR > 1) return rgb ? (K == 32 ? 72 : 84) : K == 32 ? 110 : 100;
+        if (K == 32) return ng < 5000 ? 24 : rgb ? 32 : 36;
+        return rgb ? (ng < 4000 ? 9 : ng < 5000 ? 17 : 28) : ng < 4000 ? 3 : ng < 5000 ? 7 : 16;
     }
-    constexpr int rgb32[] = {15, 20, 32, 36, 42}, gray32[] = {15, 20, 24, 30, 36};
-    constexpr int rgb16[] = {22, 32, 44, 48, 48}, gray16[] = {14, 24, 32, 44, 48};
-    const int K = a.g.K, t = std::min(a.TR, 5) - 1;
     if (K <= 8) return kEveryRow;
-    if (a.g.ngroups() < 4000) return K == 32 ? 6 : 8;
-    return K == 32 ? (a.g.C == 3 ? rgb32 : gray32)[t] : (a.g.C == 3 ? rgb16 : gray16)[t];
+    if (ng < 5000) return (rgb ? (K == 32 ? 20 : 30) : 18) * (ng < 4000 ? 2 : 3) / 3;
+    constexpr int rgb32[] = {26, 32, 38, 40, 42}, gray32[] = {24, 28, 32, 34, 36};
+    constexpr int rgb16[] = {36, 40, 48, 48, 48}, gray16[] = {26, 28, 36, 40, 48};
+    const int t = std::min(a.TR, 5) - 1;
+    return K == 32 ? (rgb ? rgb32 : gray32)[t] : (rgb ? rgb16 : gray16)[t];
 }
 
 cudaError_t launch_sample_rows(const FilterArgs& a, int most, int* st, cudaStream_t s) {
