@@ -77,6 +77,19 @@ def filter_flops_per_group(C: int, K: int) -> int:
     return K * 2 * (proj + dft) + 2 * 4 * (K - 1) * fibres + K * fibres
 
 
+def plane_flops_per_position(C: int) -> int:
+    """Flops of the projection planes at one position: a column of the row transform, which the patches along x
+    share (64 FMA per real product), and the column transform (512 FMA); C=3: one real and one complex slice, five
+    real products."""
+    return 2 * (64 + 512) * (5 if C == 3 else 1)
+
+
+def group_flops_every(C: int, K: int) -> int:
+    """Flops the group filter on planes spends on every group whatever it keeps: Haar analysis and synthesis
+    (2 (K-1) adds per fibre each), a compare per coefficient, and the weighted sum of K estimated patches."""
+    return 64 * C * (4 * (K - 1) + K + 2 * K)
+
+
 # ------------------------------------------------------------------------------------------- clocks
 
 class ClockSampler:
@@ -699,7 +712,7 @@ def run_gpu(args):
     flush = torch.empty(FLUSH_BYTES, dtype=torch.uint8, device="cuda")
     stream = torch.cuda.current_stream()
 
-    # warm-up (also grows the workspace, tunes and captures the batch graph)
+    # warm-up (also grows the workspace)
     for _ in range(args.warmup):
         res = wl.step(d_in)
     torch.cuda.synchronize()
@@ -814,9 +827,33 @@ def run_gpu(args):
     nsm = torch.cuda.get_device_properties(local).multi_processor_count
     probe = {name: float(_lib.load().htsvd_internal_alu_probe(op, 2048)) for op, name in
              ((0, "ffma"), (1, "imad"), (2, "dp4a"))}
-    if dom == "filter":
-        # (the projections are formed by the planes kernel, where the filter takes planes)
+    if dom is not None and args.workload in ("batch64", "adaptive512"):
+        # kernels of several images run at once: the sum of their times is no time of the device
+        roof = {"bound": "alu", "achieved": None, "peak": None, "unit": "TFLOP/s", "frac": None, "traffic": None,
+                "kernel": dom, "peak_basis": "not given: the images' kernels overlap on several streams"}
+    elif dom == "filter" and "planes" in prof:
+        # Projection planes and group filter: the operations every launch executes. The inverse on the rows that kept
+        # a coefficient, the FP64 decisions, and what the tile kernel spends on images with many such rows depend
+        # on the data and are not counted, so the rate is a lower bound.
+        hw = wl.host_inputs[0].shape[-3:-1]
+        positions = prof["planes"][0] * (hw[0] - 7) * (hw[1] - 7)
         n_launch, ms = prof["filter"][0], sum(prof[k][1] for k in ("filter", "planes", "sample_rows") if k in prof)
+        flops = positions * plane_flops_per_position(wl.C) + \
+            wl.groups_per_step * args.steps * group_flops_every(wl.C, wl.K)
+        achieved = flops / (ms / 1000.0) / 1e12
+        peak = nsm * FP32_LANES_PER_SM * 2 * MAX_SM_MHZ * 1e6 / 1e12
+        plane_bytes = positions * (64 * wl.C + 1) * 4 / n_launch
+        roof = {"bound": "issue", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+                "traffic": 2 * plane_bytes, "kernel": "planes + group_filter",
+                "traffic_basis": "bytes per filter launch: the planes written once and read once (the other gathers "
+                                 "hit L2: DRAM read 1.1 x the planes in profiles/group_filter_rgb512.md)",
+                "peak_basis": f"FP32 FMA: {nsm} SMs (device query) x {FP32_LANES_PER_SM} lanes x 2 flop x "
+                              f"{MAX_SM_MHZ:.0f} MHz; achieved counts one projection per position and what every "
+                              "group costs whatever it keeps, a lower bound (the group filter is bound by issue and "
+                              "latency: its FMA pipe is 15 % busy); issue-rate probe in this run: "
+                              f"{probe['ffma']:.1f} FFMA, {probe['imad']:.1f} IMAD, {probe['dp4a']:.1f} DP4A per SM clock"}
+    elif dom == "filter":
+        n_launch, ms = prof["filter"]
         flops = wl.groups_per_step * filter_flops_per_group(wl.C, wl.K) * args.steps / n_launch
         achieved = flops / (ms / n_launch / 1000.0) / 1e12
         peak = nsm * FP32_LANES_PER_SM * 2 * MAX_SM_MHZ * 1e6 / 1e12
@@ -838,6 +875,20 @@ def run_gpu(args):
                 "traffic": None, "kernel": "cube_filter",
                 "peak_basis": f"FP32 FMA: {nsm} SMs x {FP32_LANES_PER_SM} lanes x 2 flop x {MAX_SM_MHZ:.0f} MHz; "
                               "achieved counts the forward transforms only"}
+    elif dom == "volume_filter" and "volume_planes" in prof:
+        # as for images: one projection per position (two real slices and one complex, six real
+        # products: 16 FMA of the row transform, which the cubes along x share, and 64 of the column transform) and the Haar passes, compares and sums of every group
+        dims = wl.host_inputs[0].shape[-3:]
+        positions = len(wl.host_inputs) * args.steps * (dims[0] - 3) * (dims[1] - 3) * (dims[2] - 3)
+        n_launch, ms = prof["volume_filter"][0], prof["volume_filter"][1] + prof["volume_planes"][1]
+        flops = positions * 2 * 6 * (16 + 64) + wl.groups_per_step * args.steps * 64 * (4 * (wl.K - 1) + 3 * wl.K)
+        achieved = flops / (ms / 1000.0) / 1e12
+        peak = nsm * FP32_LANES_PER_SM * 2 * MAX_SM_MHZ * 1e6 / 1e12
+        roof = {"bound": "issue", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+                "traffic": 2 * positions * 65 * 4 / args.steps, "kernel": "volume_planes + volume_filter",
+                "traffic_basis": "bytes per step: the planes written once and read once",
+                "peak_basis": f"FP32 FMA: {nsm} SMs x {FP32_LANES_PER_SM} lanes x 2 flop x {MAX_SM_MHZ:.0f} MHz; "
+                              "achieved counts what every position and group costs whatever is kept, a lower bound"}
     elif dom == "volume_filter":
         n_launch, ms = prof["volume_filter"]
         flops = wl.groups_per_step * volume_flops_per_group(wl.K) * args.steps / n_launch
