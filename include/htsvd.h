@@ -237,7 +237,10 @@ htsvd_status htsvd_denoise_adaptive(const uint8_t* d_noisy, int32_t H, int32_t W
 /* Alg. 1 on n uint8 images of any sizes (one C for the whole batch) with per-image sigma
  * (>= 0). The images are spread, largest first, over up to eight streams of the library, each with
  * a workspace of its own; they start after the work already in `stream` and `stream` continues
- * after the last of them. No synchronisation with the host. Optional outputs of p are ignored. */
+ * after the last of them. Images below 3,000 references share their launches, up to 128 of them.
+ * No synchronisation with the host once the workspaces have grown. Optional outputs of p are ignored,
+ * and p->tile may be any edge (below 1: automatic). Host threads may call it on one stream at once:
+ * they take turns. */
 htsvd_status htsvd_denoise_batch(const htsvd_image* h_imgs, int32_t n, const htsvd_params* p,
                                  cudaStream_t stream);
 

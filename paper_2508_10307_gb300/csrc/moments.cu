@@ -484,7 +484,8 @@ __host__ __device__ void canonicalise(double (*Ar)[PS], double (*Vr)[PS], double
     }
 }
 
-// Device form of canonicalise for one warp: lane i < 8 ranks eigenvalue i, then lane c < 8 treats output column c. The largest-modulus entry is found on squared
+// Device form of canonicalise for one warp: lane i < 8 ranks eigenvalue i, then lane c < 8 treats output column c.
+// (Equal eigenvalues, whose vectors are not unique, keep their order.) The largest-modulus entry is found on squared
 // moduli and the phase takes one reciprocal square root (FP64 square root and division are long
 // sequences on this GPU).
 __device__ void canonicalise_warp(double (*Ar)[PS], double (*Vr)[PS], double (*Vi)[PS], double (*Out)[PS][2],
@@ -566,7 +567,7 @@ __host__ __device__ void slice_basis(const unsigned long long* mom, int C, int w
 // FP64 runs at 1.7 FMA per clock and SM on this part, and a division or square root takes it thousands of
 // cycles: the solver was 150 us for four problems, almost all of it in the rotations' angles. Any angle
 // gives a similarity transform as long as the rotation itself is unitary to working precision, so the
-// angle comes from FP32 and only cos, sin and the phase are normalised in FP64 (a Newton step on an FP32
+// angle comes from FP32 and only cos, sin and the phase are normalised in FP64 (two Newton steps on an FP32
 // reciprocal square root). The first sweeps run in FP32 altogether; their eigenvectors, made orthonormal
 // in FP64, transform the FP64 matrix to a nearly diagonal one that two or three FP64 sweeps finish: 80 us (a
 // serial chain of one warp per problem).
