@@ -860,14 +860,14 @@ htsvd_status denoise_small(Workspace* w, const htsvd_image* imgs, const int* whi
         FilterArgs fa{};
         fa.g = g;
         fa.mode = FM_FORWARD;
-        for (int e = refs < 1200 ? 2 : refs < 10000 ? 3 : 4; r.tile == 0 && e > 0; --e) {
+        for (int e = refs < 1200 ? 2 : refs < 10000 ? 3 : 4; e > 0; --e) {
             t = choose_filter_tiling(g, 1, FM_FORWARD, e);
             fa.FHmax = t.FHmax;
             fa.FWmax = t.FWmax;
             if (t.TR > 0 && filter_smem_bytes(fa) <= 112 * 1024) break;
             t.TR = 0;
         }
-        if (t.TR == 0) t = choose_filter_tiling(g, 1, FM_FORWARD, r.tile);
+        if (t.TR == 0) t = choose_filter_tiling(g, 1, FM_FORWARD, 0);
         if (t.TR == 0) return HTSVD_ERR_UNSUPPORTED;
         fa.FHmax = t.FHmax;
         fa.FWmax = t.FWmax;
@@ -895,7 +895,7 @@ htsvd_status denoise_small(Workspace* w, const htsvd_image* imgs, const int* whi
         smem_bm = std::max(smem_bm, bm_smem_bytes(ba));
         smem_f = std::max(smem_f, filter_smem_bytes(fa));
     }
-    if (smem_bm > 227 * 1024 || smem_f > 227 * 1024) return HTSVD_ERR_UNSUPPORTED;
+    if (smem_bm > 226 * 1024 || smem_f > 226 * 1024) return HTSVD_ERR_UNSUPPORTED;
     void *p_mom, *p64, *p32, *p_idx, *p_part;
     ST(ws_get(w, S_MOM, sizeof(unsigned long long) * 2 * PS2 * C * C * n, &p_mom));
     ST(ws_get(w, S_B64, sizeof(double) * 4 * C * PS2 * n, &p64));
@@ -1373,7 +1373,7 @@ htsvd_status htsvd_denoise_batch(const htsvd_image* imgs, int32_t n, const htsvd
     while (large > 0 &&
            (int64_t)ref_count(imgs[order[large - 1]].H, r.s) * ref_count(imgs[order[large - 1]].W, r.s) < kSmallGroups)
         --large;
-    if (n - large < 2) large = n;
+    if (n - large < 2 || edge > 0) large = n;        // (a forced tile edge as single calls take it)
     const int jobs = large + (n - large + kSmallImages - 1) / kSmallImages;
     const int lanes = std::min(jobs, kBatchLanes);
     std::lock_guard<std::mutex> lk(w->batch_mu);

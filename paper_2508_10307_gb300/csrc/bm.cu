@@ -656,7 +656,7 @@ cudaError_t launch_block_match(const BMArgs& a, cudaStream_t s) {
               : a.nfr > 0                    ? block_match_video_kernel
                                              : block_match_kernel;
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(fn);
         if (e != cudaSuccess) return e;
     }
     dim3 grid((a.nrx_s + a.TRx - 1) / a.TRx, (a.nry_s + a.TRy - 1) / a.TRy);
@@ -667,8 +667,7 @@ cudaError_t launch_block_match(const BMArgs& a, cudaStream_t s) {
 cudaError_t launch_block_match_small(const SmallBatch& b, int items, size_t smem, cudaStream_t s) {
     if (smem > BM_SMEM_MAX) return cudaErrorInvalidValue;
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(block_match_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+        cudaError_t e = allow_smem(block_match_small_kernel, 1024);
         if (e != cudaSuccess) return e;
     }
     block_match_small_kernel<<<items, BM_THREADS, smem, s>>>(b);
@@ -744,7 +743,7 @@ cudaError_t launch_bt(const BMArgs& a, const BtPlan& p, void* scratch, int* time
     // at most two CTAs per SM: each takes half of the tensor memory
     const int smem = std::max(bt_layout(NPL, p.nsv, p.XP, p.SR).total, 77 * 1024);
     auto fn = block_match_tc_kernel<NPL, GCP>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(fn);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     const int TY = BT_REFS / p.TX;

@@ -822,7 +822,7 @@ template <int K>
 cudaError_t launch_cube_t(const CubeArgs& a, int grid, cudaStream_t s) {
     const int smem = cube_layout(a.g.C, K).total;
     auto fn = cube_filter_kernel<K>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(fn);
     if (e != cudaSuccess) return e;
     fn<<<grid, cube_threads(a.g.C), smem, s>>>(a);
     return cudaGetLastError();
@@ -834,7 +834,7 @@ int cube_per_sm(int C) {
     const int smem = cube_layout(C, K).total;
     auto fn = cube_filter_kernel<K>;
     int n = 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+    if (allow_smem(fn) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, cube_threads(C), smem) != cudaSuccess)
         n = 1;
     return n < 1 ? 1 : n;

@@ -81,7 +81,7 @@ cudaError_t launch_filter_small_k(const SmallBatch& b, int items, size_t smem, c
               : b.K == 8 ? filter_small_kernel<8, C>
               : b.K == 16 ? filter_small_kernel<16, C>
                           : filter_small_kernel<32, C>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fn, 512);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     fn<<<items, FT_THREADS, smem, s>>>(b);

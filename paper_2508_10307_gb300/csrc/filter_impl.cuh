@@ -1558,7 +1558,7 @@ cudaError_t launch_filter_t(const FilterArgs& a, cudaStream_t s) {
                       : MODE == FM_VIDEO ? f_layout_fwd<K, C>(a.FHmax, a.FWmax, (int)sizeof(Tin), a.nfr)
                                          : f_layout<K, C>(a.FHmax, a.FWmax, (int)sizeof(Tin), MODE);
     auto fn = filter_kernel<K, C, Tin, MODE>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
+    cudaError_t e = allow_smem(fn);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     fn<<<a.left ? a.left_tiles : a.ntx * a.nty, FT_THREADS, L.total, s>>>(a);

@@ -13,7 +13,7 @@ template <int K, int C, typename Tin, bool MF, bool ADJ = false>
 cudaError_t launch_group_t(const GroupArgs& a, int grid, cudaStream_t s) {
     const int smem = group_layout<C>(a.f.FHmax, a.f.FWmax, a.cap, ADJ).total;
     auto fn = group_kernel<K, C, Tin, MF, ADJ>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(fn, 64);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     fn<<<grid, GR_THREADS, smem, s>>>(a);
@@ -211,7 +211,7 @@ cudaError_t launch_sample_rows(const FilterArgs& a, int most, int* st, cudaStrea
 
 cudaError_t launch_denom(const FilterArgs& a, int* st, cudaStream_t s) {
     const size_t smem = 2 * sizeof(float) * a.FHmax * a.FWmax;
-    cudaError_t e = cudaFuncSetAttribute(denom_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(denom_kernel);
     if (e != cudaSuccess) return e;
     denom_kernel<<<a.ntx * a.nty, DN_THREADS, smem, s>>>(a, st);
     return cudaGetLastError();

@@ -12,6 +12,15 @@ enum MatchMode { MM_GRAY = 0, MM_GCP = 1, MM_FULL = 2, MM_GREEN = 3 };
 // looked up once per device); grids and wave counts are sized from it.
 int device_sm_count();
 
+// Lets launches of fn take dynamic shared memory up to what a CTA can have beside `fixed` bytes of static. The same
+// limit whatever a launch needs: a smaller one set by another host thread, between this request and the launch
+// that needs more, would make that launch fail.
+constexpr int kSmemOptIn = 227 * 1024;
+template <typename F>
+cudaError_t allow_smem(F* fn, int fixed = 0) {
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemOptIn - fixed);
+}
+
 // ---- block matching (bm.cu)
 struct BMArgs {
     const uint8_t* img;

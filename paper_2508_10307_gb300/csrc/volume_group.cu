@@ -677,7 +677,7 @@ template <int K>
 cudaError_t launch_vg(const VolGroupArgs& a, int tiles, cudaStream_t s) {
     const int smem = vol_layout(vol_nvox(a.f.g), K * 4).total;
     auto fn = volume_group_kernel<K>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(fn, 3072);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     fn<<<tiles, VG_THREADS, smem, s>>>(a);
